@@ -139,7 +139,7 @@ typedef struct {
 /* Tuning and run options.  Zero-initialised = defaults.  No tuning field changes any
  * result bit; fsgp_autotune() picks the tuning fields. */
 typedef struct {
-    int32_t vector_words;   /* 32-bit state words per thread: 1, 2 or 4 (0 = auto: 2) */
+    int32_t vector_words;   /* 32-bit state words per thread: 1, 2 or 4 (0 = auto) */
     int32_t small_max_deg;  /* rows with in-degree <= this: one thread team per row;
                                rounded down to 2^k - 1 (0 = auto) */
     int32_t hub_min_deg;    /* rows with in-degree >= this: split over CTAs; rounded down
@@ -157,13 +157,14 @@ typedef struct {
                                graph and launch it at once (ignored when profiling) */
     int32_t lane_words;     /* words per thread of the one-thread-per-row kernel (rows with
                                1..3 in-arcs): 1, 2, 4 or 8 (0 = auto) */
-    int32_t fuse_rows;      /* 1: every row in one kernel per step (team per row when every
-                               in-degree is <= 255, else warp per row), dense steps only,
-                               for small graphs whose steps are bound by launch latency;
-                               needs in-degree < 65536; -1: never; 0: auto (graphs of at
-                               most 2^20 state words per plane, when no degree-class or
-                               frontier field is set) */
-    int32_t persistent;     /* fused team-per-row mode: 0 (auto) or 1 runs all T steps in one
+    int32_t fuse_rows;      /* 1: every row in one kernel per step (a warp each for the longest
+                               rows, a team each for the others), dense steps only, for
+                               small graphs whose steps are bound by launch latency; needs
+                               in-degree < 65536; -1: never; 0: auto (graphs of at most 2^20
+                               state words per plane, or 2^22 for epidemic models other than
+                               SWIR when every in-degree is below 8192, when no degree-class
+                               or frontier field is set) */
+    int32_t persistent;     /* fused mode: 0 (auto, up to 2^20 words) or 1 runs all T steps in one
                                cooperative launch, steps separated by grid barriers, when
                                per-realization counts and profiling are off and each thread
                                takes one word; every barrier wait is bounded (about a second)

@@ -300,7 +300,7 @@ static void release(fsgp_graph *g) {
     cudaFree(g->arc0);
     cudaFree(g->lane_tab);
     cudaFree(g->arc_w);
-    cudaFree(g->hub.d_chunk_base);
+    for (HubTable &T : g->hubs) cudaFree(T.d_chunk_base);
     cudaFree(g->ws.ptr);
     cudaFree(g->sgc.inv_din);
     cudaFree(g->sgc.in_items);

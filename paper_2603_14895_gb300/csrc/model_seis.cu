@@ -6,5 +6,5 @@ namespace fsgp {
 template int launch_rows<FSGP_SEIS>(const StepArgs &, const StepLaunch &, cudaStream_t);
 template int occupancy_rows<FSGP_SEIS>(int, int, size_t, RowOccupancy *);
 template int launch_split_rows<FSGP_SEIS>(const StepArgs &, int, int, int, int, cudaStream_t);
-template int launch_persist<FSGP_SEIS>(const StepArgs &, const PersistArgs &, int, int, size_t, int, cudaStream_t, int *);
+template int launch_persist<FSGP_SEIS>(const StepArgs &, const PersistArgs &, int, int, int, size_t, int, cudaStream_t, int *);
 }  // namespace fsgp

@@ -4,8 +4,10 @@
 #pragma once
 
 #include <algorithm>
+#include <atomic>
 
 #include "step.cuh"
+#include "tile.cuh"
 
 namespace fsgp {
 
@@ -84,6 +86,11 @@ struct ModelTraits {
     // hub rows may stop reading once every susceptible lane reaches K_sat
     static constexpr bool saturates = MODEL == FSGP_SIR || MODEL == FSGP_SIS || MODEL == FSGP_SEIR ||
                                       MODEL == FSGP_SEIS;
+    // words decided through the warp tile (SWIR's second draw depends on its first one and
+    // stays on the per-thread update)
+    static constexpr bool tiled = MODEL != FSGP_SWIR;
+    // fixed-threshold draws per word: recovery, and the latent exit of SEIR / SEIS
+    static constexpr int fixed_draws = (MODEL == FSGP_SEIR || MODEL == FSGP_SEIS) ? 2 : (cascade ? 0 : 1);
 };
 
 // Lanes that can change through their in-arcs: susceptible (SWIR: also weakened) or
@@ -148,17 +155,96 @@ __device__ __forceinline__ uint64_t ic_threshold(const StepArgs &A, int s, int32
     return __ldg(&A.sp[s].p_const);
 }
 
+// Gather the `rem` in-arcs at col[first ..] of a row into bit-sliced counters (count
+// models; rem <= 0: none).  PARTS teams of the warp share the row and take 8 arcs each per
+// round, the rounds `step` arcs apart (8 * PARTS when nobody else works on the row).  The
+// next round's column indices are loaded while the state words of this one are in flight.
+//   One team per row: its lanes load the round's indices side by side and hand them out by
+//   shuffles (a load per arc and thread would touch one cache line per row of the warp for
+//   every arc); every lane of the warp takes part until no row has arcs left.
+//   Several teams per row: the indices the warp needs lie in two or three lines anyway, and
+//   the plain loads are cheaper than the shuffles (rows of 256 to 8191 arcs, R-MAT, SIS,
+//   R = 256: 0.36 against 0.46 ms per step at n = 8M).
+template <int MODEL, int V, int B, int TEAM, int PARTS, bool CG = false>
+__device__ __forceinline__ void gather_counts(const StepArgs &A, int64_t first, int32_t rem, int32_t step, int w0,
+                                              int lane, uint32_t (&c)[V][B]) {
+    const uint32_t *src = A.cur + (size_t)ModelTraits<MODEL>::src_plane * A.plane_words + w0;
+    const uint32_t Wn = (uint32_t)A.Wn;
+    if constexpr (PARTS == 1 && TEAM > 1) {
+        constexpr int NQ = TEAM >= 8 ? 1 : 8 / TEAM;  // indices each lane of the team loads
+        const int tl = lane % TEAM, g0 = lane - tl;
+        const int32_t *cp = A.col + first + tl;
+        const bool loads = TEAM <= 8 || tl < 8;
+        int32_t mine[NQ];
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) mine[q] = loads && q * TEAM + tl < rem ? __ldg(cp + q * TEAM) : -1;
+        while (__any_sync(0xffffffffu, rem > 0)) {
+            Vec<V> xs[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int32_t u = __shfl_sync(0xffffffffu, mine[TEAM >= 8 ? 0 : j / TEAM], g0 + (TEAM >= 8 ? j : j % TEAM));
+                xs[j] = Vec<V>{};
+                if (u >= 0) xs[j] = ld_vec<V, CG>(src + (uint64_t)(uint32_t)u * Wn);
+            }
+            cp += step;
+            rem -= step;
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) mine[q] = loads && q * TEAM + tl < rem ? __ldg(cp + q * TEAM) : -1;
+#pragma unroll
+            for (int i = 0; i < V; ++i)
+                add8<B>(c[i], xs[0].w[i], xs[1].w[i], xs[2].w[i], xs[3].w[i], xs[4].w[i], xs[5].w[i], xs[6].w[i],
+                        xs[7].w[i]);
+        }
+    } else {
+        const int part = lane / TEAM % PARTS;
+        const int32_t *cp = A.col + first + 8 * part;
+        rem -= 8 * part;
+        int32_t u[8];
+        if (rem >= 8) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) u[j] = __ldg(cp + j);
+        }
+        while (rem >= 8) {
+            Vec<V> xs[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) xs[j] = ld_vec<V, CG>(src + (uint64_t)(uint32_t)u[j] * Wn);
+            cp += step;
+            rem -= step;
+            if (rem >= 8) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) u[j] = __ldg(cp + j);
+            }
+#pragma unroll
+            for (int i = 0; i < V; ++i)
+                add8<B>(c[i], xs[0].w[i], xs[1].w[i], xs[2].w[i], xs[3].w[i], xs[4].w[i], xs[5].w[i], xs[6].w[i],
+                        xs[7].w[i]);
+        }
+        // the row's last, partial group
+#pragma unroll 1
+        for (; rem > 0; rem -= 4, cp += 4) {
+            Vec<V> xs[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                xs[j] = Vec<V>{};
+                if (j < rem) xs[j] = ld_vec<V, CG>(src + (uint64_t)(uint32_t)__ldg(cp + j) * Wn);
+            }
+#pragma unroll
+            for (int i = 0; i < V; ++i) add4<B>(c[i], xs[0].w[i], xs[1].w[i], xs[2].w[i], xs[3].w[i]);
+        }
+        __syncwarp();
+    }
+}
+
 // Gather the in-arcs [e_begin, e_end) with stride `step` (groups of 4 consecutive arcs)
-// into bit-sliced counters (SIR/SIS/LT) or live-lane masks (IC).  Software pipelined:
-// the column indices of the next group are loaded while the state words of the current
-// group are in flight, so each group costs one memory latency instead of two.
-// IC draws are keyed by the arc's position in the caller's column array: arc e of the
+// into live-lane masks (IC, weighted graphs).  Software pipelined like
+// gather_counts.
+// Draws are keyed by the arc's position in the caller's column array: arc e of the
 // relabelled array is caller arc e + arcb.
-template <int MODEL, int V, int B, bool CG = false>
+template <int MODEL, int V, bool CG = false>
 __device__ __forceinline__ void gather_arcs(const StepArgs &A, int64_t e_begin, int64_t e_end,
                                             int64_t step, int64_t arcb, int w0, const uint32_t (&need)[V],
                                             const uint64_t (&ic_thr)[V], const WordCtx (&x)[V],
-                                            uint32_t (&c)[V][B], uint32_t (&newly)[V]) {
+                                            uint32_t (&newly)[V]) {
     const uint32_t *src = A.cur + (size_t)ModelTraits<MODEL>::src_plane * A.plane_words + w0;
     const size_t Wn = (size_t)A.Wn;
     int32_t u[4];
@@ -168,35 +254,23 @@ __device__ __forceinline__ void gather_arcs(const StepArgs &A, int64_t e_begin, 
         Vec<V> xs[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            if (u[j] >= 0) {
-                xs[j] = ld_vec<V, CG>(src + (size_t)u[j] * Wn);
-            } else {
-#pragma unroll
-                for (int i = 0; i < V; ++i) xs[j].w[i] = 0u;
-            }
+            xs[j] = Vec<V>{};
+            if (u[j] >= 0) xs[j] = ld_vec<V, CG>(src + (size_t)u[j] * Wn);
         }
         const int64_t en = e + step;
 #pragma unroll
         for (int j = 0; j < 4; ++j) u[j] = en + j < e_end ? __ldg(A.col + en + j) : -1;
-        if constexpr (ModelTraits<MODEL>::counts) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
 #pragma unroll
             for (int i = 0; i < V; ++i) {
-                if (xs[0].w[i] | xs[1].w[i] | xs[2].w[i] | xs[3].w[i])
-                    add4<B>(c[i], xs[0].w[i], xs[1].w[i], xs[2].w[i], xs[3].w[i]);
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-#pragma unroll
-                for (int i = 0; i < V; ++i) {
-                    const uint32_t m = xs[j].w[i] & need[i] & ~newly[i];
-                    if (m) {
-                        constexpr bool W = ModelTraits<MODEL>::weighted;
-                        const int64_t ep = e + j + arcb;   // the caller's arc position
-                        const uint64_t thr = W ? arc_threshold(A, x[i].s, ep) : ic_thr[i];
-                        newly[i] |= lanes_u_less(m, thr, (uint32_t)ep, A.t, x[i].g, W ? TAG_ARC_INFECT : TAG_IC_EDGE,
-                                                 x[i].k0, x[i].k1);
-                    }
+                const uint32_t m = xs[j].w[i] & need[i] & ~newly[i];
+                if (m) {
+                    constexpr bool W = ModelTraits<MODEL>::weighted;
+                    const int64_t ep = e + j + arcb;   // the caller's arc position
+                    const uint64_t thr = W ? arc_threshold(A, x[i].s, ep) : ic_thr[i];
+                    newly[i] |= lanes_u_less(m, thr, (uint32_t)ep, A.t, x[i].g, W ? TAG_ARC_INFECT : TAG_IC_EDGE,
+                                             x[i].k0, x[i].k1);
                 }
             }
         }
@@ -230,8 +304,8 @@ constexpr int min_ctas() { return V == 4 ? 2 : (V == 2 ? (WIDE ? 3 : 4) : 4); }
 // group of 4 arcs) and merge their counts by shuffles; the first team decides.  Shorter
 // per-thread chains for small graphs, whose steps are bound by the longest chain.
 template <int MODEL, int V, int TEAM, bool WARP_ROW, int BT, bool CG, int AG = 1>
-__device__ __forceinline__ void rows_body(const StepArgs &A, int which, int32_t *s_lane,
-                                          unsigned long long *s_pc) {
+__device__ __forceinline__ void rows_body(const StepArgs &A, int which, int32_t *s_lane, unsigned long long *s_pc,
+                                          int bid, int nb) {
     static_assert(AG == 1 || (!WARP_ROW && TEAM * AG <= 32), "arc groups: team rows within a warp");
     constexpr int B = WARP_ROW ? kWideBits : BT;
     constexpr int TPW = 32 / TEAM;
@@ -261,8 +335,8 @@ __device__ __forceinline__ void rows_body(const StepArgs &A, int which, int32_t 
     const int lane = threadIdx.x & 31;
     const int team = lane / TEAM;
     const int tl = lane % TEAM;
-    const int64_t gwarp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t gwarp = ((int64_t)bid * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)nb * blockDim.x) >> 5;
     constexpr int RPI = WARP_ROW ? 1 : TPW / AG;
     const int grp = team % AG;          // arc group of the row (AG > 1)
     const int list_slot = A.k & 1;
@@ -280,7 +354,7 @@ __device__ __forceinline__ void rows_body(const StepArgs &A, int which, int32_t 
     for (int64_t base = gwarp * RPI; base < nitems; base += nwarps * RPI) {
         const int64_t item = WARP_ROW ? base : base + team / AG;
         const bool has_row = item < nitems;
-        const int64_t ridx = has_row ? item / A.nslices : 0;
+        const int64_t ridx = has_row ? div_slices(item, A.nslices, nitems) : 0;
         const int slice = has_row ? (int)(item - ridx * A.nslices) : 0;
         const int32_t v = has_row ? (rows ? __ldg(rows + ridx) : r0 + (int32_t)ridx) : 0;   // new id
         const uint32_t node = has_row ? node_of(A, v) : 0u;                                  // Philox subject
@@ -327,18 +401,18 @@ __device__ __forceinline__ void rows_body(const StepArgs &A, int which, int32_t 
             beg = __ldg(A.rp + v);
             end = __ldg(A.rp + v + 1);
         }
-        if (any_need) {
+        if constexpr (ModelTraits<MODEL>::counts) {
+            constexpr int parts = WARP_ROW ? TPW : AG;   // teams that share a row
+            gather_counts<MODEL, V, B, TEAM, parts, CG>(A, beg, any_need ? end - beg : 0, 8 * parts, w0, lane, c);
+        } else if (any_need) {
             uint64_t ic_thr[V];
-            int64_t arcb = 0;
-            if constexpr (!ModelTraits<MODEL>::counts) arcb = (int64_t)__ldg(A.arc0 + v) - beg;
+            const int64_t arcb = (int64_t)__ldg(A.arc0 + v) - beg;
 #pragma unroll
-            for (int i = 0; i < V; ++i)
-                ic_thr[i] = ModelTraits<MODEL>::counts ? 0ull : ic_threshold(A, x[i].s, end - beg);
-            if (WARP_ROW)
-                gather_arcs<MODEL, V, B, CG>(A, (int64_t)beg + 4 * team, end, 4 * TPW, arcb, w0, need, ic_thr, x, c, newly);
-            else
-                gather_arcs<MODEL, V, B, CG>(A, (int64_t)beg + 4 * grp, end, 4 * AG, arcb, w0, need, ic_thr, x, c,
-                                             newly);
+            for (int i = 0; i < V; ++i) ic_thr[i] = ic_threshold(A, x[i].s, end - beg);
+            // teams that share a row take every TPW-th (AG-th) group of its arcs
+            const int part = WARP_ROW ? team : grp;
+            constexpr int parts = WARP_ROW ? TPW : AG;
+            gather_arcs<MODEL, V, CG>(A, (int64_t)beg + 4 * part, end, 4 * parts, arcb, w0, need, ic_thr, x, newly);
         }
         constexpr bool SPLIT = WARP_ROW && TPW >= V;   // enough teams to give each word one
         if constexpr (SPLIT && V == 2 && ModelTraits<MODEL>::counts) {
@@ -472,20 +546,604 @@ __device__ __forceinline__ void rows_body(const StepArgs &A, int which, int32_t 
         list_append(A, build, want, (int32_t)((uint32_t)v | ((fl & 1u) ? kPushBit : 0u)), list_slot);
         if (sparse && leader) atomicAnd(&A.bitmap[v >> 5], ~(1u << (v & 31)));
     }
-    if (ctx_slice >= 0) {
 #pragma unroll
-        for (int i = 0; i < V; ++i) set_acc_add(s_pc, x[i].s, d0[i], d1[i], d2[i]);
-    }
+    for (int i = 0; i < V; ++i) set_acc_add_warp(s_pc, ctx_slice >= 0 ? x[i].s : -1, d0[i], d1[i], d2[i]);
     flush_accum(A, acc, list_slot, WARP_ROW ? PK_MID : (BT == 4 ? PK_SMALL4 : PK_SMALL));
     set_acc_flush(A, s_pc);
     if (lanes_on) flush_lanes(A, s_lane, nl);
 }
 
+// ------------------------------------------------------------------ warp-tile kernels
+
+// Shape of one warp's tile: SPP word slots per pass (one row slice per team, or one row
+// slice per warp), NP passes.  128 slots keep the queues several batches of 32 long;
+// the wide rows' 16 counter planes take 64.
+template <int MODEL, int V, int TEAM, bool WARP_ROW, int BT>
+struct TileShape {
+    static constexpr bool counts = ModelTraits<MODEL>::counts;
+    static constexpr int B = counts ? (WARP_ROW ? kWideBits : BT) : 1;
+    static constexpr int SW = TEAM * V;
+    static constexpr int SPP = WARP_ROW ? SW : 32 * V;
+    static constexpr int RPP = WARP_ROW ? 1 : 32 / TEAM;
+    static constexpr int TARGET = WARP_ROW ? 64 : 128;
+    static constexpr int NP = SPP >= TARGET ? 1 : TARGET / SPP;
+    static constexpr int NS = NP * SPP;
+    static constexpr int NARC = counts ? 0 : 32 * V + 192;
+    using T = Tile<B, ModelTraits<MODEL>::fixed_draws, NS, NP * RPP, NARC>;
+    static constexpr size_t bytes = sizeof(T) * (kBlock / 32);
+    // slot -> row of the tile and word within the row's slice
+    static __device__ __forceinline__ int row_of_slot(int slot) {
+        return WARP_ROW ? slot / SW : slot / SPP * RPP + (slot & 31) / TEAM;
+    }
+    static __device__ __forceinline__ int word_of_slot(int slot) {
+        return WARP_ROW ? slot % SW : (slot & 31) % TEAM * V + (slot >> 5) % V;
+    }
+};
+
+// Largest dynamic shared memory any row kernel is launched with: its tiles and the
+// per-lane counters (run_wave bounds those by 32 KB).
+constexpr size_t kLaneCounterBytes = 32 * 1024;
+
+// Draws of the tile's count items (infection, exposure, linear thresholds): the result
+// lanes replace counter plane 0.  A lane changes iff its uniform is below its threshold
+// (LT) or reaches it (the survival tables).
+template <int MODEL, int B, class TileT, class CtxFn>
+__device__ __forceinline__ void draw_counts(const StepArgs &A, TileT &T, int n, int lane, CtxFn ctx) {
+    constexpr bool LT = MODEL == FSGP_LT;
+    constexpr uint32_t tag = LT ? TAG_LT_THRESH : TAG_INFECT;
+    const uint32_t t = LT ? 0u : A.t;
+    if (lane == 0) T.ties = 0;
+    __syncwarp();
+#pragma unroll 1
+    for (int q0 = 0; q0 < n; q0 += 32) {
+        const unsigned items = __ballot_sync(0xffffffffu, q0 + lane < n);
+        if (q0 + lane >= n) continue;
+        const int slot = T.qc[q0 + lane];
+        uint32_t c[B];
+#pragma unroll
+        for (int b = 0; b < B; ++b) c[b] = T.c[b][slot];
+        uint32_t node;
+        int w;
+        const int row = ctx(slot, node, w);
+        const SetParams &sp = A.sp[w >> A.ws_shift];
+        const uint32_t g = A.gbase + (uint32_t)(w & (A.Ws - 1));
+        const uint32_t k0 = __ldg(&sp.key0), k1 = __ldg(&sp.key1);
+        const uint32_t cand = any_count<B>(c);
+        // counter planes in use among the items at hand
+        int nb = 0;
+#pragma unroll
+        for (int b = 0; b < B; ++b) nb = __any_sync(items, c[b] != 0u) ? b + 1 : nb;
+        const Planes8 P = philox4x32_10_x2(node, t, g, tag << 8, k0, k1);
+        uint32_t tied = 0u, won = 0u;
+        auto tie_fn = [&](uint32_t lanes, uint32_t th) {
+            tied |= lanes;
+            const int at = atomicAdd(&T.ties, 1);
+            if (at < TileT::kTies) {
+                T.tie_slot[at] = (uint16_t)slot;
+                T.tie_eq[at] = lanes;
+                T.tie_thr[at] = th;
+            } else {
+                const uint32_t less = less_from(lanes, th, 2u, node, t, g, tag, k0, k1);
+                won |= LT ? less : lanes & ~less;
+            }
+        };
+        uint32_t chg;
+        if constexpr (LT) {
+            const int32_t d = __ldg(A.rp + row + 1) - __ldg(A.rp + row);
+            uint32_t sat = 0u;
+            if ((uint64_t)d < (1ull << B)) sat = ge_const<B>(c, (uint32_t)d) & cand;
+            const uint32_t rem = cand & ~sat;
+            chg = sat;
+            if (rem) chg |= counts_u_less_nb<B>(nb, P, c, rem, LtThr{(uint64_t)d}, tie_fn);
+        } else {
+            const int32_t ksat = __ldg(&sp.ksat);
+            uint32_t sat = 0u;
+            if ((uint64_t)ksat < (1ull << B)) sat = ge_const<B>(c, (uint32_t)ksat) & cand;
+            const uint32_t rem = cand & ~sat;
+            chg = cand;
+            if (rem) chg &= ~counts_u_less_nb<B>(nb, P, c, rem, SurvThr{sp.surv}, tie_fn);
+        }
+        T.c[0][slot] = (chg & ~tied) | won;
+    }
+    __syncwarp();
+    const int nt = min(T.ties, TileT::kTies);
+    for (int i = lane; i < nt; i += 32) {
+        const int slot = T.tie_slot[i];
+        const uint32_t eq = T.tie_eq[i];
+        uint32_t node;
+        int w;
+        ctx(slot, node, w);
+        const SetParams &sp = A.sp[w >> A.ws_shift];
+        const uint32_t less = less_from(eq, T.tie_thr[i], 2u, node, t, A.gbase + (uint32_t)(w & (A.Ws - 1)), tag,
+                                        __ldg(&sp.key0), __ldg(&sp.key1));
+        const uint32_t add = LT ? less : eq & ~less;
+        if (add) atomicOr(&T.c[0][slot], add);   // two groups of one word may both be tied
+    }
+    __syncwarp();
+}
+
+template <int MODEL, class TileT, class CtxFn>
+__device__ __forceinline__ void draw_arc_items(const StepArgs &A, TileT &T, int na, int lane, CtxFn ctx) {
+    constexpr bool W = ModelTraits<MODEL>::weighted;
+    draw_arcs(A, T.c[0], T.arc_eq, T.arc_pos, T.arc_slot, na, W ? TAG_ARC_INFECT : TAG_IC_EDGE, lane, ctx,
+              [&A, &T](int row, uint32_t pos, const SetParams &sp) -> uint64_t {
+                  if constexpr (W) return arc_thr(__ldg(&sp.beta_f), __ldg(A.arc_w + pos));
+                  else if (A.ic_mode == FSGP_IC_WEIGHTED_CASCADE) return (uint64_t)T.thr[row] + 1ull;
+                  else return __ldg(&sp.p_const);
+              });
+}
+
+// The tile's draws after its gather (queue lengths nq, nf, na).
+template <int MODEL, int B, class TileT, class CtxFn>
+__device__ __forceinline__ void draw_tile(const StepArgs &A, TileT &T, int nq, const int (&nf)[2], int na, int lane,
+                                          CtxFn ctx) {
+    __syncwarp();
+    if constexpr (ModelTraits<MODEL>::counts) draw_counts<MODEL, B>(A, T, nq, lane, ctx);
+    else draw_arc_items<MODEL>(A, T, na, lane, ctx);
+    if constexpr (ModelTraits<MODEL>::fixed_draws >= 1)
+        draw_fixed(A, T.f[0], T.eq(), T.qf[0], nf[0], TAG_RECOVER, lane, ctx,
+                   [](const SetParams &sp) { return __ldg(&sp.g_rec); });
+    if constexpr (ModelTraits<MODEL>::fixed_draws >= 2)
+        draw_fixed(A, T.f[1], T.eq(), T.qf[1], nf[1], TAG_LATENT, lane, ctx,
+                   [](const SetParams &sp) { return __ldg(&sp.a_lat); });
+}
+
+// Lanes of the word that may leave their state without in-arcs through fixed draw j.
+template <int MODEL>
+__device__ __forceinline__ uint32_t fixed_lanes(int j, uint32_t vm, uint32_t s0, uint32_t s1, uint32_t s2) {
+    if (j == 0) return s0 & vm;
+    return (MODEL == FSGP_SEIR ? s2 : s1) & vm;
+}
+
+// The next state of a word from its tile slot (chg: the lanes changed through in-arcs,
+// f0 / f1: the results of the fixed draws).
+template <int MODEL>
+__device__ __forceinline__ WordOut next_word(uint32_t s0, uint32_t s1, uint32_t s2, uint32_t chg, uint32_t f0,
+                                             uint32_t f1) {
+    WordOut o;
+    o.n1 = o.n2 = 0u;
+    if constexpr (ModelTraits<MODEL>::cascade) {
+        o.n0 = s0 | chg;
+        o.n1 = chg;
+    } else if constexpr (MODEL == FSGP_SEIR) {
+        o.n0 = (s0 & ~f0) | f1;
+        o.n1 = s1 | f0;
+        o.n2 = (s2 & ~f1) | chg;
+    } else if constexpr (MODEL == FSGP_SEIS) {
+        o.n0 = (s0 & ~f0) | f1;
+        o.n1 = (s1 & ~f1) | chg;
+    } else {
+        o.n0 = (s0 & ~f0) | chg;
+        if constexpr (MODEL == FSGP_SIR || MODEL == kSirW) o.n1 = s1 | f0;
+    }
+    return o;
+}
+
+// Arc models: gather the in-arcs [e_begin, e_end) with stride `step` (groups of 4) and
+// queue every (arc, word) pair whose source presses a lane that can change; the queue is
+// worked off whenever the next arcs might not fit.  The whole warp iterates together.
+template <int MODEL, int V, int NARC, bool CG, class TileT, class CtxFn>
+__device__ __forceinline__ void gather_push(const StepArgs &A, TileT &T, int64_t e_begin, int64_t e_end, int64_t step,
+                                            int64_t arcb, int w0, uint32_t (&need)[V], int slot0, int slot_step,
+                                            int lane, int &na, CtxFn ctx) {
+    const uint32_t *src = A.cur + (size_t)ModelTraits<MODEL>::src_plane * A.plane_words + w0;
+    const size_t Wn = (size_t)A.Wn;
+    int32_t u[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) u[j] = e_begin + j < e_end ? __ldg(A.col + e_begin + j) : -1;
+    for (int64_t e = e_begin; __any_sync(0xffffffffu, e < e_end); e += step) {
+        Vec<V> xs[4];
+        uint32_t any = 0u;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (u[j] >= 0) {
+                xs[j] = ld_vec<V, CG>(src + (size_t)u[j] * Wn);
+            } else {
+#pragma unroll
+                for (int i = 0; i < V; ++i) xs[j].w[i] = 0u;
+            }
+        }
+        const int64_t en = e + step;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) u[j] = en + j < e_end ? __ldg(A.col + en + j) : -1;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int i = 0; i < V; ++i) {
+                xs[j].w[i] &= need[i];
+                any |= xs[j].w[i];
+            }
+        if (!__any_sync(0xffffffffu, any != 0u)) continue;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (na > NARC - 32 * V) {
+                __syncwarp();
+                draw_arc_items<MODEL>(A, T, na, lane, ctx);
+                na = 0;
+                // lanes already reached need no more draws
+                bool left = false;
+#pragma unroll
+                for (int i = 0; i < V; ++i) {
+                    need[i] &= ~T.c[0][slot0 + i * slot_step];
+                    left |= need[i] != 0u;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) xs[q].w[i] &= need[i];
+                }
+                if (!__any_sync(0xffffffffu, left)) return;
+            }
+#pragma unroll
+            for (int i = 0; i < V; ++i) {
+                const unsigned m = __ballot_sync(0xffffffffu, xs[j].w[i] != 0u);
+                if (xs[j].w[i]) {
+                    const int at = na + __popc(m & ((1u << lane) - 1u));
+                    T.arc_slot[at] = (uint16_t)(slot0 + i * slot_step);
+                    T.arc_pos[at] = (uint32_t)(e + j + arcb);   // the caller's arc position
+                    T.arc_eq[at] = xs[j].w[i];
+                }
+                na += __popc(m);
+            }
+        }
+    }
+}
+
+// Row kernel on warp tiles: one work item is one slice (TEAM*V words) of one row.
+// WARP_ROW = false: one team per item; true: one warp per item.  which: as in rows_body.
+// CG: state planes through L2 only (persistent step loop).  bid of nb: the CTA's place among
+// those that work on these rows.
+template <int MODEL, int V, int TEAM, bool WARP_ROW, int BT, bool CG>
+__device__ __forceinline__ void rows_tile(const StepArgs &A, int which, uint8_t *smem, int32_t *s_lane,
+                                          unsigned long long *s_pc, int bid, int nb) {
+    using S = TileShape<MODEL, V, TEAM, WARP_ROW, BT>;
+    constexpr int B = S::B;
+    constexpr int TPW = 32 / TEAM;
+    constexpr int SW = TEAM * V;
+    constexpr int P = ModelTraits<MODEL>::planes;
+    constexpr int NF = ModelTraits<MODEL>::fixed_draws;
+    constexpr bool COUNTS = ModelTraits<MODEL>::counts;
+    const Ctl *C = A.ctl;
+    if (*(volatile const int32_t *)&C->stop) return;
+    const bool sparse = *(volatile const int32_t *)&C->sparse != 0;
+    const int32_t *rows = nullptr;   // frontier steps: candidate rows; dense: a range
+    int32_t r0 = 0;
+    int64_t nrows;
+    if (sparse) {
+        if (which >= 2) return;
+        rows = which ? A.cand_mid : A.cand_small;
+        nrows = (int64_t)((volatile const uint32_t *)C->cand_n)[which];
+    } else {
+        r0 = which == 0 ? A.r_small : which == 1 ? A.r_mid : A.r_small4;
+        nrows = which == 0 ? A.n_small : which == 1 ? A.n_mid : A.n_small4;
+    }
+    if (nrows == 0) return;
+    const int nl = A.Wn * 32;
+    const bool lanes_on = A.lane_cnt != nullptr;
+    const bool build = list_wanted(A);
+    if (lanes_on)
+        for (int i = threadIdx.x; i < A.np * nl; i += blockDim.x) s_lane[i] = 0;
+    set_acc_zero(s_pc, A.S);
+    typename S::T &T = reinterpret_cast<typename S::T *>(smem)[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    const int team = lane / TEAM;
+    const int tl = lane % TEAM;
+    const int64_t gwarp = ((int64_t)bid * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)nb * blockDim.x) >> 5;
+    const int list_slot = A.k & 1;
+    const int64_t nitems = nrows * A.nslices;
+    // few rows: fewer passes per tile, so that every warp gets one
+    const int np = (int)min((int64_t)S::NP, max((int64_t)1, nitems / (nwarps * S::RPP)));
+    // the passes of a tile are a whole round of the grid apart: neighbouring rows (the rows
+    // of a class come in descending degree buckets) go to different warps
+    const int64_t round = nwarps * S::RPP;
+    Accum acc;
+    int ctx_slice = -1;              // slice of the valid-lane masks below
+    uint32_t vm[V];
+    int cur_s[V];                    // set of the plane-count changes not yet flushed
+    int32_t d0[V], d1[V], d2[V];
+#pragma unroll
+    for (int i = 0; i < V; ++i) {
+        d0[i] = d1[i] = d2[i] = 0;
+        cur_s[i] = -1;
+        vm[i] = 0u;
+    }
+    auto ctx = [&T](int slot, uint32_t &node, int &w) -> int {
+        const int r = S::row_of_slot(slot);
+        node = T.node[r];
+        w = T.w0[r] + S::word_of_slot(slot);
+        return COUNTS ? T.row[r] : r;
+    };
+
+    for (int64_t base = gwarp * S::RPP; base < nitems; base += np * round) {
+        int nq = 0, na = 0;
+        int nf[2] = {0, 0};
+#pragma unroll 1
+        for (int p = 0; p < np; ++p) {
+            const int64_t item = base + p * round + (WARP_ROW ? 0 : team);
+            const bool has_row = item < nitems;
+            int64_t ridx = 0;
+            int slice = 0;
+            if (has_row) {
+                ridx = div_slices(item, A.nslices, nitems);
+                slice = (int)(item - ridx * A.nslices);
+            }
+            const int32_t v = has_row ? (rows ? __ldg(rows + ridx) : r0 + (int32_t)ridx) : 0;   // new id
+            const int w0 = slice * SW + tl * V;
+            if (slice != ctx_slice) {
+#pragma unroll
+                for (int i = 0; i < V; ++i) vm[i] = word_ctx(A, w0 + i).vm;
+                ctx_slice = slice;
+            }
+            const size_t off = (size_t)v * A.Wn + w0;
+            int32_t beg = 0, end = 0;
+            uint32_t need[V], fx[2][V];
+            {
+                Vec<V> a{}, b{}, e{};
+                if (has_row) {
+                    beg = __ldg(A.rp + v);
+                    end = __ldg(A.rp + v + 1);
+                    a = ld_vec<V, CG>(A.cur + off);
+                    if (P >= 2 && !ModelTraits<MODEL>::cascade) b = ld_vec<V, CG>(A.cur + A.plane_words + off);
+                    if (P >= 3) e = ld_vec<V, CG>(A.cur + 2 * A.plane_words + off);
+                }
+#pragma unroll
+                for (int i = 0; i < V; ++i) {
+                    const uint32_t m = has_row ? vm[i] : 0u;
+                    need[i] = need_of<MODEL>(m, a.w[i], b.w[i], e.w[i]);
+                    fx[0][i] = NF >= 1 && (A.fixed_on & 1) ? fixed_lanes<MODEL>(0, m, a.w[i], b.w[i], e.w[i]) : 0u;
+                    fx[1][i] = NF >= 2 && (A.fixed_on & 2) ? fixed_lanes<MODEL>(1, m, a.w[i], b.w[i], e.w[i]) : 0u;
+                }
+            }
+            uint32_t any_need = 0u;
+#pragma unroll
+            for (int i = 0; i < V; ++i) any_need |= need[i];
+#pragma unroll
+            for (int o = 1; o < TEAM; o <<= 1) any_need |= __shfl_xor_sync(0xffffffffu, any_need, o);
+            const int r = p * S::RPP + (WARP_ROW ? 0 : team);
+            if (WARP_ROW ? lane == 0 : tl == 0) {
+                T.row[r] = has_row ? v : -1;
+                T.node[r] = has_row ? node_of(A, v) : 0u;
+                T.w0[r] = slice * SW;
+                if (A.prof_bytes && has_row) acc.bytes += row_bytes(SW, P, any_need != 0u, end - beg);
+            }
+            const int slot0 = WARP_ROW ? p * SW + tl * V : p * S::SPP + lane;
+            constexpr int slot_step = WARP_ROW ? 1 : 32;
+            if constexpr (COUNTS) {
+                uint32_t c[V][B];
+#pragma unroll
+                for (int i = 0; i < V; ++i)
+#pragma unroll
+                    for (int b = 0; b < B; ++b) c[i][b] = 0u;
+                constexpr int parts = WARP_ROW ? TPW : 1;
+                gather_counts<MODEL, V, B, TEAM, parts, CG>(A, beg, any_need ? end - beg : 0, 8 * parts, w0, lane, c);
+                constexpr bool SPLIT = WARP_ROW && TPW >= V;   // team i < V stores word i
+                if constexpr (SPLIT && V == 2) {
+                    // merge the teams' counters, reduce-scatter first: at the first level the
+                    // partners (teams 2j, 2j+1) swap halves and keep word (team & 1) each
+                    const int par = team & 1;
+                    uint32_t d[B];
+#pragma unroll
+                    for (int b = 0; b < B; ++b) d[b] = __shfl_xor_sync(0xffffffffu, par ? c[0][b] : c[1][b], TEAM);
+#pragma unroll
+                    for (int b = 0; b < B; ++b) c[0][b] = par ? c[1][b] : c[0][b];
+                    add_sliced<B>(c[0], d);
+#pragma unroll
+                    for (int o = 2 * TEAM; o < 32; o <<= 1) {
+#pragma unroll
+                        for (int b = 0; b < B; ++b) d[b] = __shfl_xor_sync(0xffffffffu, c[0][b], o);
+                        add_sliced<B>(c[0], d);
+                    }
+#pragma unroll
+                    for (int b = 0; b < B; ++b) c[1][b] = c[0][b];
+                } else if constexpr (WARP_ROW) {
+#pragma unroll
+                    for (int o = TEAM; o < 32; o <<= 1)
+#pragma unroll
+                        for (int i = 0; i < V; ++i) {
+                            uint32_t d[B];
+#pragma unroll
+                            for (int b = 0; b < B; ++b) d[b] = __shfl_xor_sync(0xffffffffu, c[i][b], o);
+                            add_sliced<B>(c[i], d);
+                        }
+                }
+#pragma unroll
+                for (int i = 0; i < V; ++i) {
+                    // the threads that store word i of their slice
+                    const bool mine = WARP_ROW ? (SPLIT ? team == i : team == 0) : true;
+                    const int slot = slot0 + i * slot_step;
+                    uint32_t any = 0u;
+#pragma unroll
+                    for (int b = 0; b < B; ++b) {
+                        c[i][b] &= need[i];
+                        any |= c[i][b];
+                    }
+                    if (mine) {
+                        T.c[0][slot] = c[i][0];
+                        if (any)
+#pragma unroll
+                            for (int b = 1; b < B; ++b) T.c[b][slot] = c[i][b];
+                    }
+                    queue_push(T.qc, nq, mine && any != 0u, slot, lane);
+                }
+            } else {
+                // (every lane of the warp joins the gather)
+                const int64_t arcb = has_row ? (int64_t)__ldg(A.arc0 + v) - beg : 0;
+                if (MODEL == FSGP_IC && (WARP_ROW ? lane == 0 : tl == 0))
+                    T.thr[r] = 0xffffffffu / (uint32_t)max(end - beg, 1);
+                if (!WARP_ROW || team == 0)
+#pragma unroll
+                    for (int i = 0; i < V; ++i) T.c[0][slot0 + i * slot_step] = 0u;
+                __syncwarp();
+                if (!any_need) end = beg;
+                gather_push<MODEL, V, S::NARC, CG>(A, T, (int64_t)beg + (WARP_ROW ? 4 * team : 0), end,
+                                               WARP_ROW ? 4 * TPW : 4, arcb, w0, need, slot0, slot_step, lane, na, ctx);
+            }
+            if constexpr (NF >= 1) {
+#pragma unroll
+                for (int i = 0; i < V; ++i) {
+                    const bool mine = !WARP_ROW || team == 0;
+                    const int slot = slot0 + i * slot_step;
+#pragma unroll
+                    for (int j = 0; j < NF; ++j) {
+                        if (mine) T.f[j][slot] = fx[j][i];
+                        queue_push(T.qf[j], nf[j], mine && fx[j][i] != 0u, slot, lane);
+                    }
+                }
+            }
+        }
+        draw_tile<MODEL, B>(A, T, nq, nf, na, lane, ctx);
+        __syncwarp();
+        // next states
+        if constexpr (!WARP_ROW) {
+#pragma unroll 1
+            for (int p = 0; p < np; ++p) {
+                const int r = p * S::RPP + team;
+                const int32_t v = T.row[r];
+                const int w0 = T.w0[r] + tl * V;
+                uint32_t fl = 0u;
+                if (v >= 0) {
+                    const size_t off = (size_t)v * A.Wn + w0;
+                    const Vec<V> a = ld_vec<V, CG>(A.cur + off);
+                    Vec<V> b{}, e{};
+                    if (P >= 2) b = ld_vec<V, CG>(A.cur + A.plane_words + off);
+                    if (P >= 3) e = ld_vec<V, CG>(A.cur + 2 * A.plane_words + off);
+                    uint32_t n0[V], n1[V], n2[V];
+#pragma unroll
+                    for (int i = 0; i < V; ++i) {
+                        const int slot = p * S::SPP + i * 32 + lane;
+                        const WordOut o = next_word<MODEL>(a.w[i], b.w[i], e.w[i], T.c[0][slot],
+                                                           T.template fixed<0>(slot), T.template fixed<1>(slot));
+                        n0[i] = o.n0;
+                        n1[i] = o.n1;
+                        n2[i] = o.n2;
+                        const int s = (w0 + i) >> A.ws_shift;
+                        if (s != cur_s[i]) {
+                            if (cur_s[i] >= 0) set_acc_add(s_pc, cur_s[i], d0[i], d1[i], d2[i]);
+                            d0[i] = d1[i] = d2[i] = 0;
+                            cur_s[i] = s;
+                        }
+                        d0[i] += __popc(o.n0) - __popc(a.w[i]);
+                        if (P >= 2) d1[i] += __popc(o.n1) - __popc(b.w[i]);
+                        if (P >= 3) d2[i] += __popc(o.n2) - __popc(e.w[i]);
+                        if (lanes_on) {
+                            lane_deltas(s_lane, w0 + i, a.w[i], o.n0);
+                            if (P >= 2) lane_deltas(s_lane + nl, w0 + i, b.w[i], o.n1);
+                            if (P >= 3) lane_deltas(s_lane + 2 * nl, w0 + i, e.w[i], o.n2);
+                        }
+                        fl |= word_flags<MODEL>(o, a.w[i], b.w[i], e.w[i]);
+                    }
+                    st_vec<V>(A.nxt + off, n0);
+                    if (P >= 2) st_vec<V>(A.nxt + A.plane_words + off, n1);
+                    if (P >= 3) st_vec<V>(A.nxt + 2 * A.plane_words + off, n2);
+                }
+#pragma unroll
+                for (int o = 1; o < TEAM; o <<= 1) fl |= __shfl_xor_sync(0xffffffffu, fl, o);
+                const bool leader = v >= 0 && tl == 0;
+                const bool want = leader && fl != 0u;
+                if (want && (fl & 1u)) {
+                    const uint32_t node = T.node[r];
+                    acc.push_deg += (unsigned long long)(__ldg(A.out_ptr + node + 1) - __ldg(A.out_ptr + node));
+                }
+                list_append(A, build, want, (int32_t)((uint32_t)v | ((fl & 1u) ? kPushBit : 0u)), list_slot);
+                if (sparse && leader) atomicAnd(&A.bitmap[v >> 5], ~(1u << (v & 31)));
+            }
+        } else {
+            // one lane per word slot; a row's words are SW neighbouring lanes (a slice wider
+            // than the warp: several rounds of one row)
+            constexpr int GRP = SW < 32 ? SW : 32;
+            uint32_t fl = 0u;
+#pragma unroll 1
+            for (int q0 = 0; q0 < np * SW; q0 += 32) {
+                const int slot = q0 + lane;
+                const int r = slot / SW;
+                const int32_t v = slot < np * SW ? T.row[r] : -1;
+                if (q0 % SW == 0) fl = 0u;
+                if (v >= 0) {
+                    const int w = T.w0[r] + slot % SW;
+                    const size_t off = (size_t)v * A.Wn + w;
+                    const uint32_t s0 = ld_word<CG>(A.cur + off);
+                    const uint32_t s1 = P >= 2 ? ld_word<CG>(A.cur + A.plane_words + off) : 0u;
+                    const uint32_t s2 = P >= 3 ? ld_word<CG>(A.cur + 2 * A.plane_words + off) : 0u;
+                    const WordOut o = next_word<MODEL>(s0, s1, s2, T.c[0][slot], T.template fixed<0>(slot),
+                                                       T.template fixed<1>(slot));
+                    A.nxt[off] = o.n0;
+                    if (P >= 2) A.nxt[A.plane_words + off] = o.n1;
+                    if (P >= 3) A.nxt[2 * A.plane_words + off] = o.n2;
+                    const int s = w >> A.ws_shift;
+                    if (s != cur_s[0]) {
+                        if (cur_s[0] >= 0) set_acc_add(s_pc, cur_s[0], d0[0], d1[0], d2[0]);
+                        d0[0] = d1[0] = d2[0] = 0;
+                        cur_s[0] = s;
+                    }
+                    d0[0] += __popc(o.n0) - __popc(s0);
+                    if (P >= 2) d1[0] += __popc(o.n1) - __popc(s1);
+                    if (P >= 3) d2[0] += __popc(o.n2) - __popc(s2);
+                    if (lanes_on) {
+                        lane_deltas(s_lane, w, s0, o.n0);
+                        if (P >= 2) lane_deltas(s_lane + nl, w, s1, o.n1);
+                        if (P >= 3) lane_deltas(s_lane + 2 * nl, w, s2, o.n2);
+                    }
+                    fl |= word_flags<MODEL>(o, s0, s1, s2);
+                }
+                if (SW <= 32 || (q0 + 32) % SW == 0) {
+#pragma unroll
+                    for (int o = 1; o < GRP; o <<= 1) fl |= __shfl_xor_sync(0xffffffffu, fl, o);
+                    const bool leader = v >= 0 && lane % GRP == 0;
+                    const bool want = leader && fl != 0u;
+                    if (want && (fl & 1u)) {
+                        const uint32_t node = T.node[r];
+                        acc.push_deg += (unsigned long long)(__ldg(A.out_ptr + node + 1) - __ldg(A.out_ptr + node));
+                    }
+                    list_append(A, build, want, (int32_t)((uint32_t)v | ((fl & 1u) ? kPushBit : 0u)), list_slot);
+                    if (sparse && leader) atomicAnd(&A.bitmap[v >> 5], ~(1u << (v & 31)));
+                    fl = 0u;
+                }
+            }
+        }
+        __syncwarp();   // the next tile overwrites the slots
+    }
+#pragma unroll
+    for (int i = 0; i < V; ++i) set_acc_add_warp(s_pc, cur_s[i], d0[i], d1[i], d2[i]);
+    flush_accum(A, acc, list_slot, WARP_ROW ? PK_MID : (BT == 4 ? PK_SMALL4 : PK_SMALL));
+    set_acc_flush(A, s_pc);
+    if (lanes_on) flush_lanes(A, s_lane, nl);
+}
+
+// The rows of one class: through the warp tile, or in place (SWIR; AG as in rows_body).
+template <int MODEL, int V, int TEAM, bool WARP_ROW, int BT, bool CG, int AG = 1>
+__device__ __forceinline__ void rows_class(const StepArgs &A, int which, uint8_t *smem, int32_t *s_lane,
+                                           unsigned long long *s_pc, int bid, int nb) {
+    if constexpr (ModelTraits<MODEL>::tiled) rows_tile<MODEL, V, TEAM, WARP_ROW, BT, CG>(A, which, smem, s_lane, s_pc, bid, nb);
+    else rows_body<MODEL, V, TEAM, WARP_ROW, BT, CG, AG>(A, which, s_lane, s_pc, bid, nb);
+}
+
+// Dynamic shared memory of a class's tiles, and of either class's (fused kernels).
+template <int MODEL, int V, int TEAM, bool WARP_ROW, int BT>
+constexpr size_t TileBytes = ModelTraits<MODEL>::tiled ? TileShape<MODEL, V, TEAM, WARP_ROW, BT>::bytes : 0;
+template <int MODEL, int V, int TEAM>
+constexpr size_t FusedBytes = std::max(TileBytes<MODEL, V, TEAM, true, kSmallBits>,
+                                       TileBytes<MODEL, V, TEAM, false, kSmallBits>);
+
 template <int MODEL, int V, int TEAM, bool WARP_ROW, int BT = kSmallBits>
 __global__ void __launch_bounds__(kBlock, min_ctas<V, WARP_ROW>()) k_rows(StepArgs A, int which) {
-    extern __shared__ int32_t s_lane[];
+    extern __shared__ __align__(16) uint8_t s_dyn[];
     __shared__ unsigned long long s_pc[kPC * kMaxSets];
-    rows_body<MODEL, V, TEAM, WARP_ROW, BT, false>(A, which, s_lane, s_pc);
+    constexpr size_t tile = TileBytes<MODEL, V, TEAM, WARP_ROW, BT>;
+    rows_class<MODEL, V, TEAM, WARP_ROW, BT, false>(A, which, s_dyn, reinterpret_cast<int32_t *>(s_dyn + tile), s_pc,
+                                                    blockIdx.x, gridDim.x);
+}
+
+// Small graphs: both row classes in one launch, the first `warp_ctas` CTAs on the rows that
+// get a warp each, the others on the rows that get a team each, so that neither waits for
+// the other's last row.
+template <int MODEL, int V, int TEAM>
+__global__ void __launch_bounds__(kBlock, V == 4 ? 2 : 3) k_rows_fused(StepArgs A, int warp_ctas) {
+    extern __shared__ __align__(16) uint8_t s_dyn[];
+    __shared__ unsigned long long s_pc[kPC * kMaxSets];
+    int32_t *s_lane = reinterpret_cast<int32_t *>(s_dyn + FusedBytes<MODEL, V, TEAM>);
+    if ((int)blockIdx.x < warp_ctas)
+        rows_class<MODEL, V, TEAM, true, kSmallBits, false>(A, 1, s_dyn, s_lane, s_pc, blockIdx.x, warp_ctas);
+    else
+        rows_class<MODEL, V, TEAM, false, kSmallBits, false>(A, 0, s_dyn, s_lane, s_pc, blockIdx.x - warp_ctas,
+                                                            gridDim.x - warp_ctas);
 }
 
 // Persistent step loop of a small graph: all T dense steps in one launch, the row work of
@@ -497,10 +1155,11 @@ __global__ void __launch_bounds__(kBlock, min_ctas<V, WARP_ROW>()) k_rows(StepAr
 // (CG loads): a CTA reads at step k the words other CTAs wrote at step k-1.
 // (bounded for 2 resident CTAs per SM: the loop is meant for graphs that fill a few CTAs
 // per SM at most, and the body then keeps its state in registers)
-template <int MODEL, int V, int TEAM, bool WARP_ROW, int BT = kSmallBits, int AG = 1>
+template <int MODEL, int TEAM>
 __global__ void __launch_bounds__(kBlock, 2)
     k_rows_persist(const __grid_constant__ StepArgs A0, const __grid_constant__ PersistArgs Q) {
-    extern __shared__ int32_t s_lane[];
+    extern __shared__ __align__(16) uint8_t s_dyn[];
+    int32_t *s_lane = reinterpret_cast<int32_t *>(s_dyn + FusedBytes<MODEL, 1, TEAM>);
     __shared__ unsigned long long s_pc[kPC * kMaxSets];
     __shared__ StepArgs sA;
     __shared__ unsigned long long s_new[kMaxSets];   // cascade: lanes newly active at the last step
@@ -535,7 +1194,11 @@ __global__ void __launch_bounds__(kBlock, 2)
             if (blockIdx.x == 0 && threadIdx.x == 0) C->stop = 1;
             break;
         }
-        rows_body<MODEL, V, TEAM, WARP_ROW, BT, true, AG>(sA, WARP_ROW ? 1 : 0, s_lane, s_pc);
+        if ((int)blockIdx.x < Q.warp_ctas)
+            rows_class<MODEL, 1, TEAM, true, kSmallBits, true>(sA, 1, s_dyn, s_lane, s_pc, blockIdx.x, Q.warp_ctas);
+        else
+            rows_class<MODEL, 1, TEAM, false, kSmallBits, true>(sA, 0, s_dyn, s_lane, s_pc, blockIdx.x - Q.warp_ctas,
+                                                                gridDim.x - Q.warp_ctas);
         if (!grid_barrier(&C->bar_count, &C->bar_gen, gridDim.x, &C->err, Q.spin_limit)) break;
         if (blockIdx.x == 0 && threadIdx.x == 0) C->steps_done = k;
         if (cascade)
@@ -626,7 +1289,15 @@ __global__ void __launch_bounds__(kBlock, min_ctas<V, true>()) k_hub_chunks(Step
 #pragma unroll
             for (int b = 0; b < B; ++b) c[i][b] = 0u;
         }
-        gather_arcs<MODEL, V, B>(A, beg + 4 * team, end, 4 * TPB, arcb, w0, need, ic_thr, x, c, newly);
+        if constexpr (ModelTraits<MODEL>::counts)
+        {
+            // the warps take the chunk's groups of 8 arcs per team in turn
+            constexpr int per_warp = 8 * (32 / TEAM);
+            const int off = (threadIdx.x >> 5) * per_warp;
+            gather_counts<MODEL, V, B, TEAM, 32 / TEAM>(A, beg + off, (int32_t)(end - beg) - off, 8 * TPB, w0, lane, c);
+        }
+        else
+            gather_arcs<MODEL, V>(A, beg + 4 * team, end, 4 * TPB, arcb, w0, need, ic_thr, x, newly);
 #pragma unroll
         for (int o = TEAM; o < 32; o <<= 1) {
 #pragma unroll
@@ -825,11 +1496,9 @@ __device__ __forceinline__ uint32_t self_lanes(uint32_t s0, uint32_t s1, uint32_
 }
 
 template <int MODEL, int SWL>
-__global__ void __launch_bounds__(kBlock) k_rows_lane(StepArgs A) {
-    extern __shared__ int32_t s_lane[];
-    __shared__ unsigned long long s_pc[kPC * kMaxSets];
+__device__ __forceinline__ void lane_body(const StepArgs &A, uint8_t *smem, int32_t *s_lane, unsigned long long *s_pc) {
     constexpr int P = ModelTraits<MODEL>::planes;
-    __shared__ LaneStage<SWL, P> st;
+    LaneStage<SWL, P> &st = *reinterpret_cast<LaneStage<SWL, P> *>(smem);
     const Ctl *C = A.ctl;
     if (*(volatile const int32_t *)&C->stop) return;
     if (*(volatile const int32_t *)&C->sparse) return;
@@ -857,7 +1526,7 @@ __global__ void __launch_bounds__(kBlock) k_rows_lane(StepArgs A) {
         int w0 = 0;
         uint32_t busy = 0u;
         if (has) {
-            const int64_t r = item / nsl;
+            const int64_t r = div_slices(item, nsl, nitems);
             w0 = (int)(item - r * nsl) * SWL;
             int4 e;
             if (r < A.n_lane) {
@@ -986,26 +1655,265 @@ __global__ void __launch_bounds__(kBlock) k_rows_lane(StepArgs A) {
         if (A.prof_bytes && has) acc.bytes += row_bytes(SWL, P, d > 0, d);
         list_append(A, build, want, (int32_t)((uint32_t)v | ((fl & 1u) ? kPushBit : 0u)), list_slot);
     }
-    if (cur_s >= 0) set_acc_add(s_pc, cur_s, dd0, dd1, dd2);
+    set_acc_add_warp(s_pc, cur_s, dd0, dd1, dd2);
     flush_accum(A, acc, list_slot, PK_LANE);
     set_acc_flush(A, s_pc);
     if (lanes_on) flush_lanes(A, s_lane, nl);
 }
 
-// Widest slice of the one-thread-per-row kernel: its staging area (planes + 3 sources,
-// SWL words, 256 threads) must fit the 48 KB of static shared memory.
+// The same rows through the warp tile: 32 row slices of SWL words per warp.
+template <int MODEL, int SWL>
+struct LaneShape {
+    static constexpr bool counts = ModelTraits<MODEL>::counts;
+    static constexpr int B = counts ? 2 : 1;
+    static constexpr int NARC = counts ? 0 : 256;
+    using T = Tile<B, ModelTraits<MODEL>::fixed_draws, 32 * SWL, 32, NARC>;
+    static constexpr size_t bytes = sizeof(T) * (kBlock / 32);
+};
+
+template <int MODEL, int SWL>
+__device__ __forceinline__ void lane_tile(const StepArgs &A, uint8_t *smem, int32_t *s_lane, unsigned long long *s_pc) {
+    using S = LaneShape<MODEL, SWL>;
+    constexpr int P = ModelTraits<MODEL>::planes;
+    constexpr int NF = ModelTraits<MODEL>::fixed_draws;
+    constexpr int VL = SWL < 4 ? SWL : 4;
+    constexpr bool COUNTS = ModelTraits<MODEL>::counts;
+    const Ctl *C = A.ctl;
+    if (*(volatile const int32_t *)&C->stop) return;
+    if (*(volatile const int32_t *)&C->sparse) return;
+    const int nsl = A.Wn / SWL;
+    const int64_t n_rows = (int64_t)A.n_lane + *(volatile const uint32_t *)&C->d0_n;
+    const int64_t nitems = n_rows * nsl;
+    if (nitems == 0) return;
+    const int nl = A.Wn * 32;
+    const bool lanes_on = A.lane_cnt != nullptr;
+    const bool build = list_wanted(A);
+    if (lanes_on)
+        for (int i = threadIdx.x; i < A.np * nl; i += blockDim.x) s_lane[i] = 0;
+    set_acc_zero(s_pc, A.S);
+    typename S::T &T = reinterpret_cast<typename S::T *>(smem)[threadIdx.x >> 5];
+    const int list_slot = A.k & 1;
+    const int lane = threadIdx.x & 31;
+    const int64_t gwarp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const uint32_t *src_plane = A.cur + (size_t)ModelTraits<MODEL>::src_plane * A.plane_words;
+    Accum acc;
+    int cur_s = -1;           // set of the plane-count deltas not yet flushed
+    int32_t dd0 = 0, dd1 = 0, dd2 = 0;
+    auto ctx = [&T](int slot, uint32_t &node, int &w) -> int {
+        node = T.node[slot & 31];
+        w = T.w0[slot & 31] + (slot >> 5);
+        return COUNTS ? T.row[slot & 31] : (slot & 31);
+    };
+    for (int64_t base = gwarp * 32; base < nitems; base += nwarps * 32) {
+        const int64_t item = base + lane;
+        const bool has = item < nitems;
+        int nq = 0, na = 0;
+        int nf[2] = {0, 0};
+        int32_t v = 0, beg = 0, d = 0;   // v: new id
+        int w0 = 0;
+        int4 e4 = make_int4(0, -1, -1, -1);
+        if (has) {
+            const int64_t r = div_slices(item, nsl, nitems);
+            w0 = (int)(item - r * nsl) * SWL;
+            if (r < A.n_lane) {
+                e4 = __ldg(A.lane_tab + r);   // the node and its sources in one entry
+                v = A.r_lane + (int32_t)r;
+            } else {
+                v = A.d0_list[r - A.n_lane];
+                e4.x = (int32_t)node_of(A, v);
+            }
+            d = (e4.y >= 0) + (e4.z >= 0) + (e4.w >= 0);
+            if (!COUNTS && d > 0) beg = __ldg(A.arc0 + v);   // arc positions key the draws
+        }
+        T.row[lane] = has ? v : -1;
+        T.node[lane] = (uint32_t)e4.x;
+        T.w0[lane] = w0;
+        if (MODEL == FSGP_IC) T.thr[lane] = 0xffffffffu / (uint32_t)max(d, 1);
+        __syncwarp();
+        const size_t off = (size_t)v * A.Wn + w0;
+        const int32_t u[kLaneMaxDeg] = {e4.y, e4.z, e4.w};
+#pragma unroll
+        for (int q = 0; q < SWL; q += VL) {
+            Vec<VL> a{}, b{}, ee{}, x[kLaneMaxDeg];
+            if (has) {
+                a = ldg_vec<VL>(A.cur + off + q);
+                if (P >= 2 && !ModelTraits<MODEL>::cascade) b = ldg_vec<VL>(A.cur + A.plane_words + off + q);
+                if (P >= 3) ee = ldg_vec<VL>(A.cur + 2 * A.plane_words + off + q);
+            }
+#pragma unroll
+            for (int j = 0; j < kLaneMaxDeg; ++j) {
+                x[j] = Vec<VL>{};
+                if (u[j] >= 0) x[j] = ldg_vec<VL>(src_plane + (size_t)u[j] * A.Wn + w0 + q);
+            }
+#pragma unroll
+            for (int i = 0; i < VL; ++i) {
+                const int slot = (q + i) * 32 + lane;
+                const uint32_t vm = has ? word_ctx(A, w0 + q + i).vm : 0u;
+                const uint32_t need = need_of<MODEL>(vm, a.w[i], b.w[i], ee.w[i]);
+                const uint32_t x0 = x[0].w[i], x1 = x[1].w[i], x2 = x[2].w[i];
+                if constexpr (COUNTS) {
+                    const uint32_t c0 = (x0 ^ x1 ^ x2) & need;
+                    const uint32_t c1 = ((x0 & x1) | (x2 & (x0 ^ x1))) & need;
+                    T.c[0][slot] = c0;
+                    T.c[1][slot] = c1;
+                    queue_push(T.qc, nq, (c0 | c1) != 0u, slot, lane);
+                } else {
+                    T.c[0][slot] = 0u;
+                    const uint32_t xs[kLaneMaxDeg] = {x0 & need, x1 & need, x2 & need};
+#pragma unroll
+                    for (int j = 0; j < kLaneMaxDeg; ++j) {
+                        const unsigned m = __ballot_sync(0xffffffffu, xs[j] != 0u);
+                        if (m == 0u) continue;
+                        if (na > S::NARC - 32) {
+                            __syncwarp();
+                            draw_arc_items<MODEL>(A, T, na, lane, ctx);
+                            na = 0;
+                        }
+                        if (xs[j]) {
+                            const int at = na + __popc(m & ((1u << lane) - 1u));
+                            T.arc_slot[at] = (uint16_t)slot;
+                            T.arc_pos[at] = (uint32_t)(beg + j);
+                            T.arc_eq[at] = xs[j];
+                        }
+                        na += __popc(m);
+                    }
+                }
+                if constexpr (NF >= 1) {
+                    const uint32_t f0 = (A.fixed_on & 1) ? fixed_lanes<MODEL>(0, vm, a.w[i], b.w[i], ee.w[i]) : 0u;
+                    T.f[0][slot] = f0;
+                    queue_push(T.qf[0], nf[0], f0 != 0u, slot, lane);
+                }
+                if constexpr (NF >= 2) {
+                    const uint32_t f1 = (A.fixed_on & 2) ? fixed_lanes<MODEL>(1, vm, a.w[i], b.w[i], ee.w[i]) : 0u;
+                    T.f[1][slot] = f1;
+                    queue_push(T.qf[1], nf[1], f1 != 0u, slot, lane);
+                }
+            }
+        }
+        draw_tile<MODEL, S::B>(A, T, nq, nf, na, lane, ctx);
+        __syncwarp();
+        uint32_t fl = 0u;
+        if (has) {
+#pragma unroll
+            for (int q = 0; q < SWL; q += VL) {
+                const Vec<VL> a = ldg_vec<VL>(A.cur + off + q);
+                Vec<VL> b{}, ee{};
+                if (P >= 2) b = ldg_vec<VL>(A.cur + A.plane_words + off + q);
+                if (P >= 3) ee = ldg_vec<VL>(A.cur + 2 * A.plane_words + off + q);
+                uint32_t n0[VL], n1[VL], n2[VL];
+#pragma unroll
+                for (int i = 0; i < VL; ++i) {
+                    const int slot = (q + i) * 32 + lane;
+                    const WordOut o = next_word<MODEL>(a.w[i], b.w[i], ee.w[i], T.c[0][slot], T.template fixed<0>(slot),
+                                                       T.template fixed<1>(slot));
+                    n0[i] = o.n0;
+                    n1[i] = o.n1;
+                    n2[i] = o.n2;
+                    const int s = (w0 + q + i) >> A.ws_shift;
+                    if (s != cur_s) {
+                        if (cur_s >= 0) set_acc_add(s_pc, cur_s, dd0, dd1, dd2);
+                        cur_s = s;
+                        dd0 = dd1 = dd2 = 0;
+                    }
+                    dd0 += __popc(o.n0) - __popc(a.w[i]);
+                    if (P >= 2) dd1 += __popc(o.n1) - __popc(b.w[i]);
+                    if (P >= 3) dd2 += __popc(o.n2) - __popc(ee.w[i]);
+                    if (lanes_on) {
+                        lane_deltas(s_lane, w0 + q + i, a.w[i], o.n0);
+                        if (P >= 2) lane_deltas(s_lane + nl, w0 + q + i, b.w[i], o.n1);
+                        if (P >= 3) lane_deltas(s_lane + 2 * nl, w0 + q + i, ee.w[i], o.n2);
+                    }
+                    fl |= word_flags<MODEL>(o, a.w[i], b.w[i], ee.w[i]);
+                }
+                st_vec<VL>(A.nxt + off + q, n0);
+                if (P >= 2) st_vec<VL>(A.nxt + A.plane_words + off + q, n1);
+                if (P >= 3) st_vec<VL>(A.nxt + 2 * A.plane_words + off + q, n2);
+            }
+        }
+        const bool want = has && fl != 0u;
+        if (want && (fl & 1u)) {
+            const uint32_t node = (uint32_t)e4.x;
+            acc.push_deg += (unsigned long long)(__ldg(A.out_ptr + node + 1) - __ldg(A.out_ptr + node));
+        }
+        if (A.prof_bytes && has) acc.bytes += row_bytes(SWL, P, d > 0, d);
+        list_append(A, build, want, (int32_t)((uint32_t)v | ((fl & 1u) ? kPushBit : 0u)), list_slot);
+        __syncwarp();   // the next tile overwrites the slots
+    }
+    set_acc_add_warp(s_pc, cur_s, dd0, dd1, dd2);
+    flush_accum(A, acc, list_slot, PK_LANE);
+    set_acc_flush(A, s_pc);
+    if (lanes_on) flush_lanes(A, s_lane, nl);
+}
+
+// Bytes of the staging area or of the warps' tiles.
+template <int MODEL, int SWL>
+constexpr size_t kLaneSmem = ModelTraits<MODEL>::tiled ? LaneShape<MODEL, SWL>::bytes
+                                                       : sizeof(LaneStage<SWL, ModelTraits<MODEL>::planes>);
+
+template <int MODEL, int SWL>
+__global__ void __launch_bounds__(kBlock, ModelTraits<MODEL>::tiled ? 4 : 1) k_rows_lane(StepArgs A) {
+    extern __shared__ __align__(16) uint8_t s_dyn[];
+    __shared__ unsigned long long s_pc[kPC * kMaxSets];
+    int32_t *s_lane = reinterpret_cast<int32_t *>(s_dyn + kLaneSmem<MODEL, SWL>);
+    if constexpr (ModelTraits<MODEL>::tiled) lane_tile<MODEL, SWL>(A, s_dyn, s_lane, s_pc);
+    else lane_body<MODEL, SWL>(A, s_dyn, s_lane, s_pc);
+}
+
+// Resident CTAs per SM of a kernel with `tile` bytes of dynamic shared memory (`smem` with
+// the per-lane counters of this run).  The kernel also asks for no more of the SM's 256 KB
+// than those CTAs' shared memory: the default takes the largest carve-out as soon as one
+// more CTA would fit by shared memory alone, and what is left as L1 (28 KB) then has too
+// few lines for the gathered rows in flight (random 32-byte rows out of L2: 287e9 rows/s
+// with 60 KB of L1 or more, 153e9 with 28 KB).
+inline int resident_ctas(const void *kern, size_t smem, size_t tile) {
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(tile + kLaneCounterBytes));
+    int z = 1, z0 = 1;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&z, kern, kBlock, smem + tile);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&z0, kern, kBlock, tile);
+    if (z < 1) z = 1;
+    cudaFuncAttributes at{};
+    int per_sm = 0, dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess && cudaFuncGetAttributes(&at, kern) == cudaSuccess &&
+        cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) == cudaSuccess && per_sm > 0) {
+        const size_t need = (size_t)std::max(z0, 1) * (tile + at.sharedSizeBytes + 1024);   // 1 KB is the system's
+        cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
+                             (int)std::min<size_t>(100, (need * 100 + per_sm - 1) / (size_t)per_sm));
+    }
+    return z;
+}
+
+// The same, asked once per kernel, device and size in a row (a small graph's run is shorter
+// than a handful of driver queries are cheap).  The attributes set are the same every time:
+// the shared-memory limit is raised to the tiles plus the largest per-lane counter area any
+// run uses, since host threads of a batch may set it concurrently.
+template <auto Kern>
+int occupancy_one(size_t smem, size_t tile) {
+    static std::atomic<uint64_t> last{0};   // 1 << 63 | device << 48 | smem << 16 | CTAs
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev >= 1 << 15) return resident_ctas((const void *)Kern, smem, tile);
+    const uint64_t key = 1ull << 63 | (uint64_t)dev << 48 | (uint64_t)smem << 16;
+    const uint64_t seen = last.load(std::memory_order_acquire);
+    if ((seen & ~0xffffull) == key) return (int)(seen & 0xffffull);
+    const int z = resident_ctas((const void *)Kern, smem, tile);
+    last.store(key | (uint64_t)z, std::memory_order_release);
+    return z;
+}
+
+// Widest slice of the one-thread-per-row kernel: the staging area of the three-plane
+// models (planes + 3 sources, SWL words, 256 threads) grows past 48 KB with 8 words.
 template <int MODEL>
 constexpr int lane_swl_max() { return ModelTraits<MODEL>::planes >= 3 ? 4 : 8; }
 
 template <int MODEL>
 int launch_rows_lane(const StepArgs &A, int swl, int grid, size_t smem, cudaStream_t s) {
     switch (swl) {
-        case 1: k_rows_lane<MODEL, 1><<<grid, kBlock, smem, s>>>(A); break;
-        case 2: k_rows_lane<MODEL, 2><<<grid, kBlock, smem, s>>>(A); break;
-        case 4: k_rows_lane<MODEL, 4><<<grid, kBlock, smem, s>>>(A); break;
+        case 1: k_rows_lane<MODEL, 1><<<grid, kBlock, smem + kLaneSmem<MODEL, 1>, s>>>(A); break;
+        case 2: k_rows_lane<MODEL, 2><<<grid, kBlock, smem + kLaneSmem<MODEL, 2>, s>>>(A); break;
+        case 4: k_rows_lane<MODEL, 4><<<grid, kBlock, smem + kLaneSmem<MODEL, 4>, s>>>(A); break;
         case 8:
             if constexpr (lane_swl_max<MODEL>() >= 8) {
-                k_rows_lane<MODEL, 8><<<grid, kBlock, smem, s>>>(A);
+                k_rows_lane<MODEL, 8><<<grid, kBlock, smem + kLaneSmem<MODEL, 8>, s>>>(A);
                 break;
             }
             return fail(FSGP_EINVAL, "lane kernel slice width");
@@ -1016,14 +1924,7 @@ int launch_rows_lane(const StepArgs &A, int swl, int grid, size_t smem, cudaStre
 
 template <int MODEL, int SWL>
 int occupancy_lane_w(size_t smem) {
-    // the staging area is static; per-lane counters (dynamic) may push the total past the
-    // default 48 KB window.  The attribute is process-wide and host threads of a batch set
-    // it concurrently, so it is always raised to the largest per-lane counter area any run
-    // uses (32 KB), never lowered to this run's need (set before any launch or capture).
-    cudaFuncSetAttribute(k_rows_lane<MODEL, SWL>, cudaFuncAttributeMaxDynamicSharedMemorySize, 32 * 1024);
-    int z = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&z, k_rows_lane<MODEL, SWL>, kBlock, smem);
-    return z;
+    return occupancy_one<k_rows_lane<MODEL, SWL>>(smem, kLaneSmem<MODEL, SWL>);
 }
 
 template <int MODEL>
@@ -1046,6 +1947,13 @@ int occupancy_lane(int swl, size_t smem) {
 template <int MODEL, int V, int TEAM>
 int launch_rows_vt(const StepArgs &A, const StepLaunch &L, cudaStream_t s) {
     Prof *pr = L.prof;
+    if (L.fused) {
+        if (pr) pr->start(PK_SMALL, s);
+        k_rows_fused<MODEL, V, TEAM><<<L.grid_mid + L.grid_small, kBlock, L.smem_lanes + FusedBytes<MODEL, V, TEAM>, s>>>(
+            A, L.grid_mid);
+        if (pr) pr->stop(s);
+        return FSGP_OK;
+    }
     if (L.have_hub) {
         if (pr) pr->start(PK_HUB, s);
         if (A.hub_sat) {
@@ -1060,17 +1968,17 @@ int launch_rows_vt(const StepArgs &A, const StepLaunch &L, cudaStream_t s) {
     }
     if (L.have_mid) {
         if (pr) pr->start(PK_MID, s);
-        k_rows<MODEL, V, TEAM, true><<<L.grid_mid, kBlock, L.smem_lanes, s>>>(A, 1);
+        k_rows<MODEL, V, TEAM, true><<<L.grid_mid, kBlock, L.smem_lanes + TileBytes<MODEL, V, TEAM, true, kSmallBits>, s>>>(A, 1);
         if (pr) pr->stop(s);
     }
     if (L.have_small) {
         if (pr) pr->start(PK_SMALL, s);
-        k_rows<MODEL, V, TEAM, false><<<L.grid_small, kBlock, L.smem_lanes, s>>>(A, 0);
+        k_rows<MODEL, V, TEAM, false><<<L.grid_small, kBlock, L.smem_lanes + TileBytes<MODEL, V, TEAM, false, kSmallBits>, s>>>(A, 0);
         if (pr) pr->stop(s);
     }
     if (L.have_small4) {
         if (pr) pr->start(PK_SMALL4, s);
-        k_rows<MODEL, V, TEAM, false, 4><<<L.grid_small4, kBlock, L.smem_lanes, s>>>(A, 3);
+        k_rows<MODEL, V, TEAM, false, 4><<<L.grid_small4, kBlock, L.smem_lanes + TileBytes<MODEL, V, TEAM, false, 4>, s>>>(A, 3);
         if (pr) pr->stop(s);
     }
     if (L.have_lane) {
@@ -1084,15 +1992,14 @@ int launch_rows_vt(const StepArgs &A, const StepLaunch &L, cudaStream_t s) {
 
 template <int MODEL, int V, int TEAM>
 void occupancy_vt(size_t smem, RowOccupancy *o) {
-    int a = 1, m = 1, b = 1, s4 = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&s4, k_rows<MODEL, V, TEAM, false, 4>, kBlock, smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_rows<MODEL, V, TEAM, false>, kBlock, smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&m, k_rows<MODEL, V, TEAM, true>, kBlock, smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_hub_chunks<MODEL, V, TEAM>, kBlock, 0);
-    o->small = a < 1 ? 1 : a;
-    o->mid = m < 1 ? 1 : m;
-    o->hub = b < 1 ? 1 : b;
-    o->small4 = s4 < 1 ? 1 : s4;
+    if (o->fused_only) {
+        o->fused = occupancy_one<k_rows_fused<MODEL, V, TEAM>>(smem, FusedBytes<MODEL, V, TEAM>);
+        return;
+    }
+    o->hub = occupancy_one<k_hub_chunks<MODEL, V, TEAM>>(0, 0);
+    o->small4 = occupancy_one<k_rows<MODEL, V, TEAM, false, 4>>(smem, TileBytes<MODEL, V, TEAM, false, 4>);
+    o->small = occupancy_one<k_rows<MODEL, V, TEAM, false>>(smem, TileBytes<MODEL, V, TEAM, false, kSmallBits>);
+    o->mid = occupancy_one<k_rows<MODEL, V, TEAM, true>>(smem, TileBytes<MODEL, V, TEAM, true, kSmallBits>);
 }
 
 #define FSGP_VT_SWITCH(MACRO)                          \
@@ -1150,46 +2057,47 @@ int occupancy_rows(int V, int TEAM, size_t smem, RowOccupancy *o) {
 #define FSGP_O(v_, t_) occupancy_vt<MODEL, v_, t_>(smem, o)
     FSGP_VT_SWITCH(FSGP_O)
 #undef FSGP_O
-    o->lane = occupancy_lane<MODEL>(o->swl, smem);
+    if (!o->fused_only) o->lane = occupancy_lane<MODEL>(o->swl, smem);
     return FSGP_OK;
 }
 
-// Cooperative launch of the persistent step loop (one word per thread, the 8-bit team
-// kernel: fused small graphs with in-degrees <= 255).  The grid is capped at the CTAs
-// that can be resident at once; *grid_out gets the grid used.  FSGP_EUNSUPPORTED: no
-// persistent kernel for this team width (the caller runs the launched loop instead).
+// Cooperative launch of the persistent step loop (one word per thread).  The grid is what
+// can be resident at once, at most the launched step's (grid_mid + grid_small CTAs), shared
+// out between the two row classes in the same proportion; *grid_out gets the grid used.
+// FSGP_EUNSUPPORTED: it does not fit (the caller runs the launched loop instead).
 template <int MODEL, int TEAM>
-int launch_persist_t(const StepArgs &A, const PersistArgs &Q, int grid, size_t smem, int sm_count,
+int launch_persist_t(const StepArgs &A, const PersistArgs &Q, int grid_mid, int grid_small, size_t smem, int sm_count,
                      cudaStream_t s, int *grid_out) {
-    // two teams per row split its arcs (measured on ER n = 10k, R = 64: 2 teams 0.73 ms
-    // per run, 4 teams 0.79 ms, 8 teams 0.94 ms)
-    constexpr int AG = TEAM >= 32 ? 1 : 2;
-    auto kern = k_rows_persist<MODEL, 1, TEAM, false, kSmallBits, AG>;
-    int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kBlock, smem);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor (persistent)");
-    if (per_sm < 1) return FSGP_EUNSUPPORTED;
-    // one work item (row slice) per team of AG teams: AG times the launched loop's CTAs
-    grid = std::max(1, std::min(grid * AG, per_sm * sm_count));
+    auto kern = k_rows_persist<MODEL, TEAM>;
+    const int per_sm = occupancy_one<k_rows_persist<MODEL, TEAM>>(smem, FusedBytes<MODEL, 1, TEAM>);
+    const int cap = per_sm * sm_count;
+    if (cap < 2) return FSGP_EUNSUPPORTED;
+    if (grid_mid + grid_small > cap) {
+        const int m = grid_mid ? std::max(1, (int)((int64_t)grid_mid * cap / (grid_mid + grid_small))) : 0;
+        grid_mid = grid_small ? std::min(m, cap - 1) : cap;
+        grid_small = cap - grid_mid;
+    }
     StepArgs a = A;
     PersistArgs q = Q;
+    q.warp_ctas = grid_mid;
     void *args[] = {&a, &q};
-    e = cudaLaunchCooperativeKernel((const void *)kern, dim3(grid), dim3(kBlock), args, smem, s);
+    const cudaError_t e = cudaLaunchCooperativeKernel((const void *)kern, dim3(grid_mid + grid_small), dim3(kBlock), args,
+                                                      smem + FusedBytes<MODEL, 1, TEAM>, s);
     if (e != cudaSuccess) return cuda_fail(e, "cudaLaunchCooperativeKernel (persistent step loop)");
-    *grid_out = grid;
+    *grid_out = grid_mid + grid_small;
     return FSGP_OK;
 }
 
 template <int MODEL>
-int launch_persist(const StepArgs &A, const PersistArgs &Q, int TEAM, int grid, size_t smem, int sm_count,
+int launch_persist(const StepArgs &A, const PersistArgs &Q, int TEAM, int grid_mid, int grid_small, size_t smem, int sm_count,
                    cudaStream_t s, int *grid_out) {
     switch (TEAM) {
-        case 1: return launch_persist_t<MODEL, 1>(A, Q, grid, smem, sm_count, s, grid_out);
-        case 2: return launch_persist_t<MODEL, 2>(A, Q, grid, smem, sm_count, s, grid_out);
-        case 4: return launch_persist_t<MODEL, 4>(A, Q, grid, smem, sm_count, s, grid_out);
-        case 8: return launch_persist_t<MODEL, 8>(A, Q, grid, smem, sm_count, s, grid_out);
-        case 16: return launch_persist_t<MODEL, 16>(A, Q, grid, smem, sm_count, s, grid_out);
-        case 32: return launch_persist_t<MODEL, 32>(A, Q, grid, smem, sm_count, s, grid_out);
+        case 1: return launch_persist_t<MODEL, 1>(A, Q, grid_mid, grid_small, smem, sm_count, s, grid_out);
+        case 2: return launch_persist_t<MODEL, 2>(A, Q, grid_mid, grid_small, smem, sm_count, s, grid_out);
+        case 4: return launch_persist_t<MODEL, 4>(A, Q, grid_mid, grid_small, smem, sm_count, s, grid_out);
+        case 8: return launch_persist_t<MODEL, 8>(A, Q, grid_mid, grid_small, smem, sm_count, s, grid_out);
+        case 16: return launch_persist_t<MODEL, 16>(A, Q, grid_mid, grid_small, smem, sm_count, s, grid_out);
+        case 32: return launch_persist_t<MODEL, 32>(A, Q, grid_mid, grid_small, smem, sm_count, s, grid_out);
         default: return FSGP_EUNSUPPORTED;
     }
 }

@@ -377,9 +377,15 @@ __global__ void k_row_degrees(const int32_t *__restrict__ row_ptr, const int32_t
 }
 
 // Hub chunk table for (hub bucket, chunk): hub rows are rows_sorted[0 .. n_hubs).
-static int ensure_hub_table(fsgp_graph *g, int hub_min_deg, int chunk, cudaStream_t s) {
-    HubTable &H = g->hub;
-    if (H.min_deg == hub_min_deg && H.chunk == chunk) return FSGP_OK;
+static int ensure_hub_table(fsgp_graph *g, int hub_min_deg, int chunk, cudaStream_t s, const HubTable **out) {
+    for (HubTable &T : g->hubs) {
+        *out = &T;
+        if (T.min_deg == hub_min_deg && T.chunk == chunk) return FSGP_OK;
+    }
+    // two tables are kept (models with different chunks may alternate); the older one goes
+    std::swap(g->hubs[0], g->hubs[1]);
+    HubTable &H = g->hubs[1];
+    *out = &H;
     const int bh = bitlen(hub_min_deg);   // bucket of hub_min_deg (a power of two)
     const int32_t n_hubs = bh >= 1 ? g->cls.bucket_start[bh - 1] : g->n;
     cudaFree(H.d_chunk_base);
@@ -459,18 +465,18 @@ static int occupancy_model(int model, int V, int TEAM, size_t smem, RowOccupancy
     }
 }
 
-static int launch_persist_model(int model, const StepArgs &A, const PersistArgs &Q, int TEAM, int grid,
-                                size_t smem, int sm_count, cudaStream_t s, int *grid_out) {
+static int launch_persist_model(int model, const StepArgs &A, const PersistArgs &Q, int TEAM, int grid_mid,
+                                int grid_small, size_t smem, int sm_count, cudaStream_t s, int *grid_out) {
     switch (model) {
-        case FSGP_SIR: return launch_persist<FSGP_SIR>(A, Q, TEAM, grid, smem, sm_count, s, grid_out);
-        case FSGP_SIS: return launch_persist<FSGP_SIS>(A, Q, TEAM, grid, smem, sm_count, s, grid_out);
-        case FSGP_IC: return launch_persist<FSGP_IC>(A, Q, TEAM, grid, smem, sm_count, s, grid_out);
-        case FSGP_LT: return launch_persist<FSGP_LT>(A, Q, TEAM, grid, smem, sm_count, s, grid_out);
-        case FSGP_SEIR: return launch_persist<FSGP_SEIR>(A, Q, TEAM, grid, smem, sm_count, s, grid_out);
-        case FSGP_SEIS: return launch_persist<FSGP_SEIS>(A, Q, TEAM, grid, smem, sm_count, s, grid_out);
-        case FSGP_SWIR: return launch_persist<FSGP_SWIR>(A, Q, TEAM, grid, smem, sm_count, s, grid_out);
-        case kSirW: return launch_persist<kSirW>(A, Q, TEAM, grid, smem, sm_count, s, grid_out);
-        case kSisW: return launch_persist<kSisW>(A, Q, TEAM, grid, smem, sm_count, s, grid_out);
+        case FSGP_SIR: return launch_persist<FSGP_SIR>(A, Q, TEAM, grid_mid, grid_small, smem, sm_count, s, grid_out);
+        case FSGP_SIS: return launch_persist<FSGP_SIS>(A, Q, TEAM, grid_mid, grid_small, smem, sm_count, s, grid_out);
+        case FSGP_IC: return launch_persist<FSGP_IC>(A, Q, TEAM, grid_mid, grid_small, smem, sm_count, s, grid_out);
+        case FSGP_LT: return launch_persist<FSGP_LT>(A, Q, TEAM, grid_mid, grid_small, smem, sm_count, s, grid_out);
+        case FSGP_SEIR: return launch_persist<FSGP_SEIR>(A, Q, TEAM, grid_mid, grid_small, smem, sm_count, s, grid_out);
+        case FSGP_SEIS: return launch_persist<FSGP_SEIS>(A, Q, TEAM, grid_mid, grid_small, smem, sm_count, s, grid_out);
+        case FSGP_SWIR: return launch_persist<FSGP_SWIR>(A, Q, TEAM, grid_mid, grid_small, smem, sm_count, s, grid_out);
+        case kSirW: return launch_persist<kSirW>(A, Q, TEAM, grid_mid, grid_small, smem, sm_count, s, grid_out);
+        case kSisW: return launch_persist<kSisW>(A, Q, TEAM, grid_mid, grid_small, smem, sm_count, s, grid_out);
         default: return fail(FSGP_EINVAL, "model without row kernels");
     }
 }
@@ -480,7 +486,7 @@ static int launch_persist_model(int model, const StepArgs &A, const PersistArgs 
 // takes microseconds.
 constexpr long long kPersistSpinCycles = 2000000000ll;
 
-constexpr int32_t kSmallMaxFused = 255;   // in-degree bound of the 8-bit team kernel
+constexpr int32_t kHubMinDeg = 8192;      // rows split over CTAs by default
 
 static int words_per_set(int R) {
     const int W = (R + 31) / 32;
@@ -518,17 +524,35 @@ static int run_wave(fsgp_graph *g, int model, int ic_mode, int weighted, const S
     const int C = n_compartments(model);
     const int Wn = S * Ws;
     const int pd = Ws << __builtin_ctz((unsigned)S);   // largest power of two dividing Wn
-    // Small graphs: every row in one launch (team or warp per row), dense steps
-    // only, so that a step is two launches; their steps are bound by launch latency.
-    // (automatic only when no degree-class or frontier option is given)
+    // Small graphs: two degree classes (a team or a warp per row) in one launch, dense steps
+    // only, so that a step is two launches; their steps are bound by launch latency and by
+    // the longest chain of a row.  Automatic when no degree-class or frontier option is
+    // given, up to 2^20 state words per plane, and up to 2^22 when no row is long enough to
+    // outlast the rest in one warp (below the hub bound; against the degree-class launches
+    // with frontier steps, 14 graphs of 1.0M to 4.2M words: 1.0 to 1.45 times faster, R-MAT
+    // graphs with longer rows 0.87).  Not above 2^20: SWIR, which decides its words in place
+    // and wants the degree classes' own kernels (0.4 to 0.8 times), and the cascades, which
+    // want their frontier (LT, ER n = 328k, two sets of R = 104: 0.61 times).
     const bool auto_classes = opt.small_max_deg == 0 && opt.hub_min_deg == 0 && opt.hub_chunk == 0 &&
                               opt.sparse_frac == 0.0;
-    const bool fuse = g->max_deg < 65536 &&
-                      (opt.fuse_rows > 0 ||
-                       (opt.fuse_rows == 0 && auto_classes && (int64_t)n * Wn <= ((int64_t)1 << 20)));
-    // Words per thread: 2 measured best on GB300 for large graphs; small graphs, bound by
-    // the longest per-thread chain of dependent instructions, take one word per thread.
-    int V = opt.vector_words ? opt.vector_words : (fuse ? 1 : 2);
+    const int64_t words = (int64_t)n * Wn;
+    const bool cascade = model == FSGP_IC || model == FSGP_LT;
+    const bool small = words <= ((int64_t)1 << 20) ||
+                       (words <= ((int64_t)1 << 22) && g->max_deg < kHubMinDeg && model != FSGP_SWIR && !cascade);
+    const bool fuse = g->max_deg < 65536 && (opt.fuse_rows > 0 || (opt.fuse_rows == 0 && auto_classes && small));
+    // Words per thread (w: words a team covers with one word per thread).  Large graphs: 2,
+    // and 4 for rows of 16 words and more, whose teams are then at most 8 threads wide and
+    // spend less per arc (BA n = 1M, IC, R = 1024: 50.8 against 39.0 ms; R-MAT, SIS, R = 256:
+    // 178 against 179 ms).  Small graphs whose rows all get a warp at once are bound by the
+    // longest chain and take 1; the others as many as keep a team within 8 threads (BA
+    // n = 18k, SIS, R = 1010: 2.96 ms with 1, 1.38 with 2, 1.48 with 4; BA n = 20k, SIR,
+    // R = 1000: 6.4, 4.7, 4.4; BA n = 250k, SEIR, R = 100: 8.7, 9.0, 13.5).
+    const int w = std::min(32, pd);
+    const bool one_round = (int64_t)n * (Wn / w) <= (int64_t)g->sm_count * 24;
+    int V = opt.vector_words ? opt.vector_words
+            : !fuse          ? (w >= 16 ? 4 : 2)
+            : one_round      ? 1
+                             : (w >= 32 ? 4 : (w >= 16 ? 2 : 1));
     if (V != 1 && V != 2 && V != 4) return fail(FSGP_EINVAL, "vector_words must be 1, 2 or 4");
     if (V > pd) V = pd;
     const int SW = std::min(32 * V, pd);
@@ -549,8 +573,11 @@ static int run_wave(fsgp_graph *g, int model, int ic_mode, int weighted, const S
         want_steps |= sets[i]->steps_run != nullptr;
     }
     // degree classes
-    int small_max = opt.small_max_deg > 0 ? opt.small_max_deg : 255;
-    int hub_min = fuse ? 65536 : (opt.hub_min_deg > 0 ? opt.hub_min_deg : 8192);
+    // (cascades run on frontier lists, whose few rows want a warp each: BA n = 1M, IC,
+    // R = 1024: 50.8 ms with 255, 44.7 with 63; LT, n = 700k: 18.0 and 15.9; where the steps
+    // are dense it costs a little: R-MAT n = 2M, IC, R = 256: 93.9 and 98.9)
+    int small_max = opt.small_max_deg > 0 ? opt.small_max_deg : (cascade ? 63 : 255);
+    int hub_min = fuse ? 65536 : (opt.hub_min_deg > 0 ? opt.hub_min_deg : kHubMinDeg);
     int bs = bitlen(small_max + 1) - 1;              // small: d <= 2^bs - 1
     if (bs < 0) bs = 0;
     if (bs > kSmallBits) bs = kSmallBits;             // small rows count on 8-bit slices
@@ -560,15 +587,18 @@ static int run_wave(fsgp_graph *g, int model, int ic_mode, int weighted, const S
     if (bh > 32) bh = 32;
     small_max = (1 << bs) - 1;
     hub_min = 1 << (bh - 1);
-    const int chunk = opt.hub_chunk > 0 ? std::min(opt.hub_chunk, 65535) : 8192;
+    // (IC draws per arc in the gathering thread: shorter chunks, 34.4 against 31.0 ms on the
+    // BA n = 1M run; the count models lose 1 to 2% with them)
+    const int chunk = opt.hub_chunk > 0 ? std::min(opt.hub_chunk, 65535) : (model == FSGP_IC ? 2048 : 8192);
     const double sparse_frac = fuse ? -1.0 : (opt.sparse_frac == 0.0 ? 0.05 : opt.sparse_frac);
     const unsigned long long sparse_limit =
         sparse_frac < 0.0 ? 0ull : (unsigned long long)(sparse_frac * (double)g->nnz);
     const bool allow_sparse = sparse_frac >= 0.0;
 
-    int rc = ensure_hub_table(g, hub_min, chunk, s);
+    const HubTable *hub = nullptr;
+    int rc = ensure_hub_table(g, hub_min, chunk, s, &hub);
     if (rc) return rc;
-    const int32_t n_hubs = g->hub.n_hubs;
+    const int32_t n_hubs = hub->n_hubs;
     const int32_t start_mid = bh >= 1 ? g->cls.bucket_start[bh - 1] : n;
     const int32_t start_small = g->cls.bucket_start[bs];
     const int32_t n_mid = start_small - start_mid;
@@ -706,6 +736,7 @@ static int run_wave(fsgp_graph *g, int model, int ic_mode, int weighted, const S
     if (smem_lanes > 32 * 1024) return fail(FSGP_EINVAL, "per-lane counters exceed shared memory");
     RowOccupancy occ{};
     occ.swl = lane_swl;
+    occ.fused_only = fuse;
     rc = occupancy_model(kmodel, V, TEAM, smem_lanes, &occ);
     if (rc) return rc;
     Prof prof;
@@ -716,37 +747,46 @@ static int run_wave(fsgp_graph *g, int model, int ic_mode, int weighted, const S
     L.V = V;
     L.TEAM = TEAM;
     L.smem_lanes = smem_lanes;
+    // Fused rows: the rows of 2^b in-arcs and more get a warp each (16-bit counters), the
+    // others a team (8-bit counters).  A small graph's step lasts as long as its longest
+    // chain of gathers, so b is the smallest bound for which the warp rows take at most half
+    // of the warps that fit at once (60 graphs of 8k to 1M words: 1.16 times faster on average
+    // than all of them, as fast as a quarter), and at most 8.
+    const int64_t fit_warps = (int64_t)g->sm_count * std::max(occ.fused, 1) * (kBlock / 32);
+    int split_b = 0;
+    while (fuse && split_b < kSmallBits && 2 * (int64_t)g->cls.bucket_start[split_b] * nslices > fit_warps) ++split_b;
+    const int32_t fuse_split = !fuse ? 0 : (split_b == 0 ? n : g->cls.bucket_start[split_b]);
+    // All T steps in one cooperative launch (no per-lane counts).  (27 graphs of 8k to 200k
+    // words: 1.2 times faster than a launch per step on average; 16 of 200k to 1M words: 0.9
+    // to 1.26.)
+    const bool persist = fuse && opt.persistent >= 0 && !want_lanes && !profiling && V == 1 && T >= 1 &&
+                         (words <= ((int64_t)1 << 20) || opt.persistent > 0);
     // the 16..small_max kernel also takes every small row of a frontier step
-    // fused rows: the team-per-row kernel (8-bit counters) when every in-degree is below
-    // 256, else the warp-per-row kernel (16-bit counters)
-    const bool fuse_team = fuse && g->max_deg <= kSmallMaxFused;
-    // all T steps in one cooperative launch (fused team rows, no per-lane counts)
-    const bool persist = fuse_team && opt.persistent >= 0 && !want_lanes && !profiling && V == 1 && T >= 1 &&
-                         n > 0;
-    L.have_small = fuse ? (fuse_team && n > 0) : n_small_all > 0;
-    L.have_small4 = n_small4 > 0 && !fuse;
-    L.have_lane = (n_lane > 0 || n_d0 > 0) && !fuse;
-    L.swl = occ.swl;
-    L.have_mid = fuse ? (!fuse_team && n > 0) : n_mid > 0;
-    L.have_hub = n_hubs > 0;
+    L.fused = fuse;
+    L.have_small = !fuse && n_small_all > 0;
+    L.have_small4 = !fuse && n_small4 > 0;
+    L.have_lane = !fuse && (n_lane > 0 || n_d0 > 0);
+    L.swl = fuse ? 1 : occ.swl;
+    L.have_mid = !fuse && n_mid > 0;
+    L.have_hub = !fuse && n_hubs > 0;
     L.prof = profiling ? &prof : nullptr;
-    const int64_t items_small = (int64_t)(fuse_team ? n : n_small_all) * nslices;
-    const int64_t items_mid = (int64_t)(fuse ? n : n_mid) * nslices;
-    const int64_t items_lane = (int64_t)(n_lane + n_d0) * (Wn / occ.swl);
     const int per_block_small = (kBlock / 32) * (32 / TEAM);
-    auto grid_for_items = [&](int per_sm, int64_t items) {
-        return (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)g->sm_count * per_sm,
-                                                           (items + per_block_small - 1) / per_block_small));
+    auto grid_for = [&](int64_t cap, int64_t items, int per_block) {
+        return (int)std::min<int64_t>(cap, (items + per_block - 1) / per_block);
     };
-    L.grid_small = grid_for_items(occ.small, items_small);
-    L.grid_small4 = grid_for_items(occ.small4, (int64_t)n_small4 * nslices);
-    L.grid_lane = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)g->sm_count * occ.lane,
-                                                              (items_lane + kBlock - 1) / kBlock));
-    L.grid_mid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)g->sm_count * occ.mid,
-                                                             (items_mid + (kBlock / 32) - 1) / (kBlock / 32)));
-    L.grid_hub = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)g->sm_count * occ.hub,
-                                                             g->hub.n_chunks * nslices));
-    L.grid_fin = (int)std::max<int64_t>(1, ((int64_t)n_hubs + (kBlock / 32) - 1) / (kBlock / 32));
+    const int64_t sms = g->sm_count;
+    if (fuse) {
+        L.grid_mid = grid_for(sms * occ.fused, (int64_t)fuse_split * nslices, kBlock / 32);
+        L.grid_small = grid_for(std::max<int64_t>(sms * occ.fused - L.grid_mid, 1), (int64_t)(n - fuse_split) * nslices,
+                                per_block_small);
+    } else {
+        L.grid_small = std::max(1, grid_for(sms * occ.small, (int64_t)n_small_all * nslices, per_block_small));
+        L.grid_small4 = std::max(1, grid_for(sms * occ.small4, (int64_t)n_small4 * nslices, per_block_small));
+        L.grid_lane = std::max(1, grid_for(sms * occ.lane, (int64_t)(n_lane + n_d0) * (Wn / occ.swl), kBlock));
+        L.grid_mid = std::max(1, grid_for(sms * occ.mid, (int64_t)n_mid * nslices, kBlock / 32));
+        L.grid_hub = std::max(1, grid_for(sms * occ.hub, hub->n_chunks * nslices, 1));
+        L.grid_fin = std::max(1, grid_for(INT32_MAX, n_hubs, kBlock / 32));
+    }
 
     const int grid_mark = g->sm_count * 8;
     const int grid_scan = grid_cap((int64_t)n, kBlock, g->sm_count, 8);
@@ -772,26 +812,27 @@ static int run_wave(fsgp_graph *g, int model, int ic_mode, int weighted, const S
     A.plane_words = (size_t)n * Wn;
     A.sp = d_sp;
     A.ic_mode = ic_mode;
+    for (const SetParams &p : hp) A.fixed_on |= (p.g_rec ? 1 : 0) | (p.a_lat ? 2 : 0);
     A.ctl = ctl;
     A.lane_cnt = want_lanes ? (int32_t *)(ws + off[O_LANES]) : nullptr;
     A.np = P;
-    A.r_small = fuse_team ? 0 : start_small;
-    A.n_small = fuse_team ? n : n_small;
+    A.r_small = fuse ? fuse_split : start_small;
+    A.n_small = fuse ? n - fuse_split : n_small;
     A.r_small4 = std::max(start_small4, start_small);
     A.n_small4 = n_small4;
     A.r_lane = start_lane;
     A.n_lane = n_lane;
     A.r_mid = fuse ? 0 : start_mid;
-    A.n_mid = fuse ? n : n_mid;
+    A.n_mid = fuse ? fuse_split : n_mid;
     A.r_d0 = d0_start;
     A.lane_tab = (g->lane_tab && n_lane > 0) ? g->lane_tab + (start_lane - g->lane_start) : nullptr;
     A.d0_list = (int32_t *)(ws + off[O_D0]);
     A.cand_small = (int32_t *)(ws + off[O_CSMALL]);
     A.cand_mid = (int32_t *)(ws + off[O_CMID]);
     A.bitmap = (uint32_t *)(ws + off[O_BITMAP]);
-    A.hub_chunk_base = g->hub.d_chunk_base;
+    A.hub_chunk_base = hub->d_chunk_base;
     A.n_hubs = n_hubs;
-    A.n_hub_chunks = g->hub.n_chunks;
+    A.n_hub_chunks = hub->n_chunks;
     A.hub_chunk = chunk;
     A.hub_scratch = hub_scratch;
     A.hub_sat = (hub_sat && n_hubs > 0) ? (uint32_t *)(ws + off[O_HUBSAT]) : nullptr;
@@ -898,7 +939,7 @@ static int run_wave(fsgp_graph *g, int model, int ic_mode, int weighted, const S
         Q.t0 = (uint32_t)opt.t0;
         Q.spin_limit = kPersistSpinCycles;
         int grid_used = 0;
-        rc = launch_persist_model(kmodel, A, Q, TEAM, L.grid_small, L.smem_lanes, g->sm_count, s, &grid_used);
+        rc = launch_persist_model(kmodel, A, Q, TEAM, L.grid_mid, L.grid_small, L.smem_lanes, g->sm_count, s, &grid_used);
         if (rc == FSGP_OK) {
             const int width = S * kPC;
             k_pc_prefix<<<(width + 255) / 256, 256, 0, s>>>(pc, (int)T, width);
@@ -928,8 +969,8 @@ static int run_wave(fsgp_graph *g, int model, int ic_mode, int weighted, const S
         }
         rc = launch_rows_model(kmodel, A, L, s);
         if (rc) return rc;
-        launches += 1 + (allow_sparse ? 1 : 0) + (L.have_hub ? (A.hub_sat ? 3 : 2) : 0) + (L.have_mid ? 1 : 0) +
-                    (L.have_small ? 1 : 0) + (L.have_small4 ? 1 : 0) + (L.have_lane ? 1 : 0);
+        launches += 1 + (allow_sparse ? 1 : 0) + (L.fused ? 1 : 0) + (L.have_hub ? (A.hub_sat ? 3 : 2) : 0) +
+                    (L.have_mid ? 1 : 0) + (L.have_small ? 1 : 0) + (L.have_small4 ? 1 : 0) + (L.have_lane ? 1 : 0);
     }
     FSGP_CUDA(cudaGetLastError());
     if (profiling) prof.start(PK_RESULTS, s);

@@ -56,6 +56,7 @@ struct PersistArgs {
     int32_t T;
     uint32_t t0;
     long long spin_limit;          // SM clock cycles one barrier wait may last
+    int32_t warp_ctas;             // CTAs on the warp-per-row rows (the first ones)
 };
 
 // Per-set parameters (device array, one entry per set of the launch).
@@ -108,6 +109,8 @@ struct StepArgs {
     // model parameters
     const SetParams *__restrict__ sp;   // [S]
     int32_t ic_mode;
+    int32_t fixed_on;      // bit 0: some set recovers (gamma > 0), bit 1: some set's exposed
+                           // lanes turn infectious (alpha > 0)
     uint32_t t;            // absolute step index of the step being computed
     int32_t k;             // relative step index (1..T)
     // control and accumulators
@@ -139,14 +142,27 @@ struct StepArgs {
     const float *__restrict__ arc_w; // weighted graphs: [nnz] weights in the caller's arc order
 };
 
-// Weighted graphs: transmission threshold of the arc at caller position epos for a lane
-// of set s.  p = beta * w_e in single precision; 0 if p <= 0, 2^32 (certain) if p >= 1,
-// else round(p * 2^32) (the scaling by 2^32 is exact).
-__device__ __forceinline__ uint64_t arc_threshold(const StepArgs &A, int s, int64_t epos) {
-    const float p = __fmul_rn(__ldg(&A.sp[s].beta_f), __ldg(A.arc_w + epos));
+// Weighted graphs: transmission threshold of an arc.  p = beta * w_e in single precision;
+// 0 if p <= 0, 2^32 (certain) if p >= 1, else round(p * 2^32) (the scaling by 2^32 is
+// exact).
+__device__ __forceinline__ uint64_t arc_thr(float beta, float w) {
+    const float p = __fmul_rn(beta, w);
     if (!(p > 0.0f)) return 0ull;
     if (p >= 1.0f) return TWO32;
     return (uint64_t)__float2ull_rn(__fmul_rn(p, 4294967296.0f));
+}
+
+// ... of the arc at caller position epos for a lane of set s.
+__device__ __forceinline__ uint64_t arc_threshold(const StepArgs &A, int s, int64_t epos) {
+    return arc_thr(__ldg(&A.sp[s].beta_f), __ldg(A.arc_w + epos));
+}
+
+// Row of a work item (an item is one of the row's slices).  Items mostly number less than
+// 2^32, and the 64-bit division costs several times the 32-bit one.
+__device__ __forceinline__ int64_t div_slices(int64_t item, int nslices, int64_t nitems) {
+    if (nslices == 1) return item;
+    if (nitems <= 0xffffffffll) return (int64_t)((uint32_t)item / (uint32_t)nslices);
+    return item / nslices;
 }
 
 // Node (Philox subject) of new row i, and new row of node v.
@@ -192,33 +208,57 @@ __device__ __forceinline__ WordCtx word_ctx(const StepArgs &A, int w) {
 
 // ------------------------------------------------------------ bit-sliced counters
 
-// c += x0 + x1 + x2 + x3 (bit-sliced, 32 lanes per word).  Carry-save compression of
-// the four inputs to three bit-planes, then a ripple that stops at the first zero carry.
-template <int B>
-__device__ __forceinline__ void add4(uint32_t (&c)[B], uint32_t x0, uint32_t x1, uint32_t x2,
-                                     uint32_t x3) {
-    const uint32_t sA = x0 ^ x1 ^ x2;
-    const uint32_t cA = (x0 & x1) | (x2 & (x0 ^ x1));
-    const uint32_t s0 = sA ^ x3;
-    const uint32_t cB = sA & x3;
-    const uint32_t s1 = cA ^ cB;
-    const uint32_t s2 = cA & cB;
-    uint32_t carry = c[0] & s0;
-    c[0] ^= s0;
-    uint32_t t = c[1];
-    c[1] = t ^ s1 ^ carry;
-    if constexpr (B == 2) return;   // counts below 4 (rows with at most 3 in-arcs)
-    carry = (t & s1) | (carry & (t ^ s1));
-    t = c[B > 2 ? 2 : 1];
-    c[B > 2 ? 2 : 1] = t ^ s2 ^ carry;
-    carry = (t & s2) | (carry & (t ^ s2));
+// Full adder on bit planes: a += x + y modulo 2, returns the carry (two LOP3).
+__device__ __forceinline__ uint32_t full_add(uint32_t &a, uint32_t x, uint32_t y) {
+    const uint32_t carry = (a & x) | (a & y) | (x & y);
+    a ^= x ^ y;
+    return carry;
+}
+
+// c += carry * 2^FROM.  Straight-line up to plane 7, since in a warp some word's carry
+// always runs; the planes above are entered once in 256 counts.
+template <int FROM, int B>
+__device__ __forceinline__ void ripple(uint32_t (&c)[B], uint32_t carry) {
 #pragma unroll
-    for (int b = 3; b < B; ++b) {
-        if (!carry) break;
+    for (int b = FROM; b < (B < 8 ? B : 8); ++b) {
         const uint32_t nc = c[b] & carry;
         c[b] ^= carry;
         carry = nc;
     }
+    if constexpr (B > 8) {
+        if (carry) {
+#pragma unroll
+            for (int b = 8; b < B; ++b) {
+                const uint32_t nc = c[b] & carry;
+                c[b] ^= carry;
+                carry = nc;
+            }
+        }
+    }
+}
+
+// c += x0 + x1 + x2 + x3 (bit-sliced, 32 lanes per word): carry-save adders on the two
+// lowest planes, one ripple from plane 2.
+template <int B>
+__device__ __forceinline__ void add4(uint32_t (&c)[B], uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3) {
+    const uint32_t a0 = full_add(c[0], x0, x1), a1 = full_add(c[0], x2, x3);
+    const uint32_t f = full_add(c[1], a0, a1);
+    ripple<2>(c, f);
+}
+
+// The same with eight words: one ripple, from plane 3, for all eight (3 logic operations
+// per word and arc at 8 planes against 4.5 with add4).
+template <int B>
+__device__ __forceinline__ void add8(uint32_t (&c)[B], uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3, uint32_t x4,
+                                     uint32_t x5, uint32_t x6, uint32_t x7) {
+    static_assert(B >= 4, "eight words need four planes");
+    uint32_t a0 = full_add(c[0], x0, x1), a1 = full_add(c[0], x2, x3);
+    const uint32_t f0 = full_add(c[1], a0, a1);
+    a0 = full_add(c[0], x4, x5);
+    a1 = full_add(c[0], x6, x7);
+    const uint32_t f1 = full_add(c[1], a0, a1);
+    const uint32_t e = full_add(c[2], f0, f1);
+    ripple<3>(c, e);
 }
 
 // c += d (both bit-sliced, no overflow by construction)
@@ -576,6 +616,30 @@ __device__ __forceinline__ void set_acc_add(unsigned long long *s_pc, int s, lon
     if (d2) atomicAdd(&s_pc[kPC * s + 2], (unsigned long long)d2);
 }
 
+// The same for a whole warp (s < 0: nothing): one addition per set when its lanes hold the
+// same set, as they do unless several narrow sets run side by side.  A 64-bit shared
+// atomic is a compare-and-swap loop, and 256 threads adding to one counter at the end of
+// each CTA retried it 1.2 million times per launch (R-MAT n = 2M, rows of 16 to 255 arcs);
+// on a small graph that was most of a step's tail.
+__device__ __forceinline__ void set_acc_add_warp(unsigned long long *s_pc, int s, long long d0, long long d1,
+                                                 long long d2) {
+    __syncwarp();
+    const int s0 = __reduce_max_sync(0xffffffffu, s);
+    if (!__all_sync(0xffffffffu, s < 0 || s == s0)) {
+        if (s >= 0) set_acc_add(s_pc, s, d0, d1, d2);
+        return;
+    }
+    if (s0 < 0) return;
+    if (s < 0) d0 = d1 = d2 = 0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        d0 += __shfl_xor_sync(0xffffffffu, d0, o);
+        d1 += __shfl_xor_sync(0xffffffffu, d1, o);
+        d2 += __shfl_xor_sync(0xffffffffu, d2, o);
+    }
+    if ((threadIdx.x & 31) == 0) set_acc_add(s_pc, s0, d0, d1, d2);
+}
+
 // after a __syncthreads of the caller
 __device__ __forceinline__ void set_acc_flush(const StepArgs &A, const unsigned long long *s_pc) {
     for (int i = threadIdx.x; i < kPC * A.S; i += blockDim.x)
@@ -692,6 +756,8 @@ struct StepLaunch {
     int swl;               // words per thread of the one-thread-per-row kernel
     size_t smem_lanes;     // dynamic shared memory for per-lane counters (0 = off)
     bool have_small, have_mid, have_hub, have_small4, have_lane;
+    bool fused;            // both classes of a small graph in one launch: grid_mid CTAs on
+                           // the warp rows, grid_small on the team rows (either may be 0)
     struct Prof *prof;     // host-side event recorder, or null
 };
 
@@ -734,15 +800,16 @@ int run_sets(fsgp_graph *g, int model, int ic_mode, int weighted, const SetSpec 
              const fsgp_options &opt, cudaStream_t s);
 
 template <int MODEL>
-int launch_persist(const StepArgs &A, const PersistArgs &Q, int TEAM, int grid, size_t smem, int sm_count,
+int launch_persist(const StepArgs &A, const PersistArgs &Q, int TEAM, int grid_mid, int grid_small, size_t smem, int sm_count,
                    cudaStream_t s, int *grid_out);
 
 // Defined in rows.cuh, instantiated once per model (model_*.cu).
 template <int MODEL>
 int launch_rows(const StepArgs &A, const StepLaunch &L, cudaStream_t s);
 struct RowOccupancy {
-    int small, small4, lane, mid, hub;   // resident CTAs per SM of each row kernel
+    int small, small4, lane, mid, hub, fused;   // resident CTAs per SM of each row kernel
     int swl;                             // in: slice width of the lane kernel
+    bool fused_only;                     // in: only the fused kernel is wanted
 };
 template <int MODEL>
 int occupancy_rows(int V, int TEAM, size_t smem, RowOccupancy *o);
