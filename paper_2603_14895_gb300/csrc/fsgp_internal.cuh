@@ -177,6 +177,7 @@ struct fsgp_graph {
                                     // row's arcs in their original order)
     int32_t *arc0 = nullptr;        // [n] position in col of the first arc of new row i
                                     // (IC draws are keyed by the original arc position)
+    int32_t *odeg = nullptr;        // [n] out-degree of new row i
     int4 *lane_tab = nullptr;       // new rows with 1..3 in-arcs (from bucket 2 to the
                                     // start of bucket 0): {node, src0, src1, src2}, sources
                                     // as new ids, -1 = none

@@ -249,16 +249,18 @@ int exclusive_scan_i32(const int32_t *in, int64_t n, int32_t *out, int64_t *tile
 }
 
 // Relabelling (new id i = position of node rows_sorted[i]): inverse map, per-row in-degree
-// in new order (scanned into rp2 afterwards) and the original position of each row's first
-// arc.
+// in new order (scanned into rp2 afterwards), the original position of each row's first arc
+// and its out-degree.
 __global__ void k_relabel_rows(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ rows,
-                               int32_t n, int32_t *pos, int32_t *deg2, int32_t *arc0) {
+                               const int32_t *__restrict__ out_ptr, int32_t n, int32_t *pos, int32_t *deg2,
+                               int32_t *arc0, int32_t *odeg) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int32_t v = rows[i];
         pos[v] = (int32_t)i;
         const int32_t b = row_ptr[v];
         deg2[i] = row_ptr[v + 1] - b;
         arc0[i] = b;
+        odeg[i] = out_ptr[v + 1] - out_ptr[v];
     }
 }
 
@@ -298,6 +300,7 @@ static void release(fsgp_graph *g) {
     cudaFree(g->rp2);
     cudaFree(g->col2);
     cudaFree(g->arc0);
+    cudaFree(g->odeg);
     cudaFree(g->lane_tab);
     cudaFree(g->arc_w);
     for (HubTable &T : g->hubs) cudaFree(T.d_chunk_base);
@@ -485,18 +488,19 @@ extern "C" int fsgp_graph_create(const int32_t *row_ptr, const int32_t *col_idx,
             (e = cudaMalloc(&g->rp2, rp_bytes)) != cudaSuccess ||
             (e = cudaMalloc(&g->col2, col_bytes)) != cudaSuccess ||
             (e = cudaMalloc(&g->arc0, sizeof(int32_t) * (size_t)n)) != cudaSuccess ||
+            (e = cudaMalloc(&g->odeg, sizeof(int32_t) * (size_t)n)) != cudaSuccess ||
             (n_lane > 0 && (e = cudaMalloc(&g->lane_tab, sizeof(int4) * (size_t)n_lane)) != cudaSuccess)) {
             rc = cuda_fail(e, "cudaMalloc (relabelled graph)");
             break;
         }
-        g->device_bytes += 2 * sizeof(int32_t) * (size_t)n + rp_bytes + col_bytes + sizeof(int4) * (size_t)n_lane;
+        g->device_bytes += 3 * sizeof(int32_t) * (size_t)n + rp_bytes + col_bytes + sizeof(int4) * (size_t)n_lane;
         // d_cnt (n+1 entries) holds the degrees in new order; entry n = 0 ends the scan
         if ((e = cudaMemsetAsync(d_cnt + n, 0, sizeof(int32_t), s)) != cudaSuccess) {
             rc = cuda_fail(e, "cudaMemsetAsync");
             break;
         }
-        k_relabel_rows<<<grid_for(n, 256, g->sm_count), 256, 0, s>>>(g->row_ptr, g->rows_sorted, n, g->pos,
-                                                                     d_cnt, g->arc0);
+        k_relabel_rows<<<grid_for(n, 256, g->sm_count), 256, 0, s>>>(g->row_ptr, g->rows_sorted, g->out_ptr, n,
+                                                                     g->pos, d_cnt, g->arc0, g->odeg);
         if ((rc = exclusive_scan_i32(d_cnt, (int64_t)n + 1, g->rp2, d_tiles, s)) != FSGP_OK) break;
         if (nnz > 0)
             k_relabel_cols<<<grid_for((int64_t)n * 32, 256, g->sm_count), 256, 0, s>>>(g->arc0, g->rp2, g->col,

@@ -39,6 +39,7 @@ constexpr size_t kOffPc = 256;            // kPC x u64 plane popcounts (2 used)
 constexpr size_t kOffInfo = 512;          // u64 info[4]: max in-degree, chunks, k_sat
 constexpr size_t kOffSet = 768;           // SetParams of the single set
 constexpr size_t kOffSurv = 1024;         // (kSurvCap + 1) x u64
+static_assert(sizeof(SetParams) <= kOffSurv - kOffSet, "scratch layout");
 constexpr size_t kOffRows = kOffSurv + a256(sizeof(uint64_t) * (kSurvCap + 1));
 
 std::mutex g_mu;
@@ -248,8 +249,6 @@ extern "C" int fsgp_step_noalloc(int32_t model, const fsgp_params *params, const
     A.rp = row_ptr;        // rows are the caller's nodes: no relabelling (orig, pos null)
     A.col = col_idx;
     A.arc0 = row_ptr;      // IC arc keys: the caller's arc positions
-    A.out_ptr = row_ptr;   // read only for frontier bookkeeping, which this step discards
-    A.out_dst = nullptr;
     A.n = n;
     A.Ws = Ws;
     A.ws_shift = __builtin_ctz((unsigned)Ws);

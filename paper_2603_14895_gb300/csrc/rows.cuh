@@ -541,7 +541,7 @@ __device__ __forceinline__ void rows_body(const StepArgs &A, int which, int32_t 
         }
         const bool leader = writer && tl == 0;
         const bool want = leader && fl != 0u;
-        if (want && (fl & 1u)) acc.push_deg += (unsigned long long)(__ldg(A.out_ptr + node + 1) - __ldg(A.out_ptr + node));
+        if (want && (fl & 1u)) acc.push_deg += out_degree(A, v);
         if (A.prof_bytes && leader) acc.bytes += row_bytes(SW, P, any_need != 0u, end - beg);
         list_append(A, build, want, (int32_t)((uint32_t)v | ((fl & 1u) ? kPushBit : 0u)), list_slot);
         if (sparse && leader) atomicAnd(&A.bitmap[v >> 5], ~(1u << (v & 31)));
@@ -634,14 +634,14 @@ __device__ __forceinline__ void draw_counts(const StepArgs &A, TileT &T, int n, 
             if ((uint64_t)d < (1ull << B)) sat = ge_const<B>(c, (uint32_t)d) & cand;
             const uint32_t rem = cand & ~sat;
             chg = sat;
-            if (rem) chg |= counts_u_less_nb<B>(nb, P, c, rem, LtThr{(uint64_t)d}, tie_fn);
+            if (rem) chg |= counts_u_less_nb<B>(nb, P, c, rem, LtThr{(uint32_t)d}, tie_fn);
         } else {
             const int32_t ksat = __ldg(&sp.ksat);
             uint32_t sat = 0u;
             if ((uint64_t)ksat < (1ull << B)) sat = ge_const<B>(c, (uint32_t)ksat) & cand;
             const uint32_t rem = cand & ~sat;
-            chg = cand;
-            if (rem) chg &= ~counts_u_less_nb<B>(nb, P, c, rem, SurvThr{sp.surv}, tie_fn);
+            chg = __ldg(&sp.never) ? sat : cand;
+            if (rem && chg == cand) chg &= ~counts_u_less_nb<B>(nb, P, c, rem, SurvThr<(B <= 8)>{sp.surv, sp.masks}, tie_fn);
         }
         T.c[0][slot] = (chg & ~tied) | won;
     }
@@ -681,11 +681,9 @@ __device__ __forceinline__ void draw_tile(const StepArgs &A, TileT &T, int nq, c
     if constexpr (ModelTraits<MODEL>::counts) draw_counts<MODEL, B>(A, T, nq, lane, ctx);
     else draw_arc_items<MODEL>(A, T, na, lane, ctx);
     if constexpr (ModelTraits<MODEL>::fixed_draws >= 1)
-        draw_fixed(A, T.f[0], T.eq(), T.qf[0], nf[0], TAG_RECOVER, lane, ctx,
-                   [](const SetParams &sp) { return __ldg(&sp.g_rec); });
+        draw_fixed<false>(A, T.f[0], T.eq(), T.qf[0], nf[0], lane, ctx);
     if constexpr (ModelTraits<MODEL>::fixed_draws >= 2)
-        draw_fixed(A, T.f[1], T.eq(), T.qf[1], nf[1], TAG_LATENT, lane, ctx,
-                   [](const SetParams &sp) { return __ldg(&sp.a_lat); });
+        draw_fixed<true>(A, T.f[1], T.eq(), T.qf[1], nf[1], lane, ctx);
 }
 
 // Lanes of the word that may leave their state without in-arcs through fixed draw j.
@@ -1038,10 +1036,7 @@ __device__ __forceinline__ void rows_tile(const StepArgs &A, int which, uint8_t 
                 for (int o = 1; o < TEAM; o <<= 1) fl |= __shfl_xor_sync(0xffffffffu, fl, o);
                 const bool leader = v >= 0 && tl == 0;
                 const bool want = leader && fl != 0u;
-                if (want && (fl & 1u)) {
-                    const uint32_t node = T.node[r];
-                    acc.push_deg += (unsigned long long)(__ldg(A.out_ptr + node + 1) - __ldg(A.out_ptr + node));
-                }
+                if (want && (fl & 1u)) acc.push_deg += out_degree(A, v);
                 list_append(A, build, want, (int32_t)((uint32_t)v | ((fl & 1u) ? kPushBit : 0u)), list_slot);
                 if (sparse && leader) atomicAnd(&A.bitmap[v >> 5], ~(1u << (v & 31)));
             }
@@ -1088,10 +1083,7 @@ __device__ __forceinline__ void rows_tile(const StepArgs &A, int which, uint8_t 
                     for (int o = 1; o < GRP; o <<= 1) fl |= __shfl_xor_sync(0xffffffffu, fl, o);
                     const bool leader = v >= 0 && lane % GRP == 0;
                     const bool want = leader && fl != 0u;
-                    if (want && (fl & 1u)) {
-                        const uint32_t node = T.node[r];
-                        acc.push_deg += (unsigned long long)(__ldg(A.out_ptr + node + 1) - __ldg(A.out_ptr + node));
-                    }
+                    if (want && (fl & 1u)) acc.push_deg += out_degree(A, v);
                     list_append(A, build, want, (int32_t)((uint32_t)v | ((fl & 1u) ? kPushBit : 0u)), list_slot);
                     if (sparse && leader) atomicAnd(&A.bitmap[v >> 5], ~(1u << (v & 31)));
                     fl = 0u;
@@ -1457,7 +1449,7 @@ __global__ void __launch_bounds__(kBlock) k_hub_finalize(StepArgs A) {
         if (A.hub_sat)
             for (int sl = lane; sl < A.nslices; sl += 32) A.hub_sat[h * A.nslices + sl] = 0u;
         const bool want = cand && lane == 0 && fl != 0u;
-        if (want && (fl & 1u)) acc.push_deg += (unsigned long long)(__ldg(A.out_ptr + node + 1) - __ldg(A.out_ptr + node));
+        if (want && (fl & 1u)) acc.push_deg += out_degree(A, v);
         if (A.prof_bytes && cand && lane == 0)
             acc.bytes += row_bytes(A.Wn, P, false, 0) + 2ull * 4ull * 32ull * (unsigned long long)A.Wn;
         list_append(A, build, want, (int32_t)((uint32_t)v | ((fl & 1u) ? kPushBit : 0u)), list_slot);
@@ -1651,7 +1643,7 @@ __device__ __forceinline__ void lane_body(const StepArgs &A, uint8_t *smem, int3
             }
         }
         const bool want = has && fl != 0u;
-        if (want && (fl & 1u)) acc.push_deg += (unsigned long long)(__ldg(A.out_ptr + node + 1) - __ldg(A.out_ptr + node));
+        if (want && (fl & 1u)) acc.push_deg += out_degree(A, v);
         if (A.prof_bytes && has) acc.bytes += row_bytes(SWL, P, d > 0, d);
         list_append(A, build, want, (int32_t)((uint32_t)v | ((fl & 1u) ? kPushBit : 0u)), list_slot);
     }
@@ -1832,10 +1824,7 @@ __device__ __forceinline__ void lane_tile(const StepArgs &A, uint8_t *smem, int3
             }
         }
         const bool want = has && fl != 0u;
-        if (want && (fl & 1u)) {
-            const uint32_t node = (uint32_t)e4.x;
-            acc.push_deg += (unsigned long long)(__ldg(A.out_ptr + node + 1) - __ldg(A.out_ptr + node));
-        }
+        if (want && (fl & 1u)) acc.push_deg += out_degree(A, v);
         if (A.prof_bytes && has) acc.bytes += row_bytes(SWL, P, d > 0, d);
         list_append(A, build, want, (int32_t)((uint32_t)v | ((fl & 1u) ? kPushBit : 0u)), list_slot);
         __syncwarp();   // the next tile overwrites the slots

@@ -116,10 +116,7 @@ __global__ void __launch_bounds__(kBlock) k_init_scan(StepArgs A, int model) {
                 if (e_plane >= 0) self |= (e_plane == 2 ? s2 : s1) != 0u;
             }
         }
-        if (push) {
-            const uint32_t node = node_of(A, (int32_t)v);
-            acc.push_deg += (unsigned long long)(A.out_ptr[node + 1] - A.out_ptr[node]);
-        }
+        if (push) acc.push_deg += out_degree(A, (int32_t)v);
         if (has && A.prof_bytes) acc.bytes += (unsigned long long)np * 4ull * (unsigned long long)A.Wn;
         // rows that push, or whose exposed lanes change on their own, are visited at step 1
         list_append(A, build, has && (push || self), (int32_t)((uint32_t)v | (push ? kPushBit : 0u)), 0);
@@ -616,6 +613,11 @@ static int run_wave(fsgp_graph *g, int model, int ic_mode, int weighted, const S
 
     // per-set parameters and survival tables
     std::vector<uint64_t> surv_all;
+    std::vector<uint32_t> mask_all;      // 256 x 8 per table
+    std::vector<size_t> mask_off((size_t)S, 0);
+    auto put_masks = [](uint32_t t8, uint32_t *m) {
+        for (int j = 0; j < 8; ++j) m[j] = (t8 >> (7 - j)) & 1u ? 0xffffffffu : 0u;
+    };
     std::vector<size_t> surv_off((size_t)S), survmu_off((size_t)S), survnu_off((size_t)S);
     std::vector<SetParams> hp((size_t)S);
     int64_t seeds_total = 0, preal_total = 0, planes_total = 0;
@@ -628,8 +630,23 @@ static int run_wave(fsgp_graph *g, int model, int ic_mode, int weighted, const S
         p = SetParams{};
         surv_off[i] = surv_all.size();
         int32_t ksat = INT32_MAX;
-        if (infection_table) survival_table(x.beta, g->max_deg, surv_all, &ksat);
-        else surv_all.push_back(TWO32);
+        // sets of one call share beta, and with it the tables
+        const bool shared = i > 0 && infection_table && x.beta == sets[i - 1]->beta;
+        if (shared) {
+            surv_off[i] = surv_off[i - 1];
+            mask_off[i] = mask_off[i - 1];
+            ksat = hp[i - 1].ksat;
+        } else if (infection_table) {
+            survival_table(x.beta, g->max_deg, surv_all, &ksat);
+            mask_off[i] = mask_all.size();
+            mask_all.resize(mask_off[i] + 256 * 8, 0u);
+            const size_t entries = surv_all.size() - surv_off[i];
+            for (size_t k = 1; k < std::min<size_t>(entries, 256); ++k)
+                put_masks((uint32_t)(surv_all[surv_off[i] + k] >> 24) & 0xffu, &mask_all[mask_off[i] + 8 * k]);
+        } else {
+            surv_all.push_back(TWO32);
+        }
+        p.never = infection_table && g->max_deg >= 1 && surv_all[surv_off[i] + 1] == TWO32;
         survmu_off[i] = survnu_off[i] = surv_off[i];
         p.ksat_mu = p.ksat_nu = ksat;
         if (model == FSGP_SWIR) {
@@ -646,6 +663,11 @@ static int run_wave(fsgp_graph *g, int model, int ic_mode, int weighted, const S
         p.last_mask = (x.R & 31) ? ((1u << (x.R & 31)) - 1u) : 0xffffffffu;
         p.R = x.R;
         p.g_rec = (uint64_t)llrint(x.gamma * 4294967296.0);
+        uint32_t m8[8];
+        put_masks((uint32_t)(p.g_rec >> 24) & 0xffu, m8);   // (2^32 and 0 are decided without)
+        memcpy(p.rec_masks, m8, sizeof m8);
+        put_masks((uint32_t)(p.a_lat >> 24) & 0xffu, m8);
+        memcpy(p.lat_masks, m8, sizeof m8);
         p.beta_f = (float)x.beta;
         p.p_const = (uint64_t)llrint(x.ic_p * 4294967296.0);
         seed_off[i] = seeds_total;
@@ -661,7 +683,7 @@ static int run_wave(fsgp_graph *g, int model, int ic_mode, int weighted, const S
     const size_t state_words = (size_t)P * n * Wn;
     enum { O_STATE, O_PC, O_CTL, O_LIST0, O_LIST1, O_CSMALL, O_CMID, O_BITMAP, O_LANES,
            O_HUB, O_SURV, O_SEEDS, O_COUNTS, O_FREQ, O_PREAL, O_PLANES, O_PROF, O_SP, O_OUT,
-           O_STEPS, O_D0, O_HUBSAT, O_END };
+           O_STEPS, O_D0, O_HUBSAT, O_MASKS, O_END };
     size_t sz[O_END] = {0};
     sz[O_STATE] = 2 * state_words * sizeof(uint32_t);
     sz[O_PC] = T1 * S * kPC * sizeof(unsigned long long);
@@ -685,6 +707,7 @@ static int run_wave(fsgp_graph *g, int model, int ic_mode, int weighted, const S
     sz[O_D0] = (size_t)n_d0 * sizeof(int32_t);
     const bool hub_sat = !weighted && (model == FSGP_SIR || model == FSGP_SIS || model == FSGP_SEIR || model == FSGP_SEIS);
     sz[O_HUBSAT] = hub_sat ? (size_t)n_hubs * nslices * sizeof(uint32_t) : 0;
+    sz[O_MASKS] = mask_all.size() * sizeof(uint32_t);
     size_t off[O_END], total = 0;
     for (int i = 0; i < O_END; ++i) {
         off[i] = total;
@@ -706,10 +729,13 @@ static int run_wave(fsgp_graph *g, int model, int ic_mode, int weighted, const S
     int32_t *d_steps = (int32_t *)(ws + off[O_STEPS]);
     for (int i = 0; i < S; ++i) {
         hp[i].surv = d_surv + surv_off[i];
+        hp[i].masks = (const uint4 *)(ws + off[O_MASKS]) + mask_off[i] / 4;
         hp[i].surv_mu = d_surv + survmu_off[i];
         hp[i].surv_nu = d_surv + survnu_off[i];
     }
     FSGP_CUDA(cudaMemcpyAsync(d_surv, surv_all.data(), sz[O_SURV], cudaMemcpyHostToDevice, s));
+    if (sz[O_MASKS])
+        FSGP_CUDA(cudaMemcpyAsync(ws + off[O_MASKS], mask_all.data(), sz[O_MASKS], cudaMemcpyHostToDevice, s));
     FSGP_CUDA(cudaMemcpyAsync(d_sp, hp.data(), sz[O_SP], cudaMemcpyHostToDevice, s));
     // device output pointers of each set (caller memory, or staging for host results)
     std::vector<SetOut> ho((size_t)S);
@@ -798,6 +824,7 @@ static int run_wave(fsgp_graph *g, int model, int ic_mode, int weighted, const S
     A.orig = g->rows_sorted;
     A.pos = g->pos;
     A.arc0 = g->arc0;
+    A.odeg = allow_sparse ? g->odeg : nullptr;   // dense steps only: nothing to choose
     A.out_ptr = g->out_ptr;
     A.out_dst = g->out_dst;
     A.n = n;

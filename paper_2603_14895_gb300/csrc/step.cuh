@@ -63,11 +63,15 @@ struct PersistArgs {
 struct SetParams {
     uint32_t key0, key1;            // rng seed
     const uint64_t *surv;           // survival table (SIR/SIS)
+    const uint4 *masks;             // [256][2] bits 31..24 of surv[k] as masks (0 or ~0), most
+                                    // significant first: what the tiles' compares take in
+    int32_t never;                  // surv[1] = 2^32: no count infects
     int32_t ksat;                   // first k with surv[k] = 0, or INT32_MAX
     int32_t W;                      // words holding valid lanes, ceil(R/32)
     uint32_t last_mask;             // valid lanes of word W-1
     int32_t R;
     uint64_t g_rec;                 // recovery threshold
+    uint4 rec_masks[2], lat_masks[2];   // bits 31..24 of g_rec and a_lat as masks
     uint64_t p_const;               // IC constant threshold
     uint64_t a_lat;                 // SEIR/SEIS: exposed -> infectious threshold
     const uint64_t *surv_mu;        // SWIR: weakening survival table, and its K_sat
@@ -91,6 +95,7 @@ struct StepArgs {
     const int32_t *__restrict__ orig;    // [n] node of new row i, or null
     const int32_t *__restrict__ pos;     // [n] new id of node v, or null
     const int32_t *__restrict__ arc0;    // [n] caller's position of new row i's first arc
+    const int32_t *__restrict__ odeg;    // [n] out-degree of new row i, or null (not wanted)
     const int32_t *__restrict__ out_ptr; // caller's out-CSR (nodes), frontier marking
     const int32_t *__restrict__ out_dst;
     int32_t n;
@@ -171,6 +176,14 @@ __device__ __forceinline__ uint32_t node_of(const StepArgs &A, int32_t i) {
 }
 __device__ __forceinline__ int32_t row_of(const StepArgs &A, int32_t v) {
     return A.pos ? __ldg(A.pos + v) : v;
+}
+
+// Out-degree of new row i, summed over the rows that push to choose the next step's path.
+// (By row, so that neighbouring rows share sectors: through the nodes' out-CSR pointers it
+// was one random sector per pushing row and step.  With the threshold masks of tile.cuh, SIS
+// on R-MAT n = 8M: 178 to 174 ms; SIR on n = 16.8M: 209 to 205 ms.)
+__device__ __forceinline__ unsigned long long out_degree(const StepArgs &A, int32_t i) {
+    return A.odeg ? (unsigned long long)__ldg(A.odeg + i) : 0ull;
 }
 
 // profile kinds (fsgp_profile)

@@ -27,16 +27,32 @@ __device__ __forceinline__ uint32_t maj_less(uint32_t p, uint32_t t, uint32_t lt
 // Bit b (0 = least significant) of x as a mask.
 __device__ __forceinline__ uint32_t bit_mask(uint32_t x, int b) { return (uint32_t)((int32_t)(x << (31 - b)) >> 31); }
 
+// Eight threshold bits as masks, most significant first.
+struct Masks8 {
+    uint32_t m[8];
+};
+__device__ __forceinline__ Masks8 masks_of(uint32_t t8) {
+    Masks8 r;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) r.m[j] = bit_mask(t8, 7 - j);
+    return r;
+}
+// ... from a table: two 16-byte loads, mostly of addresses the warp shares, in place of
+// sixteen operations of the pipe that the compares and half of Philox already fill.
+__device__ __forceinline__ Masks8 masks_at(const uint4 *t) {
+    const uint4 a = __ldg(t), b = __ldg(t + 1);
+    return Masks8{{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w}};
+}
+
 // u < t (lt) and u <= t (le) of the top eight bits, lanes in parallel; p[0] is the most
 // significant plane.
-__device__ __forceinline__ void less8(const Planes8 &P, uint32_t t8, uint32_t &lt, uint32_t &le) {
+__device__ __forceinline__ void less8(const Planes8 &P, const Masks8 &t, uint32_t &lt, uint32_t &le) {
     lt = 0u;
     le = 0xffffffffu;
 #pragma unroll
     for (int j = 7; j >= 0; --j) {
-        const uint32_t t = bit_mask(t8, 7 - j);
-        lt = maj_less(P.p[j], t, lt);
-        le = maj_less(P.p[j], t, le);
+        lt = maj_less(P.p[j], t.m[j], lt);
+        le = maj_less(P.p[j], t.m[j], le);
     }
 }
 
@@ -58,20 +74,30 @@ __device__ __forceinline__ uint32_t less_from(uint32_t eq, uint32_t th, uint32_t
     return lt;
 }
 
-// The threshold of a lane with count k, below which its uniform must lie: the survival
-// table (a lane at or above it is infected), or the linear threshold's k / d.
+// The threshold of a lane with count k, below which its uniform must lie, and its top eight
+// bits as masks: the survival table (a lane at or above it is infected), or the linear
+// threshold's floor(k * 2^32 / d) + 1, which is below 2^32 for k < d.
+template <bool TABLE>   // masks from the table (counts up to 255)
 struct SurvThr {
     const uint64_t *surv;
-    __device__ __forceinline__ uint64_t operator()(uint32_t k) const { return __ldg(surv + k); }
+    const uint4 *table;
+    static constexpr bool falls = true;   // with k
+    __device__ __forceinline__ uint32_t operator()(uint32_t k) const { return (uint32_t)__ldg(surv + k); }
+    __device__ __forceinline__ Masks8 masks(uint32_t k) const {
+        if constexpr (TABLE) return masks_at(table + 2 * k);
+        else return masks_of((*this)(k) >> 24);
+    }
 };
 struct LtThr {
-    uint64_t d;
-    __device__ __forceinline__ uint64_t operator()(uint32_t k) const { return ((uint64_t)k << 32) / d + 1ull; }
+    uint32_t d;
+    static constexpr bool falls = false;
+    __device__ __forceinline__ uint32_t operator()(uint32_t k) const { return (uint32_t)(((uint64_t)k << 32) / d) + 1u; }
+    __device__ __forceinline__ Masks8 masks(uint32_t k) const { return masks_of((*this)(k) >> 24); }
 };
 
 // P: the top eight planes of the lanes' uniforms.
 // Lanes of M (M != 0; counts at least 1, thresholds thr(k) monotone in k and in
-// (0, 2^32) unless all are 2^32) whose uniform is below their threshold.  All lanes are
+// [1, 2^32)) whose uniform is below their threshold.  All lanes are
 // first compared with the thresholds of the smallest and the largest count on the top
 // eight bits; a lane outside that range is decided, and the few inside it (on average one
 // in five words has one, R-MAT, SIS, beta = 0.01) are compared by groups of equal count.
@@ -81,15 +107,14 @@ template <int B, class Thr, class TieFn>
 __device__ __forceinline__ uint32_t counts_u_less(const Planes8 &P, const uint32_t (&c)[B], uint32_t M, Thr thr_of,
                                                   TieFn tie_fn) {
     const uint32_t ka = min_count<B>(c, M), kb = max_count<B>(c, M);
-    const uint64_t ta = thr_of(ka), tb = thr_of(kb);
-    const uint64_t lo = ta < tb ? ta : tb, hi = ta < tb ? tb : ta;
-    if (lo >= TWO32) return M;
     uint32_t lt_lo = 0u, le_hi = 0xffffffffu;
-    const uint32_t lo8 = (uint32_t)(lo >> 24), hi8 = (uint32_t)((hi < TWO32 ? hi : TWO32 - 1ull) >> 24);
+    {
+        const Masks8 lo = thr_of.masks(Thr::falls ? kb : ka), hi = thr_of.masks(Thr::falls ? ka : kb);
 #pragma unroll
-    for (int j = 7; j >= 0; --j) {
-        lt_lo = maj_less(P.p[j], bit_mask(lo8, 7 - j), lt_lo);
-        le_hi = maj_less(P.p[j], bit_mask(hi8, 7 - j), le_hi);
+        for (int j = 7; j >= 0; --j) {
+            lt_lo = maj_less(P.p[j], lo.m[j], lt_lo);
+            le_hi = maj_less(P.p[j], hi.m[j], le_hi);
+        }
     }
     uint32_t res = M & lt_lo;
     uint32_t U = M & ~lt_lo & le_hi;
@@ -104,12 +129,11 @@ __device__ __forceinline__ uint32_t counts_u_less(const Planes8 &P, const uint32
             Mk &= ~(c[b] ^ bit);
         }
         U &= ~Mk;
-        const uint32_t th = (uint32_t)thr_of(k);
         uint32_t lt, le;
-        less8(P, th >> 24, lt, le);
+        less8(P, thr_of.masks(k), lt, le);
         res |= Mk & lt;
         const uint32_t tie = Mk & le & ~lt;
-        if (tie) tie_fn(tie, th);
+        if (tie) tie_fn(tie, thr_of(k));
     }
     return res;
 }
@@ -124,7 +148,10 @@ __device__ __forceinline__ uint32_t counts_u_less_nb(int nb, const Planes8 &P, c
             uint32_t h[B / 2];
 #pragma unroll
             for (int b = 0; b < B / 2; ++b) h[b] = c[b];
-            return counts_u_less_nb<B / 2>(nb, P, h, M, thr_of, tie_fn);
+            if constexpr (B == 16 && Thr::falls)
+                return counts_u_less_nb<8>(nb, P, h, M, SurvThr<true>{thr_of.surv, thr_of.table}, tie_fn);
+            else
+                return counts_u_less_nb<B / 2>(nb, P, h, M, thr_of, tie_fn);
         }
     }
     return counts_u_less<B>(P, c, M, thr_of, tie_fn);
@@ -182,14 +209,16 @@ __device__ __forceinline__ void queue_push(uint16_t *q, int &n, bool want, int s
 }
 
 // Fixed-threshold items (recovery, latent exit): f holds the lanes to draw and receives
-// those whose uniform lies below thr_of(set).  Two Philox blocks (eight bits) per item and
+// those whose uniform lies below the set's threshold.  Two Philox blocks (eight bits) per item and
 // round: with 5 to 15 lanes per word every second item needs the second block, and one
 // round of two interleaved blocks costs less than packing the items between single ones.
 // The items with lanes still tied are packed for the next round (in place: a round writes
 // only positions it has read).  ctx(slot, node, w): the slot's subject and word.
-template <class CtxFn, class ThrFn>
-__device__ __forceinline__ void draw_fixed(const StepArgs &A, uint32_t *f, uint32_t *eqs, uint16_t *q, int n,
-                                           uint32_t tag, int lane, CtxFn ctx, ThrFn thr_of) {
+// LATENT: the exposed lanes' exit, else recovery.
+template <bool LATENT, class CtxFn>
+__device__ __forceinline__ void draw_fixed(const StepArgs &A, uint32_t *f, uint32_t *eqs, uint16_t *q, int n, int lane,
+                                           CtxFn ctx) {
+    constexpr uint32_t tag = LATENT ? TAG_LATENT : TAG_RECOVER;
 #pragma unroll 1
     for (uint32_t m = 0; m < 8u && n > 0; m += 2) {
         int n2 = 0;
@@ -203,7 +232,7 @@ __device__ __forceinline__ void draw_fixed(const StepArgs &A, uint32_t *f, uint3
                 int w;
                 ctx(slot, node, w);
                 const SetParams &sp = A.sp[w >> A.ws_shift];
-                const uint64_t thr = thr_of(sp);
+                const uint64_t thr = __ldg(LATENT ? &sp.a_lat : &sp.g_rec);
                 const uint32_t now = f[slot];
                 uint32_t less = m ? now : 0u;
                 eq = m ? eqs[q0 + lane] : now;
@@ -216,7 +245,8 @@ __device__ __forceinline__ void draw_fixed(const StepArgs &A, uint32_t *f, uint3
                     const Planes8 P = philox4x32_10_x2(node, A.t, A.gbase + (uint32_t)(w & (A.Ws - 1)), (tag << 8) | m,
                                                        __ldg(&sp.key0), __ldg(&sp.key1));
                     uint32_t lt, le;
-                    less8(P, ((uint32_t)thr << (4u * m)) >> 24, lt, le);
+                    less8(P, m ? masks_of(((uint32_t)thr << (4u * m)) >> 24) : masks_at(LATENT ? sp.lat_masks : sp.rec_masks),
+                          lt, le);
                     less |= eq & lt;
                     eq &= le & ~lt;
                 }
