@@ -136,17 +136,20 @@ struct ExecCache {
 constexpr int kExecCacheSize = 4;
 
 // Per-graph tables of the learned surrogate's aggregation, built on first use: rows with
-// at least kSgLong arcs are split into chunks of kSgChunk arcs whose partial sums meet
-// in a float32 accumulator (zero between uses).
-constexpr int32_t kSgLong = 256;
-constexpr int32_t kSgChunk = 256;
+// at least long_min arcs are split into chunks of kSgChunk arcs whose partial sums meet in a
+// float32 accumulator (zero between uses).  long_min is a power of two, so that the long
+// in-rows are the first of the degree-bucket order, and at least four times the mean degree,
+// so that they stay few: BA n = 300k, one layer: 143 us with 256 (a tile of 255-arc rows
+// outlasts the rest), 71 with 32.
+constexpr int32_t kSgLongMin = 32, kSgLongMax = 256;
+constexpr int32_t kSgChunk = 32;
 struct SgCache {
     int built = 0;
+    int32_t long_min = kSgLongMin;
     float *inv_din = nullptr;     // [n] 1 / d_in (0 when d_in = 0)
     int4 *in_items = nullptr;     // chunks of long in-CSR rows: {row, begin, end, slot}
     int32_t n_in_items = 0;
-    int32_t *in_long = nullptr;   // [n_in_long] the long in-CSR rows, by slot
-    int32_t n_in_long = 0;
+    int32_t n_in_long = 0;        // long in-CSR rows: the first of rows_sorted, slot = position
     int4 *out_items = nullptr;    // chunks of long out-CSR rows
     int32_t n_out_items = 0;
     int32_t *out_long = nullptr;

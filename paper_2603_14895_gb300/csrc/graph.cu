@@ -307,7 +307,6 @@ static void release(fsgp_graph *g) {
     cudaFree(g->ws.ptr);
     cudaFree(g->sgc.inv_din);
     cudaFree(g->sgc.in_items);
-    cudaFree(g->sgc.in_long);
     cudaFree(g->sgc.out_items);
     cudaFree(g->sgc.out_long);
     cudaFree(g->sgc.acc);

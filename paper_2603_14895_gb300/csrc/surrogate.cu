@@ -101,93 +101,114 @@ __global__ void k_seed_bits(const int32_t *__restrict__ cand, int32_t k, int32_t
     if (advance && threadIdx.x == 0) *cur = c + 1;
 }
 
-// m_v = mean over in-arcs of h_u (bfloat16 in and out, float32 sums).  A group of
-// G = agg_arcs<F>() * F/8 threads takes one work item: F/8 threads cover the F features
-// of a source row (16 bytes each) and the subgroups take every agg_arcs-th arc, so each
-// load instruction fetches several source rows; the subgroups' sums meet by shuffle.
-// (Measured on GB300, BA n = 500k: two subgroups for F = 64, four for F = 8.)
-// Items 0..n-1 are rows (rows with >= kSgLong arcs are skipped); items n.. are the chunks
-// of those long rows, whose partial sums go to acc[slot] for k_agg_fin.
+// Screening: take back candidate *cur's seed features and set candidate *cur + 1's (at most
+// kClusterSeeds seeds), then advance *cur; past the last candidate only the taking back is
+// done.  One cluster of CTAs with cluster barriers between its phases (clear, count, write
+// the counts' logarithms) in place of seven launches of a microsecond or two each.
+constexpr int kSeedCtas = 8, kClusterSeeds = 64;
+__device__ __forceinline__ void cluster_barrier() {
+    __threadfence();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__global__ void __cluster_dims__(kSeedCtas, 1, 1) __launch_bounds__(256)
+    k_seed_next(const int32_t *__restrict__ cand, int32_t k, int32_t n_cand, int32_t *cur,
+                const int32_t *__restrict__ out_ptr, const int32_t *__restrict__ out_dst, int32_t *cnt, bf16 *x) {
+    const int c = *(volatile int32_t *)cur + 1;
+    auto each_out = [&](int cc, auto f) {
+        for (int i = blockIdx.x; i < k; i += gridDim.x) {
+            const int32_t sd = cand[(size_t)cc * k + i];
+            for (int32_t a = out_ptr[sd] + threadIdx.x; a < out_ptr[sd + 1]; a += blockDim.x) f(out_dst[a]);
+        }
+    };
+    if (c > 0) {
+        if (blockIdx.x == 0)
+            for (int i = threadIdx.x; i < k; i += blockDim.x)
+                x[(size_t)cand[(size_t)(c - 1) * k + i] * F0] = __float2bfloat16(0.f);
+        each_out(c - 1, [&](int32_t v) {
+            cnt[v] = 0;
+            x[(size_t)v * F0 + 5] = __float2bfloat16(0.f);
+        });
+    }
+    cluster_barrier();
+    if (c < n_cand) {
+        if (blockIdx.x == 0)
+            for (int i = threadIdx.x; i < k; i += blockDim.x)
+                x[(size_t)cand[(size_t)c * k + i] * F0] = __float2bfloat16(1.f);
+        each_out(c, [&](int32_t v) { atomicAdd(&cnt[v], 1); });
+    }
+    cluster_barrier();
+    if (c < n_cand)
+        each_out(c, [&](int32_t v) { x[(size_t)v * F0 + 5] = __float2bfloat16(log1pf((float)__ldcg(cnt + v))); });
+    if (blockIdx.x == 0 && threadIdx.x == 0) *cur = c;
+}
+
+// Sixteen bytes of a gathered row, zeros without a row.  In assembly so that a round's eight
+// loads are issued one behind the other: left to itself the compiler kept registers, not
+// loads (32 registers and two or so loads in flight).
+__device__ __forceinline__ uint4 ld_row16(const void *p, bool has) {
+    uint4 r;
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %5, 0;\n mov.b32 %0, 0;\n mov.b32 %1, 0;\n mov.b32 %2, 0;\n"
+                 " mov.b32 %3, 0;\n @p ld.global.nc.v4.b32 {%0, %1, %2, %3}, [%4];\n}"
+                 : "=&r"(r.x), "=&r"(r.y), "=&r"(r.z), "=&r"(r.w) : "l"(p), "r"((uint32_t)has));
+    return r;
+}
+
+__device__ __forceinline__ void add_bf16x8(float (&sum)[8], const uint4 &x) {
+    const bf162 *xp = reinterpret_cast<const bf162 *>(&x);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        sum[2 * i] += __bfloat162float(xp[i].x);
+        sum[2 * i + 1] += __bfloat162float(xp[i].y);
+    }
+}
+
+// Sums of h_u over the chunks of long in-rows (items {row, begin, end, slot}), added to
+// acc[slot] in float32.  Eight lanes take one chunk of kSgChunk arcs, eight at a time: F = 64
+// 16 bytes of every source row each, F = 8 one source row each (their sums meet by
+// shuffle).  (Chunks of 256 arcs, two at a time, took 76 us beside a layer's 182, BA
+// n = 300k: few of them, each one long chain.)
 template <int F>
-__host__ __device__ constexpr int agg_arcs() { return F == 8 ? 4 : 2; }
-template <int F>
-__global__ void k_agg(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col, int32_t n,
-                      const bf16 *__restrict__ h, bf16 *m, const int4 *__restrict__ items, int32_t n_items,
-                      float *acc) {
-    constexpr int TPR = F / 8;
-    constexpr int kAggArcs = agg_arcs<F>();
-    constexpr int G = TPR * kAggArcs;
-    static_assert(G <= 32 && (32 % G) == 0, "a group lies within a warp");
+__global__ void __launch_bounds__(256) k_agg_long(const int32_t *__restrict__ col, const bf16 *__restrict__ h,
+                                                  const int4 *__restrict__ items, int32_t n_items, float *acc) {
+    const int lane = threadIdx.x & 31, j = lane & 7, g0 = lane & 24;
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
-    const int j = (int)(t % TPR);                // 16-byte feature chunk
-    const int sub = (int)((t / TPR) % kAggArcs); // arc subgroup
-    const int64_t total = (int64_t)n + n_items;
-    // whole warps iterate together (the shuffles below need every lane of the group)
-    const int64_t v_end = (total + (nthreads / G) - 1) / (nthreads / G) * (nthreads / G);
-    for (int64_t v = t / G; v < v_end; v += nthreads / G) {
-        int32_t row = 0, b = 0, e = 0, slot = -1;
-        bool skip = v >= total;
-        if (!skip) {
-            if (v < n) {
-                row = (int32_t)v;
-                b = row_ptr[v];
-                e = row_ptr[v + 1];
-                if (e - b >= kSgLong) skip = true;
-            } else {
-                const int4 it = items[v - n];
-                row = it.x, b = it.y, e = it.z, slot = it.w;
-            }
-        }
+    const int64_t groups = ((int64_t)gridDim.x * blockDim.x) >> 3;
+    for (int64_t v = t >> 3; __any_sync(0xffffffffu, v < n_items); v += groups) {
+        int4 it = make_int4(0, 0, 0, -1);
+        if (v < n_items) it = __ldg(items + v);
         float sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        if (!skip) {
-#pragma unroll 2
-            for (int32_t a = b + sub; a < e; a += kAggArcs) {
-                const uint4 x = __ldg(reinterpret_cast<const uint4 *>(h + (size_t)__ldg(col + a) * F) + j);
-                const bf162 *xp = reinterpret_cast<const bf162 *>(&x);
+        int32_t b = it.y;
+        int32_t mine = b + j < it.z ? __ldg(col + b + j) : -1;
+        while (__any_sync(0xffffffffu, b < it.z)) {
+            if constexpr (F == H) {
+                uint4 x[8];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    sum[2 * i] += __bfloat162float(xp[i].x);
-                    sum[2 * i + 1] += __bfloat162float(xp[i].y);
+                for (int q = 0; q < 8; ++q) {
+                    const int32_t u = __shfl_sync(0xffffffffu, mine, g0 + q);
+                    x[q] = ld_row16(h + (size_t)max(u, 0) * F + 8 * j, u >= 0);
                 }
+                b += 8;
+                mine = b + j < it.z ? __ldg(col + b + j) : -1;
+#pragma unroll
+                for (int q = 0; q < 8; ++q) add_bf16x8(sum, x[q]);
+            } else {
+                const int32_t u = mine;
+                b += 8;
+                mine = b + j < it.z ? __ldg(col + b + j) : -1;
+                if (u >= 0) add_bf16x8(sum, __ldg(reinterpret_cast<const uint4 *>(h + (size_t)u * F)));
             }
         }
+        if constexpr (F != H) {
 #pragma unroll
-        for (int o = TPR; o < G; o <<= 1)
+            for (int o = 1; o < 8; o <<= 1)
 #pragma unroll
-            for (int i = 0; i < 8; ++i) sum[i] += __shfl_xor_sync(0xffffffffu, sum[i], o);
-        if (skip || sub != 0) continue;
-        if (slot < 0) {
-            const float inv = e > b ? 1.f / (float)(e - b) : 0.f;
-            uint4 o;
-            bf162 *op = reinterpret_cast<bf162 *>(&o);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) op[i] = __floats2bfloat162_rn(sum[2 * i] * inv, sum[2 * i + 1] * inv);
-            reinterpret_cast<uint4 *>(m + (size_t)row * F)[j] = o;
-        } else {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) atomicAdd(acc + (size_t)slot * F + 8 * j + i, sum[i]);
+                for (int i = 0; i < 8; ++i) sum[i] += __shfl_xor_sync(0xffffffffu, sum[i], o);
         }
+        if (it.w < 0 || (F != H && j != 0)) continue;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) atomicAdd(acc + (size_t)it.w * F + (F == H ? 8 * j : 0) + i, sum[i]);
     }
 }
-
-// Long rows: m = acc / d_in, and acc back to zero.
-template <int F>
-__global__ void k_agg_fin(const int32_t *__restrict__ long_rows, int32_t n_long, const int32_t *__restrict__ row_ptr,
-                          float *acc, bf16 *m) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (int64_t)n_long * (F / 2);
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t slot = i / (F / 2);
-        const int j = (int)(i % (F / 2));
-        const int32_t row = long_rows[slot];
-        const float inv = 1.f / (float)(row_ptr[row + 1] - row_ptr[row]);
-        float *p = acc + slot * F + 2 * j;
-        reinterpret_cast<bf162 *>(m + (size_t)row * F)[j] = __floats2bfloat162_rn(p[0] * inv, p[1] * inv);
-        p[0] = p[1] = 0.f;
-    }
-}
-
-__device__ __forceinline__ uint32_t ld_b32(const bf16 *p) { return *reinterpret_cast<const uint32_t *>(p); }
 
 __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
     asm volatile(
@@ -197,16 +218,29 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], 
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// ------------------------------------------------------- dense layer on tcgen05 / TMEM
+// ------------------------------------- one layer: aggregation and tcgen05 / TMEM product
 //
-// y = ReLU([h | m] W + b) for tiles of 128 rows, K = 2F (16 or 128), N = 64, on the
-// fifth-generation tensor cores: both operands staged in shared memory in the canonical
-// K-major layout without swizzle (8-row x 16-byte core matrices; the two K-neighbour core
-// matrices of one instruction lie 128 B apart, 8-row groups K*16 B apart), one elected
-// thread issues K/16 tcgen05.mma (kind::f16: bfloat16 in, float32 accumulate) into a
-// 128-lane x 64-column tensor-memory accumulator, commits them to an mbarrier, and the
-// four warps read their 32 lanes back (tcgen05.ld) for bias, ReLU and the bfloat16 store.
-// Persistent CTAs loop over tiles; W^T is staged once per CTA.
+// m_v = mean over in-arcs u -> v of h_u (float32 sums), y = ReLU([h | m] W + b), for tiles of
+// 128 rows, K = 2F (16 or 128), N = 64.  What bounds a layer is the gather of the source
+// rows out of L2 (d_in x 128 bytes per node); the product is a few percent of the tensor
+// pipe.  So the CTA that gathers a tile's means also multiplies it: the means go to shared
+// memory as the right half of the A operand, are never written to memory (unless the
+// backward pass wants them) and never read back, and three CTAs per SM cover one another's
+// products with their gathers.  Rows are taken in degree-bucket order, so that the rows a
+// warp gathers together are of similar length; the long rows (the first n_long of that
+// order) come summed from k_agg_long.
+//   Gather: F/8 lanes per row, 16 bytes each, eight arcs in flight per lane (F = 8: four
+//   lanes per row, one arc each).
+//   Product: both operands in the canonical K-major layout without swizzle (8-row x 16-byte
+//   core matrices; the two K-neighbour core matrices of one instruction lie 128 B apart,
+//   8-row groups K*16 B apart); one elected thread issues K/16 tcgen05.mma (kind::f16:
+//   bfloat16 in, float32 accumulate) into a 128-lane x 64-column tensor-memory accumulator
+//   and commits them to an mbarrier; the eight warps read 32 lanes x 32 columns each back
+//   (tcgen05.ld) for bias, ReLU and the bfloat16 rows, which leave through shared memory so
+//   that every store covers whole 128-byte rows.  W^T is staged once per CTA.
+// Measured on BA n = 500k, m = 4: 105 us a layer (F = 64) plus 25 for the long rows, against
+// 119 for the aggregation and 77 for the product as separate kernels; a screened candidate
+// 0.475 to 0.325 ms.
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -223,58 +257,66 @@ __device__ __forceinline__ uint32_t core_off(int r, int kc, int KC) {
 }
 
 constexpr int kTcRows = 128;            // rows per tile (MMA M)
+constexpr int kTcThreads = 256;
+constexpr int kTcCtas = 3;              // per SM
 constexpr int kTcWaitLimit = 1 << 24;   // mbarrier polls before giving up
 
-// Two A tiles (the next one is fetched with cp.async while the current one is multiplied)
-// and W^T.
+// The A tile, reused for the tile's output rows (128 x 64 bfloat16), and W^T.
 template <int F>
-constexpr size_t tc_smem_bytes() { return (size_t)(2 * kTcRows + H) * (2 * F) * 2; }
+__host__ __device__ constexpr int tc_a_bytes() { return kTcRows * 2 * F * 2 > kTcRows * H * 2 ? kTcRows * 2 * F * 2 : kTcRows * H * 2; }
+template <int F>
+constexpr size_t tc_smem_bytes() { return (size_t)tc_a_bytes<F>() + (size_t)H * (2 * F) * 2; }
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool valid) {
     // a source size of 0 fills the 16 bytes with zeros (rows past the end)
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(valid ? 16 : 0));
 }
 
+__device__ __forceinline__ uint4 scaled_bf16x8(const float (&sum)[8], float inv) {
+    uint4 o;
+    bf162 *op = reinterpret_cast<bf162 *>(&o);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) op[i] = __floats2bfloat162_rn(sum[2 * i] * inv, sum[2 * i + 1] * inv);
+    return o;
+}
+
 // HEAD: the epilogue also applies the output head, p = sigmoid(h . w_o + b_o) of the
 // bfloat16 layer output, and writes p (when p_out is set) and / or adds the sum of p
-// into psum[*cur] (screening); y (the layer output) may then be null.
+// into psum[*cur] (screening).  m_out and y may be null (not wanted).
 template <int F, bool HEAD>
-__global__ void __launch_bounds__(128) k_dense_tc(const bf16 *__restrict__ h, const bf16 *__restrict__ m,
-                                                  const bf16 *__restrict__ Ws, const bf16 *__restrict__ Wn,
-                                                  const float *__restrict__ bias, int32_t n, bf16 *y,
-                                                  const bf16 *__restrict__ wo, const float *__restrict__ bo,
-                                                  float *p_out, float *psum, const int32_t *cur, int32_t *err) {
+__global__ void __launch_bounds__(kTcThreads, kTcCtas)
+    k_layer_tc(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col, const int32_t *__restrict__ order,
+               int32_t n, const bf16 *__restrict__ h, const bf16 *__restrict__ Ws, const bf16 *__restrict__ Wn,
+               const float *__restrict__ bias, int32_t n_long, float *acc, bf16 *m_out, bf16 *y,
+               const bf16 *__restrict__ wo, const float *__restrict__ bo, float *p_out, float *psum,
+               const int32_t *cur, int32_t *err) {
     constexpr int K = 2 * F;
     constexpr int KC = K / 8;            // 16-byte chunks per row
-    constexpr int TILE = kTcRows * K * 2;
+    constexpr int FC = F / 8;            // of them own features
     extern __shared__ __align__(1024) uint8_t tc_smem[];
-    uint8_t *sA0 = tc_smem;                         // 2 x (128 x K)
-    uint8_t *sB = tc_smem + 2 * TILE;               // 64 x K (W transposed)
+    uint8_t *sA = tc_smem;                          // 128 x K, then 128 x 64 output rows
+    uint8_t *sB = tc_smem + tc_a_bytes<F>();        // 64 x K (W transposed)
     __shared__ uint64_t mbar;
     __shared__ uint32_t tmem_base;
+    __shared__ int32_t s_node[2][kTcRows];
+    __shared__ float s_bias[H], s_wo[HEAD ? H : 1], s_dot[HEAD ? 2 : 1][HEAD ? kTcRows : 1];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t tiles = ((int64_t)n + kTcRows - 1) / kTcRows;
     if ((int64_t)blockIdx.x >= tiles) return;
-    auto stage = [&](int buf, int64_t tile) {
-        const uint32_t base = smem_addr(sA0 + buf * TILE);
-        const int64_t row0 = tile * kTcRows;
-        for (int c = tid; c < kTcRows * KC; c += blockDim.x) {
-            const int r = c / KC, kc = c % KC;
-            const int64_t row = row0 + r;
-            const bool valid = row < n;
-            const int64_t rr = valid ? row : 0;
-            const bf16 *src = kc < KC / 2 ? h + (size_t)rr * F + kc * 8 : m + (size_t)rr * F + (kc - KC / 2) * 8;
-            cp_async16(base + core_off(r, kc, KC), src, valid);
-        }
-        asm volatile("cp.async.commit_group;");
-    };
-    stage(0, blockIdx.x);
-    // B: output column c holds its K inputs, Ws rows then Wn rows (coalesced row reads,
+    // B: output column c holds its K inputs, Ws rows then Wn rows (16-byte row reads,
     // element-wise transposed stores)
-    for (int i = tid; i < K * H; i += blockDim.x) {
-        const int k = i / H, col = i % H;
-        const bf16 w = k < F ? Ws[k * H + col] : Wn[(k - F) * H + col];
-        *reinterpret_cast<bf16 *>(sB + core_off(col, k >> 3, KC) + (k & 7) * 2) = w;
+#pragma unroll
+    for (int i = tid; i < K * H / 8; i += kTcThreads) {
+        const int k = i / (H / 8), c8 = i % (H / 8) * 8;
+        const uint4 x = *reinterpret_cast<const uint4 *>((k < F ? Ws + k * H : Wn + (k - F) * H) + c8);
+        const bf16 *w = reinterpret_cast<const bf16 *>(&x);
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            *reinterpret_cast<bf16 *>(sB + core_off(c8 + q, k >> 3, KC) + (k & 7) * 2) = w[q];
+    }
+    if (tid < H) {
+        s_bias[tid] = bias[tid];
+        if constexpr (HEAD) s_wo[tid] = __bfloat162float(wo[tid]);
     }
     if (tid == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&mbar)));
@@ -287,32 +329,126 @@ __global__ void __launch_bounds__(128) k_dense_tc(const bf16 *__restrict__ h, co
     // kind::f16: D f32 (bit 4), A and B bf16 (bits 7, 10), K-major, N = 64, M = 128
     constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(H >> 3) << 17) |
                                ((uint32_t)(kTcRows >> 4) << 24);
-    float wo_f[HEAD ? H : 1];
-    float bo_f = 0.f;
-    if constexpr (HEAD) {
-#pragma unroll
-        for (int j = 0; j < H; ++j) wo_f[j] = __bfloat162float(wo[j]);
-        bo_f = bo[0];
-    }
+    const float bo_f = HEAD ? bo[0] : 0.f;
     float psum_local = 0.f;
     uint32_t phase = 0;
     bool ok = true;
-    int buf = 0;
-    for (int64_t tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x, buf ^= 1) {
-        const int64_t next = tile + gridDim.x;
-        if (next < tiles) {
-            stage(buf ^ 1, next);
-            asm volatile("cp.async.wait_group 1;");   // this tile's copies are done
-        } else {
-            asm volatile("cp.async.wait_group 0;");
+    int nb = 0;
+    // This thread's rows: LPR lanes per row, ITS rows one after another.  The next tile's
+    // nodes, arc ranges and first column indices are loaded while this tile is gathered,
+    // multiplied and stored.
+    constexpr int LPR = F == H ? 8 : 4, RPW = 32 / LPR, ITS = 16 / RPW;
+    const int j = lane % LPR, g0 = lane - j, r0 = warp * 16 + lane / LPR;
+    int32_t node[ITS], beg[ITS], end[ITS], c0[ITS], c1[F == H ? 1 : ITS];
+    auto nodes_of = [&](int64_t tile) {
+#pragma unroll
+        for (int it = 0; it < ITS; ++it) {
+            const int64_t i = tile * kTcRows + r0 + it * RPW;
+            node[it] = i < n ? __ldg(order + i) : -1;
         }
+    };
+    auto ranges_of = [&](int64_t tile) {
+#pragma unroll
+        for (int it = 0; it < ITS; ++it) {
+            beg[it] = end[it] = 0;
+            if (node[it] >= 0) {
+                beg[it] = __ldg(row_ptr + node[it]);
+                end[it] = __ldg(row_ptr + node[it] + 1);
+            }
+        }
+    };
+    auto cols_of = [&](int64_t tile) {
+#pragma unroll
+        for (int it = 0; it < ITS; ++it) {
+            const bool mine = tile * kTcRows + r0 + it * RPW >= n_long;
+            c0[it] = mine && beg[it] + j < end[it] ? __ldg(col + beg[it] + j) : -1;
+            if constexpr (F != H) c1[it] = mine && beg[it] + j + 4 < end[it] ? __ldg(col + beg[it] + j + 4) : -1;
+        }
+    };
+    nodes_of(blockIdx.x);
+    ranges_of(blockIdx.x);
+    cols_of(blockIdx.x);
+    for (int64_t tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x, nb ^= 1) {
+        const int64_t i0 = tile * kTcRows;   // position in `order` of the tile's first row
+        const int64_t next = tile + gridDim.x;
+        if (j == 0)
+#pragma unroll
+            for (int it = 0; it < ITS; ++it) s_node[nb][r0 + it * RPW] = node[it];
+        __syncthreads();                     // the previous tile's rows have left sA
+#pragma unroll
+        for (int it = 0; it < ITS; ++it)     // own features, chunk j
+            if (j < FC)
+                cp_async16(smem_addr(sA) + core_off(r0 + it * RPW, j, KC),
+                           h + (size_t)max(node[it], 0) * F + j * 8, node[it] >= 0);
+        asm volatile("cp.async.commit_group;");
+#pragma unroll
+        for (int it = 0; it < ITS; ++it) {
+            const int r = r0 + it * RPW;
+            const int32_t v = node[it], e = end[it];
+            int32_t b = beg[it];
+            const float inv = e > b ? 1.f / (float)(e - b) : 0.f;
+            float sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            if (i0 + r < n_long && v >= 0) {   // summed already; the accumulator goes back to zero
+                if (F == H || j == 0) {
+                    float4 *a = reinterpret_cast<float4 *>(acc + (size_t)(i0 + r) * F + (F == H ? 8 * j : 0));
+                    const float4 s0 = a[0], s1 = a[1];
+                    a[0] = a[1] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    sum[0] = s0.x, sum[1] = s0.y, sum[2] = s0.z, sum[3] = s0.w;
+                    sum[4] = s1.x, sum[5] = s1.y, sum[6] = s1.z, sum[7] = s1.w;
+                }
+                b = e;
+            }
+            int32_t mine = c0[it];
+            if constexpr (F == H) {
+                // the row's eight lanes hold eight arcs' sources and take 16 bytes of each
+                while (__any_sync(0xffffffffu, b < e)) {
+                    uint4 x[8];
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        const int32_t u = __shfl_sync(0xffffffffu, mine, g0 + q);
+                        x[q] = ld_row16(h + (size_t)max(u, 0) * F + 8 * j, u >= 0);
+                    }
+                    b += 8;
+                    mine = b + j < e ? __ldg(col + b + j) : -1;
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) add_bf16x8(sum, x[q]);
+                }
+                const uint4 o = scaled_bf16x8(sum, inv);
+                *reinterpret_cast<uint4 *>(sA + core_off(r, FC + j, KC)) = o;
+                if (m_out && v >= 0) reinterpret_cast<uint4 *>(m_out + (size_t)v * F)[j] = o;
+            } else {
+                // a source row is 16 bytes: the four lanes take every fourth arc each, two at
+                // a time
+                int32_t mine2 = c1[it];
+                for (int32_t a = b + j; a < e; a += 8) {
+                    const uint4 x = ld_row16(h + (size_t)mine * F, true);
+                    const uint4 x2 = ld_row16(h + (size_t)max(mine2, 0) * F, mine2 >= 0);
+                    mine = a + 8 < e ? __ldg(col + a + 8) : -1;
+                    mine2 = a + 12 < e ? __ldg(col + a + 12) : -1;
+                    add_bf16x8(sum, x);
+                    add_bf16x8(sum, x2);
+                }
+                __syncwarp();
+#pragma unroll
+                for (int o = 1; o < 4; o <<= 1)
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) sum[i] += __shfl_xor_sync(0xffffffffu, sum[i], o);
+                if (j == 0) {
+                    const uint4 o = scaled_bf16x8(sum, inv);
+                    *reinterpret_cast<uint4 *>(sA + core_off(r, FC, KC)) = o;
+                    if (m_out && v >= 0) *reinterpret_cast<uint4 *>(m_out + (size_t)v * F) = o;
+                }
+            }
+        }
+        nodes_of(next);   // (past the last tile: no rows)
+        asm volatile("cp.async.wait_group 0;");
         asm volatile("fence.proxy.async.shared::cta;");   // smem writes -> tensor-core reads
         asm volatile("tcgen05.fence::before_thread_sync;");
         __syncthreads();
         asm volatile("tcgen05.fence::after_thread_sync;");
         const uint32_t tbase = tmem_base;
         if (tid == 0) {
-            const uint32_t a0 = smem_addr(sA0 + buf * TILE), b0 = smem_addr(sB);
+            const uint32_t a0 = smem_addr(sA), b0 = smem_addr(sB);
 #pragma unroll
             for (int k = 0; k < K / 16; ++k) {
                 const uint64_t ad = umma_desc(a0 + k * 256, 128, KC * 128);
@@ -325,6 +461,7 @@ __global__ void __launch_bounds__(128) k_dense_tc(const bf16 *__restrict__ h, co
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
                          ::"r"(smem_addr(&mbar)));
         }
+        ranges_of(next);
         uint32_t done = 0;
         for (int it = 0; it < kTcWaitLimit && !done; ++it)
             asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
@@ -341,47 +478,65 @@ __global__ void __launch_bounds__(128) k_dense_tc(const bf16 *__restrict__ h, co
                              " selp.u32 %0, 1, 0, p;\n}"
                              : "=r"(done) : "r"(smem_addr(&mbar)), "r"(phase ^ 1u));
         } else {
-            const int64_t row = tile * kTcRows + 32 * warp + lane;   // this thread's lane
+            cols_of(next);
+            // this thread: row 32 * (warp % 4) + lane, columns 32 * (warp / 4) .. + 31
+            const int r = 32 * (warp & 3) + lane, half = warp >> 2;
             float dot = 0.f;
 #pragma unroll
-            for (int c0 = 0; c0 < H; c0 += 16) {
-                uint32_t r[16];
-                const uint32_t taddr = tbase + ((uint32_t)(32 * warp) << 16) + (uint32_t)c0;
+            for (int cc = 0; cc < 2; ++cc) {
+                const int c0 = half * 32 + cc * 16;   // first of 16 columns
+                uint32_t d[16];
+                const uint32_t taddr = tbase + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0;
                 asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                             : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-                               "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
-                               "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                             : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3]), "=r"(d[4]), "=r"(d[5]), "=r"(d[6]),
+                               "=r"(d[7]), "=r"(d[8]), "=r"(d[9]), "=r"(d[10]), "=r"(d[11]), "=r"(d[12]),
+                               "=r"(d[13]), "=r"(d[14]), "=r"(d[15])
                              : "r"(taddr));
                 asm volatile("tcgen05.wait::ld.sync.aligned;");
                 bf162 o[8];
 #pragma unroll
                 for (int j = 0; j < 8; ++j)
-                    o[j] = __floats2bfloat162_rn(fmaxf(__uint_as_float(r[2 * j]) + bias[c0 + 2 * j], 0.f),
-                                                 fmaxf(__uint_as_float(r[2 * j + 1]) + bias[c0 + 2 * j + 1], 0.f));
+                    o[j] = __floats2bfloat162_rn(fmaxf(__uint_as_float(d[2 * j]) + s_bias[c0 + 2 * j], 0.f),
+                                                 fmaxf(__uint_as_float(d[2 * j + 1]) + s_bias[c0 + 2 * j + 1], 0.f));
                 if constexpr (HEAD) {
 #pragma unroll
                     for (int j = 0; j < 8; ++j)
-                        dot += __bfloat162float(o[j].x) * wo_f[c0 + 2 * j] + __bfloat162float(o[j].y) * wo_f[c0 + 2 * j + 1];
+                        dot += __bfloat162float(o[j].x) * s_wo[c0 + 2 * j] + __bfloat162float(o[j].y) * s_wo[c0 + 2 * j + 1];
                 }
-                if (y && row < n) {
-                    uint4 *dst = reinterpret_cast<uint4 *>(y + (size_t)row * H + c0);
-                    dst[0] = *reinterpret_cast<const uint4 *>(&o[0]);
-                    dst[1] = *reinterpret_cast<const uint4 *>(&o[4]);
+                if (y) {   // 16-byte chunk c of row r lies at chunk c ^ (r & 7): no bank conflicts
+#pragma unroll
+                    for (int q = 0; q < 2; ++q)
+                        *reinterpret_cast<uint4 *>(sA + r * 128 + (((c0 >> 3) + q) ^ (r & 7)) * 16) =
+                            *reinterpret_cast<const uint4 *>(&o[4 * q]);
                 }
             }
-            if constexpr (HEAD) {
-                if (row < n) {
-                    const float pv = 1.f / (1.f + expf(-(dot + bo_f)));
-                    if (p_out) p_out[row] = pv;
+            if constexpr (HEAD) s_dot[half][r] = dot;
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;");
+        ok = __syncthreads_and(ok) != 0;   // also orders this tile's TMEM reads before the next tile
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        if (!ok) break;
+        if (y) {
+#pragma unroll
+            for (int c = tid; c < kTcRows * 8; c += kTcThreads) {
+                const int r = c >> 3, q = c & 7;
+                const int32_t v = s_node[nb][r];
+                if (v >= 0)
+                    reinterpret_cast<uint4 *>(y + (size_t)v * H)[q] =
+                        *reinterpret_cast<const uint4 *>(sA + r * 128 + (q ^ (r & 7)) * 16);
+            }
+        }
+        if constexpr (HEAD) {
+            if (tid < kTcRows) {
+                const int32_t v = s_node[nb][tid];
+                if (v >= 0) {
+                    const float pv = 1.f / (1.f + expf(-(s_dot[0][tid] + s_dot[1][tid] + bo_f)));
+                    if (p_out) p_out[v] = pv;
                     psum_local += pv;
                 }
             }
         }
-        asm volatile("tcgen05.fence::before_thread_sync;");
-        ok = __syncthreads_and(ok) != 0;   // also orders this tile's reads before the next tile
-        asm volatile("tcgen05.fence::after_thread_sync;");
     }
-    asm volatile("cp.async.wait_group 0;");
     if constexpr (HEAD) {
         if (psum) {
 #pragma unroll
@@ -448,173 +603,228 @@ __global__ void k_head_bwd(const bf16 *__restrict__ h3, const bf16 *__restrict__
 
 // One layer backward on the tensor cores.  dz = dy * (y > 0) is rounded to bfloat16 and
 // both products take bfloat16 operands with float32 accumulation:
-//   input gradients   [dah | dam] = dz W^T      (rows x 2F, float32 out; skipped for layer 1)
+//   input gradients   [dah | dam] = dz W^T      (rows x 2F, float32 out; skipped for layer 1);
+//                     dam is written as dam / d_in, the term its adjoint aggregation sums
 //   weight gradients  [gWs ; gWn] += [h | m]^T dz   (2F x 64, accumulated in registers)
 //   bias gradient     gb += sum_rows dz          (float32, from the unrounded dz)
 // A CTA of 8 warps walks 32-row tiles staged in shared memory: dz (row-major), the input
-// tile A = [h | m] (row-major) and W = [Ws ; Wn] (2F x 64, row-major, staged once).
-// Fragments for the transposed operands are packed from two bfloat16 half-words.
-__device__ __forceinline__ uint32_t pack_bf16(bf16 lo, bf16 hi) {
-    return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
+// tile A = [h | m] (row-major) and W = [Ws ; Wn] (2F x 64, row-major, staged once).  The
+// fragments come from ldmatrix, transposed where the reduction runs over the tile's rows
+// (packing them from half-words took 20 instructions per product); a warp's eight
+// weight-gradient tiles share their column block, and with it the dz fragments.  The next
+// tile's rows are loaded into registers while this one is multiplied.  (BA n = 300k, F = 64:
+// 287 to 108 us.)
+__device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], const bf16 *p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"((uint32_t)__cvta_generic_to_shared(p)) : "memory");
+}
+__device__ __forceinline__ void ldsm_x4_t(uint32_t (&r)[4], const bf16 *p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"((uint32_t)__cvta_generic_to_shared(p)) : "memory");
+}
+__device__ __forceinline__ void ldsm_x2_t(uint32_t &a, uint32_t &b, const bf16 *p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];"
+                 : "=r"(a), "=r"(b) : "r"((uint32_t)__cvta_generic_to_shared(p)) : "memory");
 }
 
 template <int F>
-__global__ void __launch_bounds__(256) k_dense_bwd(const bf16 *__restrict__ h, const bf16 *__restrict__ m,
-                                                   const bf16 *__restrict__ y, const float *__restrict__ dy,
-                                                   const bf16 *__restrict__ Ws, const bf16 *__restrict__ Wn,
-                                                   int32_t n, float *dah, float *dam, float *grad, int l,
-                                                   int input_grad) {
+__global__ void __launch_bounds__(256, 3) k_dense_bwd(const bf16 *__restrict__ h, const bf16 *__restrict__ m,
+                                                      const bf16 *__restrict__ y, const float *__restrict__ dy,
+                                                      const bf16 *__restrict__ Ws, const bf16 *__restrict__ Wn,
+                                                      const float *__restrict__ inv_din, int32_t n, float *dah,
+                                                      float *dam, float *grad, int l, int input_grad) {
     constexpr int K = 2 * F;
     constexpr int RT = 32;            // rows per tile
     constexpr int WP = H + 8;         // padded row of W and dz (bank spread)
     constexpr int AP = K + 8;         // padded row of the input tile
-    constexpr int WT = K / 16 * 8;    // weight-gradient (16 x 8) tiles
-    constexpr int WPW = (WT + 7) / 8; // of them per warp
+    constexpr int MT = K / 16;        // weight-gradient row blocks (each warp: its 8 columns of all)
+    constexpr int AC = RT * (K / 8);  // 16-byte chunks of the input tile
+    constexpr int APT = (AC + 255) / 256;
     __shared__ __align__(16) bf16 Wsm[K * WP];
     __shared__ __align__(16) bf16 Zs[RT * WP];
     __shared__ __align__(16) bf16 As[RT * AP];
     __shared__ float s_b[8][H];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int g = lane >> 2, tg = lane & 3;
-    for (int i = threadIdx.x; i < K * H; i += blockDim.x) {
+    for (int i = tid; i < K * H; i += blockDim.x) {
         const int k = i / H, c = i % H;
         Wsm[k * WP + c] = k < F ? Ws[k * H + c] : Wn[(k - F) * H + c];
     }
-    float wacc[WPW][4];
+    float wacc[MT][4];
 #pragma unroll
-    for (int j = 0; j < WPW; ++j) wacc[j][0] = wacc[j][1] = wacc[j][2] = wacc[j][3] = 0.f;
+    for (int q = 0; q < MT; ++q) wacc[q][0] = wacc[q][1] = wacc[q][2] = wacc[q][3] = 0.f;
     float gb0 = 0.f, gb1 = 0.f;       // bias columns 2 lane, 2 lane + 1
-    for (int64_t r0 = (int64_t)blockIdx.x * RT; r0 < n; r0 += (int64_t)gridDim.x * RT) {
-        __syncthreads();              // previous tile's readers are done (and W is staged)
-        // dz tile: each thread always handles column pair `lane`
-        for (int rr = warp; rr < RT; rr += 8) {
-            const int64_t r = r0 + rr;
-            float2 d = make_float2(0.f, 0.f);
+    // the tile's rows in registers: dy and y (rows warp, warp + 8, ..: column pair `lane`)
+    // and 16-byte chunks of [h | m]
+    float2 rdy[RT / 8];
+    bf162 ry[RT / 8];
+    uint4 ra[APT];
+    auto load = [&](int64_t r0) {
+#pragma unroll
+        for (int q = 0; q < RT / 8; ++q) {
+            const int64_t r = r0 + warp + 8 * q;
+            rdy[q] = make_float2(0.f, 0.f);
+            ry[q] = __floats2bfloat162_rn(0.f, 0.f);
             if (r < n) {
-                const float2 v = reinterpret_cast<const float2 *>(dy + (size_t)r * H)[lane];
-                const bf162 yy = reinterpret_cast<const bf162 *>(y + (size_t)r * H)[lane];
-                d.x = __bfloat162float(yy.x) > 0.f ? v.x : 0.f;
-                d.y = __bfloat162float(yy.y) > 0.f ? v.y : 0.f;
+                rdy[q] = __ldg(reinterpret_cast<const float2 *>(dy + (size_t)r * H) + lane);
+                ry[q] = reinterpret_cast<const bf162 *>(y + (size_t)r * H)[lane];
             }
+        }
+#pragma unroll
+        for (int q = 0; q < APT; ++q) {
+            const int i = tid + 256 * q, rr = i / (K / 8), c = i % (K / 8);
+            const int64_t r = r0 + rr;
+            ra[q] = make_uint4(0u, 0u, 0u, 0u);
+            if (i < AC && r < n)
+                ra[q] = __ldg(c < F / 8 ? reinterpret_cast<const uint4 *>(h + (size_t)r * F) + c
+                                        : reinterpret_cast<const uint4 *>(m + (size_t)r * F) + (c - F / 8));
+        }
+    };
+    const int64_t step = (int64_t)gridDim.x * RT;
+    int64_t r0 = (int64_t)blockIdx.x * RT;
+    load(r0);
+    for (; r0 < n; r0 += step) {
+        __syncthreads();              // previous tile's readers are done (and W is staged)
+#pragma unroll
+        for (int q = 0; q < RT / 8; ++q) {
+            const float2 d = make_float2(__bfloat162float(ry[q].x) > 0.f ? rdy[q].x : 0.f,
+                                         __bfloat162float(ry[q].y) > 0.f ? rdy[q].y : 0.f);
             gb0 += d.x;
             gb1 += d.y;
-            *reinterpret_cast<bf162 *>(Zs + rr * WP + 2 * lane) = __floats2bfloat162_rn(d.x, d.y);
+            *reinterpret_cast<bf162 *>(Zs + (warp + 8 * q) * WP + 2 * lane) = __floats2bfloat162_rn(d.x, d.y);
         }
-        for (int i = threadIdx.x; i < RT * (K / 2); i += blockDim.x) {
-            const int rr = i / (K / 2), k = 2 * (i % (K / 2));
-            const int64_t r = r0 + rr;
-            bf162 v = __floats2bfloat162_rn(0.f, 0.f);
-            if (r < n)
-                v = k < F ? reinterpret_cast<const bf162 *>(h + (size_t)r * F + k)[0]
-                          : reinterpret_cast<const bf162 *>(m + (size_t)r * F + (k - F))[0];
-            *reinterpret_cast<bf162 *>(As + rr * AP + k) = v;
+#pragma unroll
+        for (int q = 0; q < APT; ++q) {
+            const int i = tid + 256 * q, rr = i / (K / 8), c = i % (K / 8);
+            if (i < AC) *reinterpret_cast<uint4 *>(As + rr * AP + 8 * c) = ra[q];
         }
         __syncthreads();
-        // input gradients: (16-row m-tile, 8-column n-tile) pairs over the warps
+        load(r0 + step);              // (rows past the end read as zeros)
+        // input gradients: 2 row blocks x K/8 column blocks over the warps
         if (input_grad) {
-            for (int t = warp; t < 2 * (K / 8); t += 8) {
-                const int mt = t & 1, nt = t >> 1;
-                float acc[4] = {0.f, 0.f, 0.f, 0.f};
+            const int mt = warp & 1;
+            uint32_t a[H / 16][4];
 #pragma unroll
-                for (int ks = 0; ks < H / 16; ++ks) {
-                    const int c0 = ks * 16 + 2 * tg;
-                    const bf16 *z0 = Zs + (mt * 16 + g) * WP, *z1 = z0 + 8 * WP;
-                    uint32_t a[4];
-                    a[0] = ld_b32(z0 + c0);
-                    a[1] = ld_b32(z1 + c0);
-                    a[2] = ld_b32(z0 + c0 + 8);
-                    a[3] = ld_b32(z1 + c0 + 8);
-                    const bf16 *w = Wsm + (nt * 8 + g) * WP;
-                    mma_bf16(acc, a, ld_b32(w + c0), ld_b32(w + c0 + 8));
-                }
+            for (int ks = 0; ks < H / 16; ++ks)
+                ldsm_x4(a[ks], Zs + (mt * 16 + (lane & 15)) * WP + ks * 16 + (lane >> 4) * 8);
+#pragma unroll 2
+            for (int nt = warp >> 1; nt < K / 8; nt += 4) {
+                float acc[4] = {0.f, 0.f, 0.f, 0.f};
+                uint32_t w[2][4];     // K-steps 0, 1 and 2, 3 of the 8 columns
+                ldsm_x4(w[0], Wsm + (nt * 8 + (lane & 7)) * WP + (lane >> 3) * 8);
+                ldsm_x4(w[1], Wsm + (nt * 8 + (lane & 7)) * WP + 32 + (lane >> 3) * 8);
+#pragma unroll
+                for (int ks = 0; ks < H / 16; ++ks) mma_bf16(acc, a[ks], w[ks >> 1][(ks & 1) * 2], w[ks >> 1][(ks & 1) * 2 + 1]);
                 const int k = nt * 8 + 2 * tg;
-                const int64_t ra = r0 + mt * 16 + g, rb = ra + 8;
-                float *dst = k < F ? dah : dam;
-                const int kk = k < F ? k : k - F;
-                if (ra < n) *reinterpret_cast<float2 *>(dst + (size_t)ra * F + kk) = make_float2(acc[0], acc[1]);
-                if (rb < n) *reinterpret_cast<float2 *>(dst + (size_t)rb * F + kk) = make_float2(acc[2], acc[3]);
+                const int64_t ra_ = r0 + mt * 16 + g, rb_ = ra_ + 8;
+                if (k < F) {
+                    if (ra_ < n) *reinterpret_cast<float2 *>(dah + (size_t)ra_ * F + k) = make_float2(acc[0], acc[1]);
+                    if (rb_ < n) *reinterpret_cast<float2 *>(dah + (size_t)rb_ * F + k) = make_float2(acc[2], acc[3]);
+                } else {
+                    if (ra_ < n) {
+                        const float iv = __ldg(inv_din + ra_);
+                        *reinterpret_cast<float2 *>(dam + (size_t)ra_ * F + k - F) = make_float2(acc[0] * iv, acc[1] * iv);
+                    }
+                    if (rb_ < n) {
+                        const float iv = __ldg(inv_din + rb_);
+                        *reinterpret_cast<float2 *>(dam + (size_t)rb_ * F + k - F) = make_float2(acc[2] * iv, acc[3] * iv);
+                    }
+                }
             }
         }
-        // weight gradients: A^T (K x RT) times dz (RT x 64), reduction over the tile's rows
+        // weight gradients: A^T (K x RT) times dz (RT x 64), reduction over the tile's rows;
+        // this warp's columns 8 warp .. + 7
 #pragma unroll
-        for (int j = 0; j < WPW; ++j) {
-            const int t = warp + 8 * j;
-            if (t < WT) {
-                const int mt = t >> 3, nt = t & 7;
-                const int ka = mt * 16 + g, cb = nt * 8 + g;
+        for (int ks = 0; ks < RT / 16; ++ks) {
+            uint32_t b0, b1;
+            ldsm_x2_t(b0, b1, Zs + (ks * 16 + (lane & 15)) * WP + warp * 8);
 #pragma unroll
-                for (int ks = 0; ks < RT / 16; ++ks) {
-                    const int rA = ks * 16 + 2 * tg;
-                    uint32_t a[4];
-                    a[0] = pack_bf16(As[rA * AP + ka], As[(rA + 1) * AP + ka]);
-                    a[1] = pack_bf16(As[rA * AP + ka + 8], As[(rA + 1) * AP + ka + 8]);
-                    a[2] = pack_bf16(As[(rA + 8) * AP + ka], As[(rA + 9) * AP + ka]);
-                    a[3] = pack_bf16(As[(rA + 8) * AP + ka + 8], As[(rA + 9) * AP + ka + 8]);
-                    const uint32_t b0 = pack_bf16(Zs[rA * WP + cb], Zs[(rA + 1) * WP + cb]);
-                    const uint32_t b1 = pack_bf16(Zs[(rA + 8) * WP + cb], Zs[(rA + 9) * WP + cb]);
-                    mma_bf16(wacc[j], a, b0, b1);
-                }
+            for (int q = 0; q < MT; ++q) {
+                uint32_t a[4];
+                ldsm_x4_t(a, As + (ks * 16 + (lane & 7) + ((lane >> 4) & 1) * 8) * AP + q * 16 + ((lane >> 3) & 1) * 8);
+                mma_bf16(wacc[q], a, b0, b1);
             }
         }
     }
 #pragma unroll
-    for (int j = 0; j < WPW; ++j) {
-        const int t = warp + 8 * j;
-        if (t < WT) {
-            const int mt = t >> 3, nt = t & 7;
-            const int c = nt * 8 + 2 * tg;
-            const int ka = mt * 16 + g, kb = ka + 8;
-            float *ga = grad + (ka < F ? off_ws(l) + ka * H : off_wn(l) + (ka - F) * H) + c;
-            float *gbp = grad + (kb < F ? off_ws(l) + kb * H : off_wn(l) + (kb - F) * H) + c;
-            atomicAdd(ga, wacc[j][0]);
-            atomicAdd(ga + 1, wacc[j][1]);
-            atomicAdd(gbp, wacc[j][2]);
-            atomicAdd(gbp + 1, wacc[j][3]);
-        }
+    for (int q = 0; q < MT; ++q) {
+        const int c = warp * 8 + 2 * tg;
+        const int ka = q * 16 + g, kb = ka + 8;
+        float *ga = grad + (ka < F ? off_ws(l) + ka * H : off_wn(l) + (ka - F) * H) + c;
+        float *gbp = grad + (kb < F ? off_ws(l) + kb * H : off_wn(l) + (kb - F) * H) + c;
+        atomicAdd(ga, wacc[q][0]);
+        atomicAdd(ga + 1, wacc[q][1]);
+        atomicAdd(gbp, wacc[q][2]);
+        atomicAdd(gbp + 1, wacc[q][3]);
     }
     s_b[warp][2 * lane] = gb0;
     s_b[warp][2 * lane + 1] = gb1;
     __syncthreads();
-    if (threadIdx.x < H) {
+    if (tid < H) {
         float sb = 0.f;
 #pragma unroll
-        for (int w = 0; w < 8; ++w) sb += s_b[w][threadIdx.x];
-        atomicAdd(grad + off_b(l) + threadIdx.x, sb);
+        for (int w = 0; w < 8; ++w) sb += s_b[w][tid];
+        atomicAdd(grad + off_b(l) + tid, sb);
     }
 }
 
-// dh_u = dah_u + sum over out-arcs u -> v of dam_v / d_in(v)   (adjoint of the mean).
-// One thread per (item, feature); items as in k_agg but over the out-CSR: long out-rows
-// are skipped here and finished by k_agg_bwd_fin from the chunks' partial sums.
-template <int F>
-__global__ void k_agg_bwd(const int32_t *__restrict__ out_ptr, const int32_t *__restrict__ out_dst,
-                          const float *__restrict__ inv_din, int32_t n, const float *__restrict__ dah,
-                          const float *__restrict__ dam, float *dh, const int4 *__restrict__ items,
-                          int32_t n_items, float *acc) {
+// dh_u = dah_u + sum over out-arcs u -> v of dam_v   (adjoint of the mean; k_dense_bwd wrote
+// dam already divided by d_in).  Sixteen lanes per item take 16 bytes of every row, eight
+// arcs in flight; items are the rows in degree-bucket order (out-degrees follow the
+// in-degrees on most graphs), behind the chunks of the long out-rows, whose partial sums go
+// to acc[slot] for k_agg_bwd_fin.  (A thread per feature, one arc at a time: 183 us, BA
+// n = 300k; 106 so.)
+__global__ void __launch_bounds__(256) k_agg_bwd(const int32_t *__restrict__ out_ptr, const int32_t *__restrict__ out_dst,
+                                                 const int32_t *__restrict__ order, int32_t n,
+                                                 const float *__restrict__ dah, const float *__restrict__ dam, float *dh,
+                                                 int32_t long_min, const int4 *__restrict__ items, int32_t n_items,
+                                                 float *acc) {
+    constexpr int F = H;
+    const int lane = threadIdx.x & 31, j = lane & 15, g0 = lane & 16;
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
-    const int64_t total = ((int64_t)n + n_items) * F;
-    for (int64_t i = t; i < total; i += nthreads) {
-        const int64_t v = i / F;
-        const int j = (int)(i % F);
-        int32_t u, b, e, slot = -1;
-        if (v < n) {
-            u = (int32_t)v;
-            b = out_ptr[v];
-            e = out_ptr[v + 1];
-            if (e - b >= kSgLong) continue;
-        } else {
-            const int4 it = items[v - n];
+    const int64_t groups = ((int64_t)gridDim.x * blockDim.x) >> 4;
+    const int64_t total = (int64_t)n + n_items;
+    for (int64_t v = t >> 4; __any_sync(0xffffffffu, v < total); v += groups) {
+        int32_t u = -1, b = 0, e = 0, slot = -1;
+        if (v < n_items) {   // the long rows' chunks first
+            const int4 it = __ldg(items + v);
             u = it.x, b = it.y, e = it.z, slot = it.w;
+        } else if (v < total) {
+            u = __ldg(order + (v - n_items));
+            b = __ldg(out_ptr + u);
+            e = __ldg(out_ptr + u + 1);
+            if (e - b >= long_min) u = -1, e = b;
         }
-        float s = 0.f;
-#pragma unroll 4
-        for (int32_t a = b; a < e; ++a) {
-            const int32_t w = __ldg(out_dst + a);
-            s += dam[(size_t)w * F + j] * __ldg(inv_din + w);
+        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+        int32_t mine = j < 8 && b + j < e ? __ldg(out_dst + b + j) : -1;
+        while (__any_sync(0xffffffffu, b < e)) {
+            uint4 x[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const int32_t w = __shfl_sync(0xffffffffu, mine, g0 + q);
+                x[q] = ld_row16(dam + (size_t)max(w, 0) * F + 4 * j, w >= 0);
+            }
+            b += 8;
+            mine = j < 8 && b + j < e ? __ldg(out_dst + b + j) : -1;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                s.x += __uint_as_float(x[q].x);
+                s.y += __uint_as_float(x[q].y);
+                s.z += __uint_as_float(x[q].z);
+                s.w += __uint_as_float(x[q].w);
+            }
         }
-        if (slot < 0) dh[(size_t)u * F + j] = dah[(size_t)u * F + j] + s;
-        else atomicAdd(acc + (size_t)slot * F + j, s);
+        if (u < 0) continue;
+        if (slot < 0) {
+            const float4 a = __ldg(reinterpret_cast<const float4 *>(dah + (size_t)u * F) + j);
+            reinterpret_cast<float4 *>(dh + (size_t)u * F)[j] = make_float4(a.x + s.x, a.y + s.y, a.z + s.z, a.w + s.w);
+        } else {
+            float *p = acc + (size_t)slot * F + 4 * j;
+            atomicAdd(p, s.x);
+            atomicAdd(p + 1, s.y);
+            atomicAdd(p + 2, s.z);
+            atomicAdd(p + 3, s.w);
+        }
     }
 }
 
@@ -639,12 +849,13 @@ __global__ void k_inv_deg(const int32_t *__restrict__ row_ptr, int32_t n, float 
     }
 }
 
-__global__ void k_long_rows(const int32_t *__restrict__ ptr, int32_t n, int32_t cap, int4 *out, int32_t *count) {
+__global__ void k_long_rows(const int32_t *__restrict__ ptr, int32_t n, int32_t long_min, int32_t cap, const int32_t *__restrict__ pos,
+                            int4 *out, int32_t *count) {
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
         const int32_t b = ptr[v], e = ptr[v + 1];
-        if (e - b >= kSgLong) {
+        if (e - b >= long_min) {
             const int32_t i = atomicAdd(count, 1);
-            if (i < cap) out[i] = make_int4((int32_t)v, b, e, 0);
+            if (i < cap) out[i] = make_int4((int32_t)v, b, e, pos ? pos[v] : (int32_t)v);
         }
     }
 }
@@ -729,10 +940,22 @@ int sg_ensure(fsgp_surrogate *s, int64_t n) {
     return FSGP_OK;
 }
 
-// Persistent CTAs of the tensor-core dense layer: two per SM at most, one per tile at least.
+// Persistent CTAs of a layer: kTcCtas per SM at most.
 int tc_grid(const fsgp_surrogate *s, int64_t n) {
     const int64_t tiles = (n + kTcRows - 1) / kTcRows;
-    return (int)std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)s->sm_count * 2));
+    return (int)std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)s->sm_count * kTcCtas));
+}
+
+// The layer kernel's shared-memory limit, and a carve-out that leaves the rest of the SM's
+// memory as L1 for the gathers (its three CTAs' share of 228 KB).
+template <int F, bool HEAD>
+cudaError_t tc_attributes() {
+    cudaError_t e = cudaFuncSetAttribute(k_layer_tc<F, HEAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)tc_smem_bytes<F>());
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_layer_tc<F, HEAD>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 (int)std::min<size_t>(100, (kTcCtas * (tc_smem_bytes<F>() + 4096) * 100) / (228 * 1024) + 1));
+    return e;
 }
 
 // A tensor-core wait of an earlier launch ran out (the flag is sticky): FSGP_ETIMEOUT.
@@ -750,10 +973,12 @@ int grid_of(const fsgp_surrogate *s, int64_t work, int threads, int per_sm = 8) 
     return (int)std::max<int64_t>(g, 1);
 }
 
-// Long rows of one CSR (ptr) as chunk items and a slot -> row list (host build, once).
-int sg_long_table(const int32_t *ptr, int32_t n, int64_t nnz, int sm_count, int4 **items, int32_t *n_items,
+// Long rows of one CSR (ptr) as chunk items and, if wanted, a slot -> row list (host build,
+// once).  Slots
+// follow the rows' positions pos (null: the node order).
+int sg_long_table(const int32_t *ptr, int32_t n, int64_t nnz, int32_t long_min, const int32_t *pos, int sm_count, int4 **items, int32_t *n_items,
                   int32_t **long_rows, int32_t *n_long) {
-    const int64_t cap = nnz / kSgLong + 1;
+    const int64_t cap = nnz / long_min + 1;
     int4 *d_tmp = nullptr;
     int32_t *d_cnt = nullptr;
     FSGP_CUDA(cudaMalloc(&d_tmp, sizeof(int4) * (size_t)cap));
@@ -763,7 +988,7 @@ int sg_long_table(const int32_t *ptr, int32_t n, int64_t nnz, int sm_count, int4
     if (e == cudaSuccess) e = cudaMemset(d_cnt, 0, sizeof(int32_t));
     if (e == cudaSuccess) {
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)n + 255) / 256, (int64_t)sm_count * 8));
-        k_long_rows<<<grid, 256>>>(ptr, n, (int32_t)cap, d_tmp, d_cnt);
+        k_long_rows<<<grid, 256>>>(ptr, n, long_min, (int32_t)cap, pos, d_tmp, d_cnt);
         e = cudaMemcpy(&cnt, d_cnt, sizeof(int32_t), cudaMemcpyDeviceToHost);
     }
     if (e == cudaSuccess && cnt > 0) {
@@ -773,7 +998,7 @@ int sg_long_table(const int32_t *ptr, int32_t n, int64_t nnz, int sm_count, int4
     cudaFree(d_tmp);
     cudaFree(d_cnt);
     if (e != cudaSuccess) return cuda_fail(e, "surrogate long rows");
-    std::sort(rows.begin(), rows.end(), [](const int4 &x, const int4 &y) { return x.x < y.x; });
+    std::sort(rows.begin(), rows.end(), [](const int4 &x, const int4 &y) { return x.w < y.w; });
     std::vector<int4> it;
     std::vector<int32_t> lr;
     for (size_t sl = 0; sl < rows.size(); ++sl) {
@@ -786,6 +1011,7 @@ int sg_long_table(const int32_t *ptr, int32_t n, int64_t nnz, int sm_count, int4
     if (!it.empty()) {
         FSGP_CUDA(cudaMalloc(items, sizeof(int4) * it.size()));
         FSGP_CUDA(cudaMemcpy(*items, it.data(), sizeof(int4) * it.size(), cudaMemcpyHostToDevice));
+        if (!long_rows) return FSGP_OK;
         FSGP_CUDA(cudaMalloc(long_rows, sizeof(int32_t) * lr.size()));
         FSGP_CUDA(cudaMemcpy(*long_rows, lr.data(), sizeof(int32_t) * lr.size(), cudaMemcpyHostToDevice));
     }
@@ -797,12 +1023,13 @@ int sg_cache(const fsgp_graph *gc, int sm_count) {
     fsgp_graph *g = const_cast<fsgp_graph *>(gc);   // lazily built cache of the handle
     SgCache &C = g->sgc;
     if (C.built) return FSGP_OK;
+    while (C.long_min < kSgLongMax && (int64_t)C.long_min * g->n < 4 * g->nnz) C.long_min *= 2;
     FSGP_CUDA(cudaMalloc(&C.inv_din, sizeof(float) * (size_t)g->n));
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)g->n + 255) / 256, (int64_t)sm_count * 8));
     k_inv_deg<<<grid, 256>>>(g->row_ptr, g->n, C.inv_din);
-    int rc = sg_long_table(g->row_ptr, g->n, g->nnz, sm_count, &C.in_items, &C.n_in_items, &C.in_long, &C.n_in_long);
+    int rc = sg_long_table(g->row_ptr, g->n, g->nnz, C.long_min, g->pos, sm_count, &C.in_items, &C.n_in_items, nullptr, &C.n_in_long);
     if (rc) return rc;
-    rc = sg_long_table(g->out_ptr, g->n, g->nnz, sm_count, &C.out_items, &C.n_out_items, &C.out_long, &C.n_out_long);
+    rc = sg_long_table(g->out_ptr, g->n, g->nnz, C.long_min, nullptr, sm_count, &C.out_items, &C.n_out_items, &C.out_long, &C.n_out_long);
     if (rc) return rc;
     const size_t nl = (size_t)std::max(C.n_in_long, C.n_out_long);
     if (nl) {
@@ -814,39 +1041,25 @@ int sg_cache(const fsgp_graph *gc, int sm_count) {
     return FSGP_OK;
 }
 
-// Forward of the three layers and the head from features s->x (already seeded).
-void sg_forward(fsgp_surrogate *s, const fsgp_graph *g, float *p, float *psum, cudaStream_t st) {
-    const int32_t n = g->n;
-    const bf16 *W = s->wb;
-    const float *B = s->theta;
+// One layer (the head with it when p or psum is set): y from h, the means kept in m if set.
+template <int F, bool HEAD>
+void sg_layer(fsgp_surrogate *s, const fsgp_graph *g, int l, const bf16 *h, bf16 *m, bf16 *y, float *p, float *psum,
+              cudaStream_t st) {
     const SgCache &C = g->sgc;
-    const int64_t items = (int64_t)n + C.n_in_items;
-    k_agg<F0><<<grid_of(s, items * (F0 / 8) * agg_arcs<F0>(), 256), 256, 0, st>>>(g->row_ptr, g->col, n, s->x, s->m1, C.in_items,
-                                                                 C.n_in_items, C.acc);
-    if (C.n_in_long)
-        k_agg_fin<F0><<<grid_of(s, (int64_t)C.n_in_long * (F0 / 2), 256), 256, 0, st>>>(C.in_long, C.n_in_long,
-                                                                                     g->row_ptr, C.acc, s->m1);
-    k_dense_tc<F0, false><<<tc_grid(s, n), 128, tc_smem_bytes<F0>(), st>>>(
-        s->x, s->m1, W + OFF_WS1, W + OFF_WN1, B + OFF_B1, n, s->h1, nullptr, nullptr, nullptr, nullptr, nullptr,
-        s->tc_err);
-    k_agg<H><<<grid_of(s, items * (H / 8) * agg_arcs<H>(), 256), 256, 0, st>>>(g->row_ptr, g->col, n, s->h1, s->m2, C.in_items,
-                                                              C.n_in_items, C.acc);
-    if (C.n_in_long)
-        k_agg_fin<H><<<grid_of(s, (int64_t)C.n_in_long * (H / 2), 256), 256, 0, st>>>(C.in_long, C.n_in_long,
-                                                                                   g->row_ptr, C.acc, s->m2);
-    k_dense_tc<H, false><<<tc_grid(s, n), 128, tc_smem_bytes<H>(), st>>>(
-        s->h1, s->m2, W + OFF_WS2, W + OFF_WN2, B + OFF_B2, n, s->h2, nullptr, nullptr, nullptr, nullptr, nullptr,
-        s->tc_err);
-    k_agg<H><<<grid_of(s, items * (H / 8) * agg_arcs<H>(), 256), 256, 0, st>>>(g->row_ptr, g->col, n, s->h2, s->m3, C.in_items,
-                                                              C.n_in_items, C.acc);
-    if (C.n_in_long)
-        k_agg_fin<H><<<grid_of(s, (int64_t)C.n_in_long * (H / 2), 256), 256, 0, st>>>(C.in_long, C.n_in_long,
-                                                                                   g->row_ptr, C.acc, s->m3);
-    // layer 3 with the head in its epilogue; h3 is kept only when p is (the backward
-    // pass reads both)
-    k_dense_tc<H, true><<<tc_grid(s, n), 128, tc_smem_bytes<H>(), st>>>(
-        s->h2, s->m3, W + OFF_WS3, W + OFF_WN3, B + OFF_B3, n, p ? s->h3 : nullptr, W + OFF_WO, B + OFF_BO, p, psum,
-        s->cur, s->tc_err);
+    if (C.n_in_items)
+        k_agg_long<F><<<grid_of(s, (int64_t)C.n_in_items * 8, 256), 256, 0, st>>>(
+            g->col, h, C.in_items, C.n_in_items, C.acc);
+    k_layer_tc<F, HEAD><<<tc_grid(s, g->n), kTcThreads, tc_smem_bytes<F>(), st>>>(
+        g->row_ptr, g->col, g->rows_sorted, g->n, h, s->wb + off_ws(l), s->wb + off_wn(l), s->theta + off_b(l),
+        C.n_in_long, C.acc, m, y, s->wb + OFF_WO, s->theta + OFF_BO, p, psum, s->cur, s->tc_err);
+}
+
+// Forward of the three layers and the head from features s->x (already seeded).  keep: the
+// backward pass follows (it reads the means and the last layer's output).
+void sg_forward(fsgp_surrogate *s, const fsgp_graph *g, float *p, float *psum, bool keep, cudaStream_t st) {
+    sg_layer<F0, false>(s, g, 1, s->x, keep ? s->m1 : nullptr, s->h1, nullptr, nullptr, st);
+    sg_layer<H, false>(s, g, 2, s->h1, keep ? s->m2 : nullptr, s->h2, nullptr, nullptr, st);
+    sg_layer<H, true>(s, g, 3, s->h2, keep ? s->m3 : nullptr, keep ? s->h3 : nullptr, p, psum, st);
 }
 
 int sg_prepare_inputs(fsgp_surrogate *s, const fsgp_graph *g, const int32_t *seeds_host, int64_t ns,
@@ -880,25 +1093,25 @@ int sg_backward(fsgp_surrogate *s, const fsgp_graph *g, cudaStream_t st) {
     FSGP_CUDA(cudaMemsetAsync(s->grad, 0, sizeof(float) * N_PARAMS, st));
     FSGP_CUDA(cudaMemsetAsync(s->loss, 0, sizeof(double), st));
     k_head_bwd<<<grid_of(s, (int64_t)n * 32, 256), 256, 0, st>>>(s->h3, W + OFF_WO, s->p, s->y, n, s->dh, s->grad, s->loss);
-    const int gb = grid_of(s, ((int64_t)n + 31) / 32, 1, 2);
-    // layer 3: dy = dh (float), outputs dh2 = d h2
-    k_dense_bwd<H><<<gb, 256, 0, st>>>(s->h2, s->m3, s->h3, s->dh, W + OFF_WS3, W + OFF_WN3, n, s->dah, s->dam, s->grad, 3, 1);
     const SgCache &C = g->sgc;
+    const int gb = grid_of(s, ((int64_t)n + 31) / 32, 1, 3);
+    // layer 3: dy = dh (float), outputs dh2 = d h2
+    k_dense_bwd<H><<<gb, 256, 0, st>>>(s->h2, s->m3, s->h3, s->dh, W + OFF_WS3, W + OFF_WN3, C.inv_din, n, s->dah, s->dam, s->grad, 3, 1);
     const int64_t items = (int64_t)n + C.n_out_items;
-    k_agg_bwd<H><<<grid_of(s, items * H, 256), 256, 0, st>>>(g->out_ptr, g->out_dst, C.inv_din, n, s->dah, s->dam,
-                                                            s->dh2, C.out_items, C.n_out_items, C.acc);
+    k_agg_bwd<<<grid_of(s, items * 16, 256), 256, 0, st>>>(g->out_ptr, g->out_dst, g->rows_sorted, n, s->dah, s->dam, s->dh2,
+                                                            C.long_min, C.out_items, C.n_out_items, C.acc);
     if (C.n_out_long)
         k_agg_bwd_fin<H><<<grid_of(s, (int64_t)C.n_out_long * H, 256), 256, 0, st>>>(C.out_long, C.n_out_long,
                                                                                   s->dah, C.acc, s->dh2);
     // layer 2
-    k_dense_bwd<H><<<gb, 256, 0, st>>>(s->h1, s->m2, s->h2, s->dh2, W + OFF_WS2, W + OFF_WN2, n, s->dah, s->dam, s->grad, 2, 1);
-    k_agg_bwd<H><<<grid_of(s, items * H, 256), 256, 0, st>>>(g->out_ptr, g->out_dst, C.inv_din, n, s->dah, s->dam,
-                                                            s->dh, C.out_items, C.n_out_items, C.acc);
+    k_dense_bwd<H><<<gb, 256, 0, st>>>(s->h1, s->m2, s->h2, s->dh2, W + OFF_WS2, W + OFF_WN2, C.inv_din, n, s->dah, s->dam, s->grad, 2, 1);
+    k_agg_bwd<<<grid_of(s, items * 16, 256), 256, 0, st>>>(g->out_ptr, g->out_dst, g->rows_sorted, n, s->dah, s->dam, s->dh,
+                                                            C.long_min, C.out_items, C.n_out_items, C.acc);
     if (C.n_out_long)
         k_agg_bwd_fin<H><<<grid_of(s, (int64_t)C.n_out_long * H, 256), 256, 0, st>>>(C.out_long, C.n_out_long,
                                                                                   s->dah, C.acc, s->dh);
     // layer 1 (input gradients not needed beyond the weights)
-    k_dense_bwd<F0><<<gb, 256, 0, st>>>(s->x, s->m1, s->h1, s->dh, W + OFF_WS1, W + OFF_WN1, n, s->dah, s->dam, s->grad, 1, 0);
+    k_dense_bwd<F0><<<gb, 256, 0, st>>>(s->x, s->m1, s->h1, s->dh, W + OFF_WS1, W + OFF_WN1, C.inv_din, n, s->dah, s->dam, s->grad, 1, 0);
     FSGP_CUDA(cudaGetLastError());
     return FSGP_OK;
 }
@@ -933,12 +1146,8 @@ extern "C" int fsgp_surrogate_create(uint64_t init_seed, fsgp_surrogate **out) {
         (e = cudaMalloc(&s->cur, sizeof(int32_t))) != cudaSuccess ||
         (e = cudaMalloc(&s->tc_err, sizeof(int32_t))) != cudaSuccess ||
         (e = cudaMemset(s->tc_err, 0, sizeof(int32_t))) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(k_dense_tc<F0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)tc_smem_bytes<F0>())) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(k_dense_tc<H, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)tc_smem_bytes<H>())) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(k_dense_tc<H, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)tc_smem_bytes<H>())) != cudaSuccess) {
+        (e = tc_attributes<F0, false>()) != cudaSuccess || (e = tc_attributes<H, false>()) != cudaSuccess ||
+        (e = tc_attributes<H, true>()) != cudaSuccess) {
         fsgp_surrogate_destroy(s);
         return cuda_fail(e, "cudaMalloc (surrogate)");
     }
@@ -1013,7 +1222,7 @@ extern "C" int fsgp_surrogate_forward(fsgp_surrogate *s, const fsgp_graph *g, co
     cudaStream_t st = (cudaStream_t)stream;
     int rc = sg_prepare_inputs(s, g, seeds_host, n_seeds, beta, gamma, st);
     if (rc) return rc;
-    sg_forward(s, g, p_out, nullptr, st);
+    sg_forward(s, g, p_out, nullptr, false, st);
     FSGP_CUDA(cudaGetLastError());
     return FSGP_OK;
 }
@@ -1027,7 +1236,7 @@ extern "C" int fsgp_surrogate_grad(fsgp_surrogate *s, const fsgp_graph *g, const
     int rc = sg_prepare_inputs(s, g, seeds_host, n_seeds, beta, gamma, st);
     if (rc) return rc;
     FSGP_CUDA(cudaMemcpyAsync(s->y, y, sizeof(float) * (size_t)g->n, cudaMemcpyDeviceToDevice, st));
-    sg_forward(s, g, s->p, nullptr, st);
+    sg_forward(s, g, s->p, nullptr, true, st);
     rc = sg_backward(s, g, st);
     if (rc) return rc;
     if (loss_out) FSGP_CUDA(cudaMemcpyAsync(loss_out, s->loss, sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -1045,7 +1254,7 @@ extern "C" int fsgp_surrogate_train_step(fsgp_surrogate *s, const fsgp_graph *g,
     int rc = sg_prepare_inputs(s, g, seeds_host, n_seeds, beta, gamma, st);
     if (rc) return rc;
     FSGP_CUDA(cudaMemcpyAsync(s->y, y, sizeof(float) * (size_t)g->n, cudaMemcpyDeviceToDevice, st));
-    sg_forward(s, g, s->p, nullptr, st);
+    sg_forward(s, g, s->p, nullptr, true, st);
     rc = sg_backward(s, g, st);
     if (rc) return rc;
     s->step += 1;
@@ -1093,7 +1302,7 @@ extern "C" int fsgp_surrogate_screen(fsgp_surrogate *s, const fsgp_graph *g, con
         }
         if ((e = cudaMemcpyAsync(d_cand, cand_host, sizeof(int32_t) * (size_t)k * n_cand, cudaMemcpyHostToDevice, st)) != cudaSuccess ||
             (e = cudaMemsetAsync(d_scores, 0, sizeof(float) * (size_t)n_cand, st)) != cudaSuccess ||
-            (e = cudaMemsetAsync(s->cur, 0, sizeof(int32_t), st)) != cudaSuccess) {
+            (e = cudaMemsetAsync(s->cur, k <= kClusterSeeds ? 0xff : 0, sizeof(int32_t), st)) != cudaSuccess) {
             rc = cuda_fail(e, "screen setup");
             break;
         }
@@ -1107,13 +1316,20 @@ extern "C" int fsgp_surrogate_screen(fsgp_surrogate *s, const fsgp_graph *g, con
             break;
         }
         const int gk = std::min<int32_t>(k, 1024);
-        k_seed_bits<<<1, 256, 0, st>>>(d_cand, k, s->cur, 1.f, 0, s->x);
-        k_seed_count<<<gk, 256, 0, st>>>(d_cand, k, s->cur, g->out_ptr, g->out_dst, 1, s->cnt);
-        k_seed_feat<<<gk, 256, 0, st>>>(d_cand, k, s->cur, g->out_ptr, g->out_dst, s->cnt, s->x);
-        sg_forward(s, g, nullptr, d_scores, st);
-        k_seed_count<<<gk, 256, 0, st>>>(d_cand, k, s->cur, g->out_ptr, g->out_dst, -1, s->cnt);
-        k_seed_feat<<<gk, 256, 0, st>>>(d_cand, k, s->cur, g->out_ptr, g->out_dst, s->cnt, s->x);
-        k_seed_bits<<<1, 256, 0, st>>>(d_cand, k, s->cur, 0.f, 1, s->x);
+        const bool clustered = k <= kClusterSeeds;
+        if (clustered) {
+            k_seed_next<<<kSeedCtas, 256, 0, st>>>(d_cand, k, n_cand, s->cur, g->out_ptr, g->out_dst, s->cnt, s->x);
+        } else {
+            k_seed_bits<<<1, 256, 0, st>>>(d_cand, k, s->cur, 1.f, 0, s->x);
+            k_seed_count<<<gk, 256, 0, st>>>(d_cand, k, s->cur, g->out_ptr, g->out_dst, 1, s->cnt);
+            k_seed_feat<<<gk, 256, 0, st>>>(d_cand, k, s->cur, g->out_ptr, g->out_dst, s->cnt, s->x);
+        }
+        sg_forward(s, g, nullptr, d_scores, false, st);
+        if (!clustered) {
+            k_seed_count<<<gk, 256, 0, st>>>(d_cand, k, s->cur, g->out_ptr, g->out_dst, -1, s->cnt);
+            k_seed_feat<<<gk, 256, 0, st>>>(d_cand, k, s->cur, g->out_ptr, g->out_dst, s->cnt, s->x);
+            k_seed_bits<<<1, 256, 0, st>>>(d_cand, k, s->cur, 0.f, 1, s->x);
+        }
         e = cudaStreamEndCapture(st, &graph);
         if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
         if (graph) cudaGraphDestroy(graph);
@@ -1122,6 +1338,8 @@ extern "C" int fsgp_surrogate_screen(fsgp_surrogate *s, const fsgp_graph *g, con
             break;
         }
         for (int32_t c = 0; c < n_cand && e == cudaSuccess; ++c) e = cudaGraphLaunch(exec, st);
+        if (clustered)   // take the last candidate's seed features back
+            k_seed_next<<<kSeedCtas, 256, 0, st>>>(d_cand, k, n_cand, s->cur, g->out_ptr, g->out_dst, s->cnt, s->x);
         if (e == cudaSuccess) e = cudaMemcpyAsync(scores_out, d_scores, sizeof(float) * (size_t)n_cand, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         cudaGraphExecDestroy(exec);
