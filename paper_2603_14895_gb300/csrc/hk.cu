@@ -72,93 +72,154 @@ __global__ void __launch_bounds__(256) k_hk_out(const float *__restrict__ src, i
     }
 }
 
-constexpr int kHkUnroll = 8;   // gathered rows in flight per node
+constexpr int kHkUnroll = 8;     // gathered rows in flight per node
+constexpr int kHkStages = 4;     // blocks of rows in flight for a long row
 
-// One synchronous step.  TL lanes take the segment of 4 * TL realizations of one node; the
-// nodes come in degree-bucket order, so that the teams of a warp have rows of similar
-// length.  changes: (node, realization) pairs whose opinion changed.
+// Sixteen bytes of an in-neighbour's opinions; infinities (never within eps) without one.
+// In assembly so that a round's loads are issued one behind the other.
+__device__ __forceinline__ float4 hk_row16(const float *p, bool has) {
+    float4 r;
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %5, 0;\n mov.b32 %0, 0x7f800000;\n mov.b32 %1, 0x7f800000;\n"
+                 " mov.b32 %2, 0x7f800000;\n mov.b32 %3, 0x7f800000;\n @p ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];\n}"
+                 : "=&f"(r.x), "=&f"(r.y), "=&f"(r.z), "=&f"(r.w) : "l"(p), "r"((uint32_t)has));
+    return r;
+}
+
+// The four realizations of one lane: own opinions, running sum and count of neighbours
+// within eps, in the order the arcs are added.
+struct HkAcc {
+    float h[4], sum[4];
+    int32_t cnt[4];
+    __device__ __forceinline__ HkAcc(const float4 &own) : h{own.x, own.y, own.z, own.w}, sum{}, cnt{} {}
+    __device__ __forceinline__ void add(const float4 &o, float eps) {
+        const float x[4] = {o.x, o.y, o.z, o.w};
+#pragma unroll
+        for (int v = 0; v < 4; ++v)
+            if (fabsf(__fsub_rn(h[v], x[v])) < eps) {
+                sum[v] = __fadd_rn(sum[v], x[v]);
+                ++cnt[v];
+            }
+    }
+    // writes the new opinions, returns how many of the realizations r0 .. R-1 changed
+    __device__ __forceinline__ uint32_t store(float *p, int32_t r0, int32_t R) const {
+        float out[4];
+        uint32_t ch = 0u;
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            out[v] = cnt[v] > 0 ? __fdiv_rn(sum[v], (float)cnt[v]) : h[v];
+            if (r0 + v < R && out[v] != h[v]) ++ch;
+        }
+        *reinterpret_cast<float4 *>(p) = make_float4(out[0], out[1], out[2], out[3]);
+        return ch;
+    }
+};
+
+// One synchronous step.  changes: (node, realization) pairs whose opinion changed.
+// TL lanes take the segment of 4 * TL realizations of one node; the nodes come in
+// degree-bucket order, so that the teams of a warp have rows of similar length.
+// The first n_long * segments CTAs take one long row each: its sum has to run through all
+// arcs in order, so one team adds while the whole CTA copies the next kHkStages blocks of
+// rows to shared memory (a team on its own waits a memory latency for every eight arcs, and
+// the hub of a BA graph then outlasts the step: BA n = 1M, R = 64, a step 1.55 ms so, 0.66 with
+// the copies ahead and the padding arcs' infinities in place of their tests).
 template <int TL>
 __global__ void __launch_bounds__(256) k_hk_step(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
-                                                 const int32_t *__restrict__ order, int32_t n, int32_t R, int32_t Rp,
-                                                 float eps, const float *__restrict__ cur, float *__restrict__ nxt,
-                                                 unsigned long long *changes) {
+                                                 const int32_t *__restrict__ order, int32_t n, int32_t n_long, int32_t R,
+                                                 int32_t Rp, float eps, const float *__restrict__ cur,
+                                                 float *__restrict__ nxt, unsigned long long *changes) {
     constexpr int TPW = 32 / TL;
-    const int lane = threadIdx.x & 31, tl = lane % TL, g0 = lane - tl;
+    constexpr int RPS = 256 / TL;       // rows of a block
+    __shared__ float4 s_row[kHkStages][256];
+    const int tid = threadIdx.x, lane = tid & 31, tl = lane % TL, g0 = lane - tl;
     const int segs = Rp / (4 * TL);     // segments of a node's row
-    const int64_t items = (int64_t)n * segs;
-    const int64_t team = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * TPW + lane / TL;
-    const int64_t nteams = (((int64_t)gridDim.x * blockDim.x) >> 5) * TPW;
+    const int64_t long_items = (int64_t)n_long * segs;
     unsigned long long ch = 0ull;
-    // node, segment and arcs of the team's next item
-    int32_t i = -1, seg = 0, beg = 0, end = 0;
-    auto fetch = [&](int64_t it) {
-        i = -1;
-        beg = end = 0;
-        if (it < items) {
-            const int64_t q = segs == 1 ? it : it / segs;
-            seg = (int32_t)(it - q * segs);
-            i = __ldg(order + q);
-            beg = __ldg(row_ptr + i);
-            end = __ldg(row_ptr + i + 1);
-        }
-    };
-    fetch(team);
-    // the whole warp iterates together (the column indices are handed out by shuffles)
-    for (int64_t it = team; __any_sync(0xffffffffu, i >= 0); it += nteams) {
-        const int32_t node = i, b = beg, e = end;
-        const float *base = cur + (seg * TL + tl) * 4;
-        const size_t own = (size_t)(node < 0 ? 0 : node) * Rp;
-        const int32_t r0 = (seg * TL + tl) * 4;
-        int32_t mine = tl < kHkUnroll && b + tl < e ? __ldg(col + b + tl) : -1;
-        float4 h = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (node >= 0) h = __ldg(reinterpret_cast<const float4 *>(base + own));
-        fetch(it + nteams);
-        const float hi[4] = {h.x, h.y, h.z, h.w};
-        float sum[4] = {0.f, 0.f, 0.f, 0.f};
-        int32_t cnt[4] = {0, 0, 0, 0};
-        for (int32_t a = b; __any_sync(0xffffffffu, a < e); a += kHkUnroll) {
-            float4 hj[kHkUnroll];
-            unsigned has = 0u;
+    if ((int64_t)blockIdx.x < long_items) {
+        const int32_t q = (int32_t)(blockIdx.x / segs), seg = (int32_t)blockIdx.x - q * segs;
+        const int32_t node = __ldg(order + q), b = __ldg(row_ptr + node), e = __ldg(row_ptr + node + 1);
+        const int t = tid % TL;         // this thread's 16 bytes of row tid / TL of a block
+        const float *base = cur + (seg * TL + t) * 4;
+        const int32_t r0 = (seg * TL + t) * 4;
+        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&s_row[0][tid]);
+        const int32_t blocks = (e - b + RPS - 1) / RPS;
+        auto col_of = [&](int32_t k) { return b + k * RPS + tid / TL < e ? __ldg(col + b + k * RPS + tid / TL) : -1; };
+        int32_t c = col_of(0);
+        auto copy = [&](int32_t k) {    // block k, whose column index is in c; c of the next
+            if (c >= 0)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + (uint32_t)(k % kHkStages) * 4096u),
+                             "l"(base + (size_t)c * Rp));
+            asm volatile("cp.async.commit_group;");
+            c = col_of(k + 1);
+        };
+        for (int32_t k = 0; k < kHkStages - 1; ++k) copy(k);
+        HkAcc acc(__ldg(reinterpret_cast<const float4 *>(base + (size_t)node * Rp)));
+        for (int32_t k = 0; k < blocks; ++k) {
+            asm volatile("cp.async.wait_group %0;" ::"n"(kHkStages - 2));
+            __syncthreads();            // block k has landed; block k - 1 has been added
+            copy(k + kHkStages - 1);
+            if (tid < TL) {
+                const float4 *x = s_row[k % kHkStages] + t;
+                const int m = min(RPS, e - b - k * RPS);
+                if (m == RPS) {
 #pragma unroll
-            for (int u = 0; u < kHkUnroll; ++u) {
-                const int32_t j = __shfl_sync(0xffffffffu, mine, g0 + u);
-                if (j >= 0) {
-                    hj[u] = __ldg(reinterpret_cast<const float4 *>(base + (size_t)j * Rp));
-                    has |= 1u << u;
-                }
-            }
-            const int32_t an = a + kHkUnroll + tl;
-            mine = tl < kHkUnroll && an < e ? __ldg(col + an) : -1;
-#pragma unroll
-            for (int u = 0; u < kHkUnroll; ++u) {
-                const float x[4] = {hj[u].x, hj[u].y, hj[u].z, hj[u].w};
-#pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    if ((has >> u & 1u) && fabsf(__fsub_rn(hi[v], x[v])) < eps) {
-                        sum[v] = __fadd_rn(sum[v], x[v]);
-                        ++cnt[v];
-                    }
+                    for (int u = 0; u < RPS; ++u) acc.add(x[u * TL], eps);
+                } else {
+                    for (int u = 0; u < m; ++u) acc.add(x[u * TL], eps);
                 }
             }
         }
-        if (node >= 0) {
-            float out[4];
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                out[v] = cnt[v] > 0 ? __fdiv_rn(sum[v], (float)cnt[v]) : hi[v];
-                if (r0 + v < R && out[v] != hi[v]) ++ch;
+        asm volatile("cp.async.wait_group 0;");
+        if (tid < TL) ch = acc.store(nxt + (size_t)node * Rp + r0, r0, R);
+    } else {
+        const int64_t items = (int64_t)n * segs;
+        const int64_t team = ((((int64_t)blockIdx.x - long_items) * blockDim.x + tid) >> 5) * TPW + lane / TL + long_items;
+        const int64_t nteams = ((((int64_t)gridDim.x - long_items) * blockDim.x) >> 5) * TPW;
+        // node, segment and arcs of the team's next item
+        int32_t i = -1, seg = 0, beg = 0, end = 0;
+        auto fetch = [&](int64_t it) {
+            i = -1;
+            beg = end = 0;
+            if (it < items) {
+                const int64_t q = segs == 1 ? it : it / segs;
+                seg = (int32_t)(it - q * segs);
+                i = __ldg(order + q);
+                beg = __ldg(row_ptr + i);
+                end = __ldg(row_ptr + i + 1);
             }
-            *reinterpret_cast<float4 *>(nxt + own + r0) = make_float4(out[0], out[1], out[2], out[3]);
+        };
+        fetch(team);
+        // the whole warp iterates together (the column indices are handed out by shuffles)
+        for (int64_t it = team; __any_sync(0xffffffffu, i >= 0); it += nteams) {
+            const int32_t node = i, e = end, r0 = (seg * TL + tl) * 4;
+            int32_t b = beg;
+            const float *base = cur + r0;
+            const size_t own = (size_t)max(node, 0) * Rp;
+            int32_t mine = tl < kHkUnroll && b + tl < e ? __ldg(col + b + tl) : -1;
+            HkAcc acc(hk_row16(base + own, node >= 0));
+            fetch(it + nteams);
+            while (__any_sync(0xffffffffu, b < e)) {
+                float4 x[kHkUnroll];
+#pragma unroll
+                for (int u = 0; u < kHkUnroll; ++u) {
+                    const int32_t j = __shfl_sync(0xffffffffu, mine, g0 + u);
+                    x[u] = hk_row16(base + (size_t)max(j, 0) * Rp, j >= 0);
+                }
+                b += kHkUnroll;
+                mine = tl < kHkUnroll && b + tl < e ? __ldg(col + b + tl) : -1;
+#pragma unroll
+                for (int u = 0; u < kHkUnroll; ++u) acc.add(x[u], eps);
+            }
+            if (node >= 0) ch += acc.store(nxt + own + r0, r0, R);
         }
     }
     __shared__ unsigned long long s_ch;
-    if (threadIdx.x == 0) s_ch = 0ull;
+    if (tid == 0) s_ch = 0ull;
     __syncthreads();
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) ch += __shfl_xor_sync(0xffffffffu, ch, o);
     if (lane == 0 && ch) atomicAdd(&s_ch, ch);
     __syncthreads();
-    if (threadIdx.x == 0 && s_ch) atomicAdd(changes, s_ch);
+    if (tid == 0 && s_ch) atomicAdd(changes, s_ch);
 }
 
 }  // namespace
@@ -221,16 +282,22 @@ extern "C" int fsgp_hk(const fsgp_graph *gc, const float *h0, int32_t R, int32_t
     // lanes per node: as wide a segment as divides the row (the column indices are loaded
     // once per segment)
     const int TL = Rp % 128 == 0 ? 32 : (Rp % 64 == 0 ? 16 : 8);
-    const int64_t teams = (int64_t)n * (Rp / (4 * TL));
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((teams * TL + 255) / 256, (int64_t)g->sm_count * 8));
+    const int segs = Rp / (4 * TL);
+    // long rows: at least 256 in-arcs and sixteen times the mean, a power of two, so that they
+    // are the first of the degree-bucket order
+    int lb = 8;
+    while (lb < 31 && ((int64_t)n << lb) < 16 * g->nnz) ++lb;
+    const int32_t n_long = g->cls.bucket_start[lb];
+    const int64_t teams = (int64_t)(n - n_long) * segs;
+    const int grid = (int)(std::min<int64_t>((teams * TL + 255) / 256, (int64_t)g->sm_count * 8) + (int64_t)n_long * segs);
     float *cur = buf0, *nxt = buf1;
     for (int32_t k = 1; k <= T && n > 0; ++k) {
         if (TL == 32)
-            k_hk_step<32><<<grid, 256, 0, s>>>(g->row_ptr, g->col, g->rows_sorted, n, R, Rp, eps_f, cur, nxt, d_ch + k);
+            k_hk_step<32><<<grid, 256, 0, s>>>(g->row_ptr, g->col, g->rows_sorted, n, n_long, R, Rp, eps_f, cur, nxt, d_ch + k);
         else if (TL == 16)
-            k_hk_step<16><<<grid, 256, 0, s>>>(g->row_ptr, g->col, g->rows_sorted, n, R, Rp, eps_f, cur, nxt, d_ch + k);
+            k_hk_step<16><<<grid, 256, 0, s>>>(g->row_ptr, g->col, g->rows_sorted, n, n_long, R, Rp, eps_f, cur, nxt, d_ch + k);
         else
-            k_hk_step<8><<<grid, 256, 0, s>>>(g->row_ptr, g->col, g->rows_sorted, n, R, Rp, eps_f, cur, nxt, d_ch + k);
+            k_hk_step<8><<<grid, 256, 0, s>>>(g->row_ptr, g->col, g->rows_sorted, n, n_long, R, Rp, eps_f, cur, nxt, d_ch + k);
         std::swap(cur, nxt);
     }
     FSGP_CUDA(cudaGetLastError());
