@@ -288,9 +288,11 @@ __device__ __forceinline__ uint32_t pick(const uint32_t (&c)[V][B], int i, int b
 }
 
 // Resident CTAs per SM the register allocation is bounded for: wider thread words hold
-// more counters, narrower ones run more warps to keep more loads in flight.
+// more counters.  Three with two words per thread: a fourth leaves 64 registers, which spill
+// in the gather (R-MAT n = 8M, R = 256, a SIS step: team rows 602 us with four, 541 with
+// three, 669 with five; warp rows 333 with three, 377 with two, 586 with four).
 template <int V, bool WIDE>
-constexpr int min_ctas() { return V == 4 ? 2 : (V == 2 ? (WIDE ? 3 : 4) : 4); }
+constexpr int min_ctas() { return V == 4 ? 2 : (V == 2 ? 3 : 4); }
 
 // Row kernel: one work item is one slice (TEAM*V words) of one row.
 // WARP_ROW = false: one team per item; true: one warp per item.
@@ -617,6 +619,10 @@ __device__ __forceinline__ void draw_counts(const StepArgs &A, TileT &T, int n, 
         uint32_t tied = 0u, won = 0u;
         auto tie_fn = [&](uint32_t lanes, uint32_t th) {
             tied |= lanes;
+            if (LT && (th & 0xffffffu) == 0u) {   // T's other bits are all ones: every tied u is <= T
+                won |= lanes;
+                return;
+            }
             const int at = atomicAdd(&T.ties, 1);
             if (at < TileT::kTies) {
                 T.tie_slot[at] = (uint16_t)slot;
@@ -1841,7 +1847,7 @@ constexpr size_t kLaneSmem = ModelTraits<MODEL>::tiled ? LaneShape<MODEL, SWL>::
                                                        : sizeof(LaneStage<SWL, ModelTraits<MODEL>::planes>);
 
 template <int MODEL, int SWL>
-__global__ void __launch_bounds__(kBlock, ModelTraits<MODEL>::tiled ? 4 : 1) k_rows_lane(StepArgs A) {
+__global__ void __launch_bounds__(kBlock, ModelTraits<MODEL>::tiled ? 3 : 1) k_rows_lane(StepArgs A) {
     extern __shared__ __align__(16) uint8_t s_dyn[];
     __shared__ unsigned long long s_pc[kPC * kMaxSets];
     int32_t *s_lane = reinterpret_cast<int32_t *>(s_dyn + kLaneSmem<MODEL, SWL>);

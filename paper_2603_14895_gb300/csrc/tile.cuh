@@ -74,9 +74,10 @@ __device__ __forceinline__ uint32_t less_from(uint32_t eq, uint32_t th, uint32_t
     return lt;
 }
 
-// The threshold of a lane with count k, below which its uniform must lie, and its top eight
-// bits as masks: the survival table (a lane at or above it is infected), or the linear
-// threshold's floor(k * 2^32 / d) + 1, which is below 2^32 for k < d.
+// The threshold of a lane with count k < 2^24, below which its uniform must lie, and eight
+// bits as masks that decide every uniform whose own top eight bits differ from them: the
+// survival table (a lane at or above it is infected), or the linear threshold's
+// floor(k * 2^32 / d) + 1, which is below 2^32 for k < d.
 template <bool TABLE>   // masks from the table (counts up to 255)
 struct SurvThr {
     const uint64_t *surv;
@@ -88,11 +89,13 @@ struct SurvThr {
         else return masks_of((*this)(k) >> 24);
     }
 };
+// (u < floor(k * 2^32 / d) + 1 is u <= T, T = floor(k * 2^32 / d), whose top eight bits are
+// floor(256 k / d): the 64-bit division is left to the ties.)
 struct LtThr {
     uint32_t d;
     static constexpr bool falls = false;
     __device__ __forceinline__ uint32_t operator()(uint32_t k) const { return (uint32_t)(((uint64_t)k << 32) / d) + 1u; }
-    __device__ __forceinline__ Masks8 masks(uint32_t k) const { return masks_of((*this)(k) >> 24); }
+    __device__ __forceinline__ Masks8 masks(uint32_t k) const { return masks_of((k << 8) / d); }
 };
 
 // P: the top eight planes of the lanes' uniforms.
