@@ -240,7 +240,7 @@ __device__ __forceinline__ void gather_counts(const StepArgs &A, int64_t first, 
 // gather_counts.
 // Draws are keyed by the arc's position in the caller's column array: arc e of the
 // relabelled array is caller arc e + arcb.
-template <int MODEL, int V, bool CG = false>
+template <int MODEL, int V>
 __device__ __forceinline__ void gather_arcs(const StepArgs &A, int64_t e_begin, int64_t e_end,
                                             int64_t step, int64_t arcb, int w0, const uint32_t (&need)[V],
                                             const uint64_t (&ic_thr)[V], const WordCtx (&x)[V],
@@ -255,7 +255,7 @@ __device__ __forceinline__ void gather_arcs(const StepArgs &A, int64_t e_begin, 
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             xs[j] = Vec<V>{};
-            if (u[j] >= 0) xs[j] = ld_vec<V, CG>(src + (size_t)u[j] * Wn);
+            if (u[j] >= 0) xs[j] = ldg_vec<V>(src + (size_t)u[j] * Wn);
         }
         const int64_t en = e + step;
 #pragma unroll
@@ -294,7 +294,9 @@ __device__ __forceinline__ uint32_t pick(const uint32_t (&c)[V][B], int i, int b
 template <int V, bool WIDE>
 constexpr int min_ctas() { return V == 4 ? 2 : (V == 2 ? 3 : 4); }
 
-// Row kernel: one work item is one slice (TEAM*V words) of one row.
+// Row kernel that decides every word in the thread that gathered it (count models; SWIR,
+// whose second draw depends on its first): one work item is one slice (TEAM*V words) of one
+// row.
 // WARP_ROW = false: one team per item; true: one warp per item.
 // BT: counter bits of a team kernel, sized to its rows' in-degree bound (fewer planes =
 // fewer registers and cheaper counting and grouping).
@@ -302,13 +304,11 @@ constexpr int min_ctas() { return V == 4 ? 2 : (V == 2 ? 3 : 4); }
 // step), 1 = mid rows, 3 = rows with 4..15 in-arcs (dense steps only).
 // CG: the state planes are read through L2 only (the persistent step loop, which reads
 // in one launch the planes that other CTAs wrote at the previous step).
-// AG (team rows only): each row is taken by AG teams that split its arcs (every AG-th
-// group of 4 arcs) and merge their counts by shuffles; the first team decides.  Shorter
-// per-thread chains for small graphs, whose steps are bound by the longest chain.
-template <int MODEL, int V, int TEAM, bool WARP_ROW, int BT, bool CG, int AG = 1>
+// bid of nb: the CTA's place among those that work on these rows.
+template <int MODEL, int V, int TEAM, bool WARP_ROW, int BT, bool CG>
 __device__ __forceinline__ void rows_body(const StepArgs &A, int which, int32_t *s_lane, unsigned long long *s_pc,
                                           int bid, int nb) {
-    static_assert(AG == 1 || (!WARP_ROW && TEAM * AG <= 32), "arc groups: team rows within a warp");
+    static_assert(ModelTraits<MODEL>::counts, "arc models go through the warp tile");
     constexpr int B = WARP_ROW ? kWideBits : BT;
     constexpr int TPW = 32 / TEAM;
     constexpr int SW = TEAM * V;
@@ -339,8 +339,7 @@ __device__ __forceinline__ void rows_body(const StepArgs &A, int which, int32_t 
     const int tl = lane % TEAM;
     const int64_t gwarp = ((int64_t)bid * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)nb * blockDim.x) >> 5;
-    constexpr int RPI = WARP_ROW ? 1 : TPW / AG;
-    const int grp = team % AG;          // arc group of the row (AG > 1)
+    constexpr int RPI = WARP_ROW ? 1 : TPW;
     const int list_slot = A.k & 1;
     const int64_t nitems = nrows * A.nslices;
     Accum acc;
@@ -354,7 +353,7 @@ __device__ __forceinline__ void rows_body(const StepArgs &A, int which, int32_t 
     for (int i = 0; i < V; ++i) d0[i] = d1[i] = d2[i] = 0;
 
     for (int64_t base = gwarp * RPI; base < nitems; base += nwarps * RPI) {
-        const int64_t item = WARP_ROW ? base : base + team / AG;
+        const int64_t item = WARP_ROW ? base : base + team;
         const bool has_row = item < nitems;
         const int64_t ridx = has_row ? div_slices(item, A.nslices, nitems) : 0;
         const int slice = has_row ? (int)(item - ridx * A.nslices) : 0;
@@ -391,33 +390,19 @@ __device__ __forceinline__ void rows_body(const StepArgs &A, int which, int32_t 
         for (int o = 1; o < TEAM; o <<= 1) any_need |= __shfl_xor_sync(0xffffffffu, any_need, o);
 
         uint32_t c[V][B];
-        uint32_t newly[V];
 #pragma unroll
-        for (int i = 0; i < V; ++i) {
-            newly[i] = 0u;
+        for (int i = 0; i < V; ++i)
 #pragma unroll
             for (int b = 0; b < B; ++b) c[i][b] = 0u;
-        }
         int32_t beg = 0, end = 0;
         if (has_row) {
             beg = __ldg(A.rp + v);
             end = __ldg(A.rp + v + 1);
         }
-        if constexpr (ModelTraits<MODEL>::counts) {
-            constexpr int parts = WARP_ROW ? TPW : AG;   // teams that share a row
-            gather_counts<MODEL, V, B, TEAM, parts, CG>(A, beg, any_need ? end - beg : 0, 8 * parts, w0, lane, c);
-        } else if (any_need) {
-            uint64_t ic_thr[V];
-            const int64_t arcb = (int64_t)__ldg(A.arc0 + v) - beg;
-#pragma unroll
-            for (int i = 0; i < V; ++i) ic_thr[i] = ic_threshold(A, x[i].s, end - beg);
-            // teams that share a row take every TPW-th (AG-th) group of its arcs
-            const int part = WARP_ROW ? team : grp;
-            constexpr int parts = WARP_ROW ? TPW : AG;
-            gather_arcs<MODEL, V, CG>(A, (int64_t)beg + 4 * part, end, 4 * parts, arcb, w0, need, ic_thr, x, newly);
-        }
+        constexpr int parts = WARP_ROW ? TPW : 1;   // teams that share a row
+        gather_counts<MODEL, V, B, TEAM, parts, CG>(A, beg, any_need ? end - beg : 0, 8 * parts, w0, lane, c);
         constexpr bool SPLIT = WARP_ROW && TPW >= V;   // enough teams to give each word one
-        if constexpr (SPLIT && V == 2 && ModelTraits<MODEL>::counts) {
+        if constexpr (SPLIT && V == 2) {
             // merge the teams' counters, reduce-scatter first: at the first butterfly level
             // the partners (teams 2j, 2j+1) swap halves and keep word (team & 1) each, so
             // the remaining levels add one word instead of two; team i < 2 ends up with
@@ -437,20 +422,16 @@ __device__ __forceinline__ void rows_body(const StepArgs &A, int which, int32_t 
             }
 #pragma unroll
             for (int b = 0; b < B; ++b) c[1][b] = c[0][b];
-        } else if (WARP_ROW || AG > 1) {
+        } else if constexpr (WARP_ROW) {
             // merge the teams' partial results (the warp is converged here)
 #pragma unroll
-            for (int o = TEAM; o < (WARP_ROW ? 32 : TEAM * AG); o <<= 1) {
+            for (int o = TEAM; o < 32; o <<= 1) {
 #pragma unroll
                 for (int i = 0; i < V; ++i) {
-                    if constexpr (ModelTraits<MODEL>::counts) {
-                        uint32_t d[B];
+                    uint32_t d[B];
 #pragma unroll
-                        for (int b = 0; b < B; ++b) d[b] = __shfl_xor_sync(0xffffffffu, c[i][b], o);
-                        add_sliced<B>(c[i], d);
-                    } else {
-                        newly[i] |= __shfl_xor_sync(0xffffffffu, newly[i], o);
-                    }
+                    for (int b = 0; b < B; ++b) d[b] = __shfl_xor_sync(0xffffffffu, c[i][b], o);
+                    add_sliced<B>(c[i], d);
                 }
             }
         }
@@ -467,18 +448,13 @@ __device__ __forceinline__ void rows_body(const StepArgs &A, int which, int32_t 
 #pragma unroll
                 for (int b = 0; b < B; ++b) cw[b] = pick<V, B>(c, i, b);
                 WordCtx xw = x[0];
-                uint32_t nw = newly[0];
 #pragma unroll
-                for (int q = 1; q < V; ++q) {
-                    if (i == q) {
-                        xw = x[q];
-                        nw = newly[q];
-                    }
-                }
+                for (int q = 1; q < V; ++q)
+                    if (i == q) xw = x[q];
                 const uint32_t s0 = ld_word<CG>(A.cur + off + i);
                 const uint32_t s1 = P >= 2 ? ld_word<CG>(A.cur + A.plane_words + off + i) : 0u;
                 const uint32_t s2 = P >= 3 ? ld_word<CG>(A.cur + 2 * A.plane_words + off + i) : 0u;
-                const WordOut o = update_word<MODEL, B>(A, node, xw, s0, s1, s2, end - beg, cw, nw);
+                const WordOut o = update_word<MODEL, B>(A, node, xw, s0, s1, s2, end - beg, cw, 0u);
                 A.nxt[off + i] = o.n0;
                 if (P >= 2) A.nxt[A.plane_words + off + i] = o.n1;
                 if (P >= 3) A.nxt[2 * A.plane_words + off + i] = o.n2;
@@ -501,7 +477,7 @@ __device__ __forceinline__ void rows_body(const StepArgs &A, int which, int32_t 
             for (int o = 1; o < 32; o <<= 1) fl |= __shfl_xor_sync(0xffffffffu, fl, o);
             writer = has_row && team == 0;
         } else {
-        writer = has_row && (WARP_ROW ? team == 0 : grp == 0);
+        writer = has_row && (!WARP_ROW || team == 0);
         if (writer) {
             // own state again (L1/L2-resident): not kept live across the gather
             uint32_t s0[V], s1[V], s2[V];
@@ -520,7 +496,7 @@ __device__ __forceinline__ void rows_body(const StepArgs &A, int which, int32_t 
             uint32_t n0[V], n1[V], n2[V];
 #pragma unroll
             for (int i = 0; i < V; ++i) {
-                const WordOut o = update_word<MODEL, B>(A, node, x[i], s0[i], s1[i], s2[i], end - beg, c[i], newly[i]);
+                const WordOut o = update_word<MODEL, B>(A, node, x[i], s0[i], s1[i], s2[i], end - beg, c[i], 0u);
                 n0[i] = o.n0;
                 n1[i] = o.n1;
                 n2[i] = o.n2;
@@ -1105,12 +1081,12 @@ __device__ __forceinline__ void rows_tile(const StepArgs &A, int which, uint8_t 
     if (lanes_on) flush_lanes(A, s_lane, nl);
 }
 
-// The rows of one class: through the warp tile, or in place (SWIR; AG as in rows_body).
-template <int MODEL, int V, int TEAM, bool WARP_ROW, int BT, bool CG, int AG = 1>
+// The rows of one class: through the warp tile, or in place (SWIR).
+template <int MODEL, int V, int TEAM, bool WARP_ROW, int BT, bool CG>
 __device__ __forceinline__ void rows_class(const StepArgs &A, int which, uint8_t *smem, int32_t *s_lane,
                                            unsigned long long *s_pc, int bid, int nb) {
     if constexpr (ModelTraits<MODEL>::tiled) rows_tile<MODEL, V, TEAM, WARP_ROW, BT, CG>(A, which, smem, s_lane, s_pc, bid, nb);
-    else rows_body<MODEL, V, TEAM, WARP_ROW, BT, CG, AG>(A, which, s_lane, s_pc, bid, nb);
+    else rows_body<MODEL, V, TEAM, WARP_ROW, BT, CG>(A, which, s_lane, s_pc, bid, nb);
 }
 
 // Dynamic shared memory of a class's tiles, and of either class's (fused kernels).

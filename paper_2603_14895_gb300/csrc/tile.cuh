@@ -9,9 +9,9 @@
 // blocks at every word (17 to 23 of 32 threads active per instruction, measured on R-MAT,
 // SIS, R = 256); the queues keep the threads full, because a thread works on an item that
 // has something to draw, and items that need more blocks are packed again before the next
-// one.  Against deciding in place, with the counters and gathers of rows.cuh as they are now:
-// SIR on R-MAT n = 16.8M, R = 256, T = 100: 282 to 209 ms; SIS on n = 8M: 257 to 178 ms;
-// weighted SIR on n = 4.2M: 153 to 120 ms; batch of 32 mixed requests: 278 to 126 ms.
+// one.  Deciding in place before, and now, with the counters and gathers of rows.cuh: SIR on
+// R-MAT n = 16.8M, R = 256, T = 100: 283 to 201 ms; SIS on n = 8M: 257 to 167 ms; weighted
+// SIR on n = 4.2M: 154 to 113 ms; batch of 32 mixed requests: 281 to 96 ms.
 #pragma once
 
 #include "step.cuh"
