@@ -117,6 +117,7 @@ struct HkAcc {
 // One synchronous step.  changes: (node, realization) pairs whose opinion changed.
 // TL lanes take the segment of 4 * TL realizations of one node; the nodes come in
 // degree-bucket order, so that the teams of a warp have rows of similar length.
+// order may be null (node order) when there are no long rows.
 // The first n_long * segments CTAs take one long row each: its sum has to run through all
 // arcs in order, so one team adds while the whole CTA copies the next kHkStages blocks of
 // rows to shared memory (a team on its own waits a memory latency for every eight arcs, and
@@ -182,7 +183,7 @@ __global__ void __launch_bounds__(256) k_hk_step(const int32_t *__restrict__ row
             if (it < items) {
                 const int64_t q = segs == 1 ? it : it / segs;
                 seg = (int32_t)(it - q * segs);
-                i = __ldg(order + q);
+                i = order ? __ldg(order + q) : (int32_t)q;
                 beg = __ldg(row_ptr + i);
                 end = __ldg(row_ptr + i + 1);
             }
@@ -284,20 +285,26 @@ extern "C" int fsgp_hk(const fsgp_graph *gc, const float *h0, int32_t R, int32_t
     const int TL = Rp % 128 == 0 ? 32 : (Rp % 64 == 0 ? 16 : 8);
     const int segs = Rp / (4 * TL);
     // long rows: at least 256 in-arcs and sixteen times the mean, a power of two, so that they
-    // are the first of the degree-bucket order
+    // are the first of the degree-bucket order; from 32 arcs and four times the mean where four
+    // CTAs per SM hold them all, since a small graph's step lasts as long as its longest row
     int lb = 8;
     while (lb < 31 && ((int64_t)n << lb) < 16 * g->nnz) ++lb;
+    for (int b = 5; b < lb; ++b)
+        if (((int64_t)n << b) >= 4 * g->nnz && (int64_t)g->cls.bucket_start[b] * segs <= (int64_t)g->sm_count * 4) lb = b;
     const int32_t n_long = g->cls.bucket_start[lb];
     const int64_t teams = (int64_t)(n - n_long) * segs;
     const int grid = (int)(std::min<int64_t>((teams * TL + 255) / 256, (int64_t)g->sm_count * 8) + (int64_t)n_long * segs);
+    // (where every team has one row at most and none is long, the order gains nothing and is
+    // one more load in the step's chain)
+    const int32_t *order = n_long == 0 && teams * TL <= (int64_t)g->sm_count * 8 * 256 ? nullptr : g->rows_sorted;
     float *cur = buf0, *nxt = buf1;
     for (int32_t k = 1; k <= T && n > 0; ++k) {
         if (TL == 32)
-            k_hk_step<32><<<grid, 256, 0, s>>>(g->row_ptr, g->col, g->rows_sorted, n, n_long, R, Rp, eps_f, cur, nxt, d_ch + k);
+            k_hk_step<32><<<grid, 256, 0, s>>>(g->row_ptr, g->col, order, n, n_long, R, Rp, eps_f, cur, nxt, d_ch + k);
         else if (TL == 16)
-            k_hk_step<16><<<grid, 256, 0, s>>>(g->row_ptr, g->col, g->rows_sorted, n, n_long, R, Rp, eps_f, cur, nxt, d_ch + k);
+            k_hk_step<16><<<grid, 256, 0, s>>>(g->row_ptr, g->col, order, n, n_long, R, Rp, eps_f, cur, nxt, d_ch + k);
         else
-            k_hk_step<8><<<grid, 256, 0, s>>>(g->row_ptr, g->col, g->rows_sorted, n, n_long, R, Rp, eps_f, cur, nxt, d_ch + k);
+            k_hk_step<8><<<grid, 256, 0, s>>>(g->row_ptr, g->col, order, n, n_long, R, Rp, eps_f, cur, nxt, d_ch + k);
         std::swap(cur, nxt);
     }
     FSGP_CUDA(cudaGetLastError());

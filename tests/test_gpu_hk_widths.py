@@ -32,3 +32,21 @@ def test_widths(cuda_lib, R, n):
     bad[R - 1, n - 1] = float("nan")
     with pytest.raises(cuda_lib.FsgpError):
         cuda_lib.hk(graph, bad, 1, 0.4)
+
+
+@pytest.mark.parametrize("longest", [17, 31, 32, 33, 65, 255])
+@pytest.mark.parametrize("R", [32, 64, 128])
+def test_long_rows(cuda_lib, R, longest):
+    # rows on both sides of the bound for a CTA of their own, and graphs without such rows
+    n = 700
+    rng = np.random.default_rng(longest * R)
+    d = rng.choice([0, 1, 2, 7], size=n)
+    d[[3, 350, n - 1]] = longest
+    row_ptr = np.zeros(n + 1, dtype=np.int32)
+    row_ptr[1:] = np.cumsum(d)
+    col = rng.integers(0, n, size=int(row_ptr[-1])).astype(np.int32)
+    h0 = rng.uniform(-1, 1, size=(R, n)).astype(np.float32)
+    want, changes = O.hk(row_ptr, col, h0, T=4, eps=0.4)
+    h, ch = cuda_lib.hk(cuda_lib.Graph(row_ptr, col), h0, 4, 0.4)
+    assert np.array_equal(h.view(np.uint32), want.view(np.uint32))
+    assert np.array_equal(ch.astype(np.uint64), changes)
