@@ -540,16 +540,20 @@ static int run_wave(fsgp_graph *g, int model, int ic_mode, int weighted, const S
     // Words per thread (w: words a team covers with one word per thread).  Large graphs: 2,
     // and 4 for rows of 16 words and more, whose teams are then at most 8 threads wide and
     // spend less per arc (BA n = 1M, IC, R = 1024: 50.8 against 39.0 ms; R-MAT, SIS, R = 256:
-    // 178 against 179 ms).  Small graphs whose rows all get a warp at once are bound by the
-    // longest chain and take 1; the others as many as keep a team within 8 threads (BA
-    // n = 18k, SIS, R = 1010: 2.96 ms with 1, 1.38 with 2, 1.48 with 4; BA n = 20k, SIR,
-    // R = 1000: 6.4, 4.7, 4.4; BA n = 250k, SEIR, R = 100: 8.7, 9.0, 13.5).
+    // 178 against 179 ms).  Small graphs whose rows all get a warp in one or two rounds, none
+    // with hundreds of arcs, are bound by the chain of a row and the barrier and take 1, and
+    // with it the persistent loop (BA n = 6434, LT, R = 152, two sets: 0.39 ms, 0.72 with 2; ER
+    // n = 5000, IC, R = 500: 0.68 and 0.83).  The others take as many as keep a team within 8
+    // threads, so that a hub's warp has several teams to share its arcs (R-MAT n = 1899, SEIS,
+    // R = 750: 7.0 ms with 1, 2.8 with 2, 2.3 with 4; BA n = 18k, SIS, R = 1010: 2.96, 1.38,
+    // 1.48; BA n = 20k, SIR, R = 1000: 6.4, 4.7, 4.4; BA n = 250k, SEIR, R = 100: 8.7, 9.0,
+    // 13.5); rows of 16 words 2, for IC 4 (R-MAT n = 20k, R = 300: 15.7, 8.3, 6.3).
     const int w = std::min(32, pd);
-    const bool one_round = (int64_t)n * (Wn / w) <= (int64_t)g->sm_count * 24;
+    const bool few = (int64_t)n * (Wn / w) <= (int64_t)g->sm_count * 48 && g->max_deg < 256;
     int V = opt.vector_words ? opt.vector_words
             : !fuse          ? (w >= 16 ? 4 : 2)
-            : one_round      ? 1
-                             : (w >= 32 ? 4 : (w >= 16 ? 2 : 1));
+            : few            ? 1
+                             : (w >= 32 || (w >= 16 && model == FSGP_IC) ? 4 : (w >= 16 ? 2 : 1));
     if (V != 1 && V != 2 && V != 4) return fail(FSGP_EINVAL, "vector_words must be 1, 2 or 4");
     if (V > pd) V = pd;
     const int SW = std::min(32 * V, pd);

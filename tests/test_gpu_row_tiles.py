@@ -93,3 +93,19 @@ def test_graph_between_the_fused_bounds(cuda_lib, R):
     sets = [W.seed_set(g.n, 50, seed=32 + i) for i in range(12 if R == 64 else 1)]
     assert (1 << 20) < n_words * len(sets) <= (1 << 22)
     _check(cuda_lib, g, O.SIS, sets, R, 3, 16, {}, beta=0.1, gamma=0.1)
+
+
+@pytest.mark.parametrize("longest", [255, 256])
+@pytest.mark.parametrize("R", [500, 1000])
+def test_longest_row_of_a_small_graph(cuda_lib, R, longest):
+    """The words per thread of a small graph follow from its longest row (below 256 arcs: one,
+    and the persistent loop)."""
+    rng = np.random.default_rng(31)
+    d = rng.integers(0, 6, size=400)
+    d[[0, 250]] = longest
+    row_ptr = np.zeros(401, dtype=np.int32)
+    row_ptr[1:] = np.cumsum(d)
+    g = W.Graph(row_ptr, rng.integers(0, 400, size=int(row_ptr[-1])).astype(np.int32), "longest")
+    for model in (O.SEIS, O.IC, O.LT, O.SWIR):
+        _check(cuda_lib, g, model, [W.seed_set(g.n, 20, seed=32)], R, 5, 16, {}, beta=0.05, gamma=0.2, alpha=0.4, mu=0.1,
+               nu=0.5, ic_mode=O.IC_CONSTANT, ic_p=0.1)
