@@ -92,7 +92,7 @@ extern "C" int fsgp_autotune(const fsgp_graph *gc, int32_t model, const fsgp_par
     if (T_probe < 1) return fail(FSGP_EINVAL, "T_probe must be >= 1");
     cudaStream_t s = (cudaStream_t)stream;
     uint64_t *d_counts = nullptr;
-    FSGP_CUDA(cudaMalloc(&d_counts, sizeof(uint64_t) * 3 * ((size_t)T_probe + 1)));
+    FSGP_CUDA(cudaMalloc(&d_counts, sizeof(uint64_t) * (size_t)fsgp_model_compartments(model) * ((size_t)T_probe + 1)));
     const int Ws = ws_of(R);
     const int vws[3] = {1, 2, 4};
     const int smalls[2] = {63, 255};
