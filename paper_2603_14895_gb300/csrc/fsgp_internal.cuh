@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "fsgp.h"
+#include "hub_slots.h"
 
 namespace fsgp {
 
@@ -114,14 +115,6 @@ struct ClassInfo {
     int32_t bucket_start[34];   // start of each bucket in rows_sorted (descending order)
 };
 
-struct HubTable {
-    int32_t min_deg = -1;       // table built for this hub threshold and chunk size
-    int32_t chunk = -1;
-    int32_t n_hubs = 0;
-    int64_t n_chunks = 0;
-    int64_t *d_chunk_base = nullptr;  // [n_hubs + 1] (hub rows are new ids 0 .. n_hubs-1)
-};
-
 struct Workspace {
     void *ptr = nullptr;
     size_t bytes = 0;
@@ -187,7 +180,7 @@ struct fsgp_graph {
     int32_t lane_start = 0;         // new id of lane_tab[0]
     int32_t d0_start = 0;           // new id of the first row without in-arcs
     fsgp::ClassInfo cls{};
-    fsgp::HubTable hubs[2];          // (see ensure_hub_table)
+    fsgp::HubTable hubs[2];         // (see hub_slot)
     fsgp::Workspace ws{};
     std::vector<fsgp::ExecCache> execs;   // most recent last (they point into ws)
     float *arc_w = nullptr;         // [nnz] arc weights in the caller's arc order, or null

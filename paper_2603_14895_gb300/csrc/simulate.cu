@@ -374,24 +374,8 @@ __global__ void k_row_degrees(const int32_t *__restrict__ row_ptr, const int32_t
 }
 
 // Hub chunk table for (hub bucket, chunk): hub rows are rows_sorted[0 .. n_hubs).
-static int ensure_hub_table(fsgp_graph *g, int hub_min_deg, int chunk, cudaStream_t s, const HubTable **out) {
-    for (HubTable &T : g->hubs) {
-        *out = &T;
-        if (T.min_deg == hub_min_deg && T.chunk == chunk) return FSGP_OK;
-    }
-    // two tables are kept (models with different chunks may alternate); the older one goes
-    std::swap(g->hubs[0], g->hubs[1]);
-    HubTable &H = g->hubs[1];
-    *out = &H;
-    const int bh = bitlen(hub_min_deg);   // bucket of hub_min_deg (a power of two)
-    const int32_t n_hubs = bh >= 1 ? g->cls.bucket_start[bh - 1] : g->n;
-    cudaFree(H.d_chunk_base);
-    H.d_chunk_base = nullptr;
-    H.n_hubs = n_hubs;
-    H.n_chunks = 0;
-    H.min_deg = hub_min_deg;
-    H.chunk = chunk;
-    if (n_hubs == 0) return FSGP_OK;
+static int build_hub_table(const fsgp_graph *g, int chunk, cudaStream_t s, HubTable &H) {
+    const int32_t n_hubs = H.n_hubs;
     int32_t *d_deg = nullptr;
     FSGP_CUDA(cudaMalloc(&d_deg, sizeof(int32_t) * (size_t)n_hubs));
     k_row_degrees<<<grid_cap(n_hubs, 256, g->sm_count), 256, 0, s>>>(g->row_ptr, g->rows_sorted, n_hubs, d_deg);
@@ -410,6 +394,14 @@ static int ensure_hub_table(fsgp_graph *g, int hub_min_deg, int chunk, cudaStrea
     FSGP_CUDA(cudaStreamSynchronize(s));
     H.n_chunks = base[n_hubs];
     return FSGP_OK;
+}
+
+static int ensure_hub_table(fsgp_graph *g, int hub_min_deg, int chunk, cudaStream_t s, const HubTable **out) {
+    const int bh = bitlen(hub_min_deg);   // bucket of hub_min_deg (a power of two)
+    const int32_t n_hubs = bh >= 1 ? g->cls.bucket_start[bh - 1] : g->n;
+    return hub_slot(
+        g->hubs, hub_min_deg, chunk, n_hubs, [](HubTable &H) { cudaFree(H.d_chunk_base); },
+        [&](HubTable &H) { return build_hub_table(g, chunk, s, H); }, out);
 }
 
 static size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
