@@ -18,6 +18,7 @@
 #include <string>
 #include <vector>
 
+#include "fused_split.h"
 #include "step.cuh"
 
 namespace fsgp {
@@ -769,15 +770,12 @@ static int run_wave(fsgp_graph *g, int model, int ic_mode, int weighted, const S
     L.V = V;
     L.TEAM = TEAM;
     L.smem_lanes = smem_lanes;
-    // Fused rows: the rows of 2^b in-arcs and more get a warp each (16-bit counters), the
-    // others a team (8-bit counters).  A small graph's step lasts as long as its longest
-    // chain of gathers, so b is the smallest bound for which the warp rows take at most half
-    // of the warps that fit at once (60 graphs of 8k to 1M words: 1.16 times faster on average
-    // than all of them, as fast as a quarter), and at most 8.
-    const int64_t fit_warps = (int64_t)g->sm_count * std::max(occ.fused, 1) * (kBlock / 32);
-    int split_b = 0;
-    while (fuse && split_b < kSmallBits && 2 * (int64_t)g->cls.bucket_start[split_b] * nslices > fit_warps) ++split_b;
-    const int32_t fuse_split = !fuse ? 0 : (split_b == 0 ? n : g->cls.bucket_start[split_b]);
+    const int per_block_small = (kBlock / 32) * (32 / TEAM);
+    FusedSplit split{};
+    if (fuse)
+        split = fused_split(g->cls.bucket_start, n, g->nnz, nslices, (int64_t)g->sm_count * std::max(occ.fused, 1),
+                            kBlock / 32, per_block_small, kSmallBits);
+    const int32_t fuse_split = split.warp_rows;
     // All T steps in one cooperative launch (no per-lane counts).  (27 graphs of 8k to 200k
     // words: 1.2 times faster than a launch per step on average; 16 of 200k to 1M words: 0.9
     // to 1.26.)
@@ -792,15 +790,13 @@ static int run_wave(fsgp_graph *g, int model, int ic_mode, int weighted, const S
     L.have_mid = !fuse && n_mid > 0;
     L.have_hub = !fuse && n_hubs > 0;
     L.prof = profiling ? &prof : nullptr;
-    const int per_block_small = (kBlock / 32) * (32 / TEAM);
     auto grid_for = [&](int64_t cap, int64_t items, int per_block) {
         return (int)std::min<int64_t>(cap, (items + per_block - 1) / per_block);
     };
     const int64_t sms = g->sm_count;
     if (fuse) {
-        L.grid_mid = grid_for(sms * occ.fused, (int64_t)fuse_split * nslices, kBlock / 32);
-        L.grid_small = grid_for(std::max<int64_t>(sms * occ.fused - L.grid_mid, 1), (int64_t)(n - fuse_split) * nslices,
-                                per_block_small);
+        L.grid_mid = split.grid_mid;
+        L.grid_small = split.grid_small;
     } else {
         L.grid_small = std::max(1, grid_for(sms * occ.small, (int64_t)n_small_all * nslices, per_block_small));
         L.grid_small4 = std::max(1, grid_for(sms * occ.small4, (int64_t)n_small4 * nslices, per_block_small));
