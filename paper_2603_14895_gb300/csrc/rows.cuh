@@ -1836,39 +1836,66 @@ __global__ void __launch_bounds__(kBlock, ModelTraits<MODEL>::tiled ? 3 : 1) k_r
 // than those CTAs' shared memory: the default takes the largest carve-out as soon as one
 // more CTA would fit by shared memory alone, and what is left as L1 (28 KB) then has too
 // few lines for the gathered rows in flight (random 32-byte rows out of L2: 287e9 rows/s
-// with 60 KB of L1 or more, 153e9 with 28 KB).
-inline int resident_ctas(const void *kern, size_t smem, size_t tile) {
+// with 60 KB of L1 or more, 153e9 with 28 KB).  The kernel's own preference is that of runs
+// without per-lane counters, the same every time, since host threads of a batch may set it
+// concurrently; a run with counters asks for its share at each launch (RowFit::carve; with
+// the kernel's preference one CTA of two stayed out: SIR with per-realization counts, R = 1000,
+// T = 40, BA n = 250k: 36.1 and 24.1 ms; n = 20k: 4.9 and 3.2; SIS, R-MAT n = 1M, T = 20: 26.5 and
+// 19.5).
+inline RowFit resident_ctas(const void *kern, size_t smem, size_t tile) {
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(tile + kLaneCounterBytes));
     int z = 1, z0 = 1;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&z, kern, kBlock, smem + tile);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&z0, kern, kBlock, tile);
-    if (z < 1) z = 1;
+    RowFit f{std::max(z, 1), 0};
     cudaFuncAttributes at{};
     int per_sm = 0, dev = 0;
     if (cudaGetDevice(&dev) == cudaSuccess && cudaFuncGetAttributes(&at, kern) == cudaSuccess &&
         cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) == cudaSuccess && per_sm > 0) {
-        const size_t need = (size_t)std::max(z0, 1) * (tile + at.sharedSizeBytes + 1024);   // 1 KB is the system's
-        cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             (int)std::min<size_t>(100, (need * 100 + per_sm - 1) / (size_t)per_sm));
+        auto percent = [&](int ctas, size_t dynamic) {   // 1 KB of each CTA is the system's
+            const size_t need = (size_t)ctas * (dynamic + at.sharedSizeBytes + 1024);
+            return (int)std::min<size_t>(100, (need * 100 + per_sm - 1) / (size_t)per_sm);
+        };
+        cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, percent(std::max(z0, 1), tile));
+        if (smem) f.carve = percent(f.ctas, smem + tile);
     }
-    return z;
+    return f;
 }
 
 // The same, asked once per kernel, device and size in a row (a small graph's run is shorter
-// than a handful of driver queries are cheap).  The attributes set are the same every time:
-// the shared-memory limit is raised to the tiles plus the largest per-lane counter area any
-// run uses, since host threads of a batch may set it concurrently.
+// than a handful of driver queries are cheap).
 template <auto Kern>
-int occupancy_one(size_t smem, size_t tile) {
-    static std::atomic<uint64_t> last{0};   // 1 << 63 | device << 48 | smem << 16 | CTAs
+RowFit occupancy_one(size_t smem, size_t tile) {
+    static std::atomic<uint64_t> last{0};   // 1 << 63 | device << 48 | smem << 16 | carve << 8 | CTAs
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev >= 1 << 15) return resident_ctas((const void *)Kern, smem, tile);
     const uint64_t key = 1ull << 63 | (uint64_t)dev << 48 | (uint64_t)smem << 16;
     const uint64_t seen = last.load(std::memory_order_acquire);
-    if ((seen & ~0xffffull) == key) return (int)(seen & 0xffffull);
-    const int z = resident_ctas((const void *)Kern, smem, tile);
-    last.store(key | (uint64_t)z, std::memory_order_release);
-    return z;
+    if ((seen & ~0xffffull) == key) return RowFit{(int)(seen & 0xff), (int)(seen >> 8 & 0xff)};
+    const RowFit f = resident_ctas((const void *)Kern, smem, tile);
+    last.store(key | (uint64_t)f.carve << 8 | (uint64_t)f.ctas, std::memory_order_release);
+    return f;
+}
+
+// Launch of a row kernel; carve: the share of the SM's memory asked for as shared memory, in
+// percent (0: the kernel's own preference).
+template <class... P, class... Q>
+void launch_row_kernel(void (*kern)(P...), int grid, size_t smem, int carve, cudaStream_t s, Q... args) {
+    if (carve == 0) {
+        kern<<<grid, kBlock, smem, s>>>(args...);
+        return;
+    }
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    at.val.sharedMemCarveout = (unsigned)carve;
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3((unsigned)grid);
+    c.blockDim = dim3(kBlock);
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    cudaLaunchKernelEx(&c, kern, args...);
 }
 
 // Widest slice of the one-thread-per-row kernel: the staging area of the three-plane
@@ -1877,14 +1904,14 @@ template <int MODEL>
 constexpr int lane_swl_max() { return ModelTraits<MODEL>::planes >= 3 ? 4 : 8; }
 
 template <int MODEL>
-int launch_rows_lane(const StepArgs &A, int swl, int grid, size_t smem, cudaStream_t s) {
+int launch_rows_lane(const StepArgs &A, int swl, int grid, size_t smem, int carve, cudaStream_t s) {
     switch (swl) {
-        case 1: k_rows_lane<MODEL, 1><<<grid, kBlock, smem + kLaneSmem<MODEL, 1>, s>>>(A); break;
-        case 2: k_rows_lane<MODEL, 2><<<grid, kBlock, smem + kLaneSmem<MODEL, 2>, s>>>(A); break;
-        case 4: k_rows_lane<MODEL, 4><<<grid, kBlock, smem + kLaneSmem<MODEL, 4>, s>>>(A); break;
+        case 1: launch_row_kernel(k_rows_lane<MODEL, 1>, grid, smem + kLaneSmem<MODEL, 1>, carve, s, A); break;
+        case 2: launch_row_kernel(k_rows_lane<MODEL, 2>, grid, smem + kLaneSmem<MODEL, 2>, carve, s, A); break;
+        case 4: launch_row_kernel(k_rows_lane<MODEL, 4>, grid, smem + kLaneSmem<MODEL, 4>, carve, s, A); break;
         case 8:
             if constexpr (lane_swl_max<MODEL>() >= 8) {
-                k_rows_lane<MODEL, 8><<<grid, kBlock, smem + kLaneSmem<MODEL, 8>, s>>>(A);
+                launch_row_kernel(k_rows_lane<MODEL, 8>, grid, smem + kLaneSmem<MODEL, 8>, carve, s, A);
                 break;
             }
             return fail(FSGP_EINVAL, "lane kernel slice width");
@@ -1894,23 +1921,20 @@ int launch_rows_lane(const StepArgs &A, int swl, int grid, size_t smem, cudaStre
 }
 
 template <int MODEL, int SWL>
-int occupancy_lane_w(size_t smem) {
+RowFit occupancy_lane_w(size_t smem) {
     return occupancy_one<k_rows_lane<MODEL, SWL>>(smem, kLaneSmem<MODEL, SWL>);
 }
 
 template <int MODEL>
-int occupancy_lane(int swl, size_t smem) {
-    int z = 1;
+RowFit occupancy_lane(int swl, size_t smem) {
     switch (swl) {
-        case 1: z = occupancy_lane_w<MODEL, 1>(smem); break;
-        case 2: z = occupancy_lane_w<MODEL, 2>(smem); break;
-        case 4: z = occupancy_lane_w<MODEL, 4>(smem); break;
+        case 1: return occupancy_lane_w<MODEL, 1>(smem);
+        case 2: return occupancy_lane_w<MODEL, 2>(smem);
+        case 4: return occupancy_lane_w<MODEL, 4>(smem);
         default:
-            if constexpr (lane_swl_max<MODEL>() >= 8) z = occupancy_lane_w<MODEL, 8>(smem);
-            else z = occupancy_lane_w<MODEL, 4>(smem);
-            break;
+            if constexpr (lane_swl_max<MODEL>() >= 8) return occupancy_lane_w<MODEL, 8>(smem);
+            else return occupancy_lane_w<MODEL, 4>(smem);
     }
-    return z < 1 ? 1 : z;
 }
 
 // ------------------------------------------------------------------------- launch
@@ -1920,8 +1944,8 @@ int launch_rows_vt(const StepArgs &A, const StepLaunch &L, cudaStream_t s) {
     Prof *pr = L.prof;
     if (L.fused) {
         if (pr) pr->start(PK_SMALL, s);
-        k_rows_fused<MODEL, V, TEAM><<<L.grid_mid + L.grid_small, kBlock, L.smem_lanes + FusedBytes<MODEL, V, TEAM>, s>>>(
-            A, L.grid_mid);
+        launch_row_kernel(k_rows_fused<MODEL, V, TEAM>, L.grid_mid + L.grid_small,
+                          L.smem_lanes + FusedBytes<MODEL, V, TEAM>, L.carve_fused, s, A, L.grid_mid);
         if (pr) pr->stop(s);
         return FSGP_OK;
     }
@@ -1939,22 +1963,25 @@ int launch_rows_vt(const StepArgs &A, const StepLaunch &L, cudaStream_t s) {
     }
     if (L.have_mid) {
         if (pr) pr->start(PK_MID, s);
-        k_rows<MODEL, V, TEAM, true><<<L.grid_mid, kBlock, L.smem_lanes + TileBytes<MODEL, V, TEAM, true, kSmallBits>, s>>>(A, 1);
+        launch_row_kernel(k_rows<MODEL, V, TEAM, true>, L.grid_mid,
+                          L.smem_lanes + TileBytes<MODEL, V, TEAM, true, kSmallBits>, L.carve_mid, s, A, 1);
         if (pr) pr->stop(s);
     }
     if (L.have_small) {
         if (pr) pr->start(PK_SMALL, s);
-        k_rows<MODEL, V, TEAM, false><<<L.grid_small, kBlock, L.smem_lanes + TileBytes<MODEL, V, TEAM, false, kSmallBits>, s>>>(A, 0);
+        launch_row_kernel(k_rows<MODEL, V, TEAM, false>, L.grid_small,
+                          L.smem_lanes + TileBytes<MODEL, V, TEAM, false, kSmallBits>, L.carve_small, s, A, 0);
         if (pr) pr->stop(s);
     }
     if (L.have_small4) {
         if (pr) pr->start(PK_SMALL4, s);
-        k_rows<MODEL, V, TEAM, false, 4><<<L.grid_small4, kBlock, L.smem_lanes + TileBytes<MODEL, V, TEAM, false, 4>, s>>>(A, 3);
+        launch_row_kernel(k_rows<MODEL, V, TEAM, false, 4>, L.grid_small4,
+                          L.smem_lanes + TileBytes<MODEL, V, TEAM, false, 4>, L.carve_small4, s, A, 3);
         if (pr) pr->stop(s);
     }
     if (L.have_lane) {
         if (pr) pr->start(PK_LANE, s);
-        const int rc = launch_rows_lane<MODEL>(A, L.swl, L.grid_lane, L.smem_lanes, s);
+        const int rc = launch_rows_lane<MODEL>(A, L.swl, L.grid_lane, L.smem_lanes, L.carve_lane, s);
         if (pr) pr->stop(s);
         if (rc) return rc;
     }
@@ -2040,7 +2067,7 @@ template <int MODEL, int TEAM>
 int launch_persist_t(const StepArgs &A, const PersistArgs &Q, int grid_mid, int grid_small, size_t smem, int sm_count,
                      cudaStream_t s, int *grid_out) {
     auto kern = k_rows_persist<MODEL, TEAM>;
-    const int per_sm = occupancy_one<k_rows_persist<MODEL, TEAM>>(smem, FusedBytes<MODEL, 1, TEAM>);
+    const int per_sm = occupancy_one<k_rows_persist<MODEL, TEAM>>(smem, FusedBytes<MODEL, 1, TEAM>).ctas;
     const int cap = per_sm * sm_count;
     if (cap < 2) return FSGP_EUNSUPPORTED;
     if (grid_mid + grid_small > cap) {

@@ -770,10 +770,15 @@ static int run_wave(fsgp_graph *g, int model, int ic_mode, int weighted, const S
     L.V = V;
     L.TEAM = TEAM;
     L.smem_lanes = smem_lanes;
+    L.carve_small = occ.small.carve;
+    L.carve_mid = occ.mid.carve;
+    L.carve_small4 = occ.small4.carve;
+    L.carve_lane = occ.lane.carve;
+    L.carve_fused = occ.fused.carve;
     const int per_block_small = (kBlock / 32) * (32 / TEAM);
     FusedSplit split{};
     if (fuse)
-        split = fused_split(g->cls.bucket_start, n, g->nnz, nslices, (int64_t)g->sm_count * std::max(occ.fused, 1),
+        split = fused_split(g->cls.bucket_start, n, g->nnz, nslices, (int64_t)g->sm_count * std::max(occ.fused.ctas, 1),
                             kBlock / 32, per_block_small, kSmallBits);
     const int32_t fuse_split = split.warp_rows;
     // All T steps in one cooperative launch (no per-lane counts).  (27 graphs of 8k to 200k
@@ -798,11 +803,11 @@ static int run_wave(fsgp_graph *g, int model, int ic_mode, int weighted, const S
         L.grid_mid = split.grid_mid;
         L.grid_small = split.grid_small;
     } else {
-        L.grid_small = std::max(1, grid_for(sms * occ.small, (int64_t)n_small_all * nslices, per_block_small));
-        L.grid_small4 = std::max(1, grid_for(sms * occ.small4, (int64_t)n_small4 * nslices, per_block_small));
-        L.grid_lane = std::max(1, grid_for(sms * occ.lane, (int64_t)(n_lane + n_d0) * (Wn / occ.swl), kBlock));
-        L.grid_mid = std::max(1, grid_for(sms * occ.mid, (int64_t)n_mid * nslices, kBlock / 32));
-        L.grid_hub = std::max(1, grid_for(sms * occ.hub, hub->n_chunks * nslices, 1));
+        L.grid_small = std::max(1, grid_for(sms * occ.small.ctas, (int64_t)n_small_all * nslices, per_block_small));
+        L.grid_small4 = std::max(1, grid_for(sms * occ.small4.ctas, (int64_t)n_small4 * nslices, per_block_small));
+        L.grid_lane = std::max(1, grid_for(sms * occ.lane.ctas, (int64_t)(n_lane + n_d0) * (Wn / occ.swl), kBlock));
+        L.grid_mid = std::max(1, grid_for(sms * occ.mid.ctas, (int64_t)n_mid * nslices, kBlock / 32));
+        L.grid_hub = std::max(1, grid_for(sms * occ.hub.ctas, hub->n_chunks * nslices, 1));
         L.grid_fin = std::max(1, grid_for(INT32_MAX, n_hubs, kBlock / 32));
     }
 

@@ -767,6 +767,7 @@ struct StepLaunch {
     int V, TEAM;           // words per thread, threads per slice team
     int grid_small, grid_mid, grid_hub, grid_fin, grid_small4, grid_lane;
     int swl;               // words per thread of the one-thread-per-row kernel
+    int carve_small, carve_mid, carve_small4, carve_lane, carve_fused;   // (see RowFit)
     size_t smem_lanes;     // dynamic shared memory for per-lane counters (0 = off)
     bool have_small, have_mid, have_hub, have_small4, have_lane;
     bool fused;            // both classes of a small graph in one launch: grid_mid CTAs on
@@ -819,8 +820,12 @@ int launch_persist(const StepArgs &A, const PersistArgs &Q, int TEAM, int grid_m
 // Defined in rows.cuh, instantiated once per model (model_*.cu).
 template <int MODEL>
 int launch_rows(const StepArgs &A, const StepLaunch &L, cudaStream_t s);
+struct RowFit {
+    int ctas;    // resident CTAs per SM
+    int carve;   // their share of the SM's memory, in percent (0: the kernel's own preference)
+};
 struct RowOccupancy {
-    int small, small4, lane, mid, hub, fused;   // resident CTAs per SM of each row kernel
+    RowFit small, small4, lane, mid, hub, fused;
     int swl;                             // in: slice width of the lane kernel
     bool fused_only;                     // in: only the fused kernel is wanted
 };
