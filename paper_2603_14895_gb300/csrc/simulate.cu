@@ -533,7 +533,9 @@ static int run_wave(fsgp_graph *g, int model, int ic_mode, int weighted, const S
     // Words per thread (w: words a team covers with one word per thread).  Large graphs: 2,
     // and 4 for rows of 16 words and more, whose teams are then at most 8 threads wide and
     // spend less per arc (BA n = 1M, IC, R = 1024: 50.8 against 39.0 ms; R-MAT, SIS, R = 256:
-    // 178 against 179 ms).  Small graphs whose rows all get a warp in one or two rounds, none
+    // 178 against 179 ms); SWIR, decided in place, stays at 2 (BA n = 250k, R = 1000, T = 40, with
+    // per-realization counts: 43.2 ms with 4, 26.8 with 2; R-MAT n = 1M, R = 1000: 28.7 and
+    // 24.6).  Small graphs whose rows all get a warp in one or two rounds, none
     // with hundreds of arcs, are bound by the chain of a row and the barrier and take 1, and
     // with it the persistent loop (BA n = 6434, LT, R = 152, two sets: 0.39 ms, 0.72 with 2; ER
     // n = 5000, IC, R = 500: 0.68 and 0.83).  The others take as many as keep a team within 8
@@ -544,7 +546,7 @@ static int run_wave(fsgp_graph *g, int model, int ic_mode, int weighted, const S
     const int w = std::min(32, pd);
     const bool few = (int64_t)n * (Wn / w) <= (int64_t)g->sm_count * 48 && g->max_deg < 256;
     int V = opt.vector_words ? opt.vector_words
-            : !fuse          ? (w >= 16 ? 4 : 2)
+            : !fuse          ? (w >= 16 && model != FSGP_SWIR ? 4 : 2)
             : few            ? 1
                              : (w >= 32 || (w >= 16 && model == FSGP_IC) ? 4 : (w >= 16 ? 2 : 1));
     if (V != 1 && V != 2 && V != 4) return fail(FSGP_EINVAL, "vector_words must be 1, 2 or 4");
