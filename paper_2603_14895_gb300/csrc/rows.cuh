@@ -304,12 +304,13 @@ constexpr int min_ctas() { return V == 4 ? 2 : (V == 2 ? 3 : 4); }
 // step), 1 = mid rows, 3 = rows with 4..15 in-arcs (dense steps only).
 // CG: the state planes are read through L2 only (the persistent step loop, which reads
 // in one launch the planes that other CTAs wrote at the previous step).
+// B: counter bits.  AG: teams that share a team row's arcs.
 // bid of nb: the CTA's place among those that work on these rows.
-template <int MODEL, int V, int TEAM, bool WARP_ROW, int BT, bool CG>
+template <int MODEL, int V, int TEAM, bool WARP_ROW, int BT, bool CG, int B, int AG>
 __device__ __forceinline__ void rows_body(const StepArgs &A, int which, int32_t *s_lane, unsigned long long *s_pc,
                                           int bid, int nb) {
     static_assert(ModelTraits<MODEL>::counts, "arc models go through the warp tile");
-    constexpr int B = WARP_ROW ? kWideBits : BT;
+    static_assert(AG == 1 || (!WARP_ROW && V == 1 && TEAM * AG <= 32), "arc groups: team rows within a warp");
     constexpr int TPW = 32 / TEAM;
     constexpr int SW = TEAM * V;
     constexpr int P = ModelTraits<MODEL>::planes;
@@ -339,7 +340,7 @@ __device__ __forceinline__ void rows_body(const StepArgs &A, int which, int32_t 
     const int tl = lane % TEAM;
     const int64_t gwarp = ((int64_t)bid * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)nb * blockDim.x) >> 5;
-    constexpr int RPI = WARP_ROW ? 1 : TPW;
+    constexpr int RPI = WARP_ROW ? 1 : TPW / AG;
     const int list_slot = A.k & 1;
     const int64_t nitems = nrows * A.nslices;
     Accum acc;
@@ -353,7 +354,7 @@ __device__ __forceinline__ void rows_body(const StepArgs &A, int which, int32_t 
     for (int i = 0; i < V; ++i) d0[i] = d1[i] = d2[i] = 0;
 
     for (int64_t base = gwarp * RPI; base < nitems; base += nwarps * RPI) {
-        const int64_t item = WARP_ROW ? base : base + team;
+        const int64_t item = WARP_ROW ? base : base + team / AG;
         const bool has_row = item < nitems;
         const int64_t ridx = has_row ? div_slices(item, A.nslices, nitems) : 0;
         const int slice = has_row ? (int)(item - ridx * A.nslices) : 0;
@@ -399,7 +400,7 @@ __device__ __forceinline__ void rows_body(const StepArgs &A, int which, int32_t 
             beg = __ldg(A.rp + v);
             end = __ldg(A.rp + v + 1);
         }
-        constexpr int parts = WARP_ROW ? TPW : 1;   // teams that share a row
+        constexpr int parts = WARP_ROW ? TPW : AG;   // teams that share a row
         gather_counts<MODEL, V, B, TEAM, parts, CG>(A, beg, any_need ? end - beg : 0, 8 * parts, w0, lane, c);
         constexpr bool SPLIT = WARP_ROW && TPW >= V;   // enough teams to give each word one
         if constexpr (SPLIT && V == 2) {
@@ -422,10 +423,10 @@ __device__ __forceinline__ void rows_body(const StepArgs &A, int which, int32_t 
             }
 #pragma unroll
             for (int b = 0; b < B; ++b) c[1][b] = c[0][b];
-        } else if constexpr (WARP_ROW) {
+        } else if constexpr (parts > 1) {
             // merge the teams' partial results (the warp is converged here)
 #pragma unroll
-            for (int o = TEAM; o < 32; o <<= 1) {
+            for (int o = TEAM; o < TEAM * parts; o <<= 1) {
 #pragma unroll
                 for (int i = 0; i < V; ++i) {
                     uint32_t d[B];
@@ -477,7 +478,7 @@ __device__ __forceinline__ void rows_body(const StepArgs &A, int which, int32_t 
             for (int o = 1; o < 32; o <<= 1) fl |= __shfl_xor_sync(0xffffffffu, fl, o);
             writer = has_row && team == 0;
         } else {
-        writer = has_row && (!WARP_ROW || team == 0);
+        writer = has_row && team % parts == 0;
         if (writer) {
             // own state again (L1/L2-resident): not kept live across the gather
             uint32_t s0[V], s1[V], s2[V];
@@ -1082,11 +1083,11 @@ __device__ __forceinline__ void rows_tile(const StepArgs &A, int which, uint8_t 
 }
 
 // The rows of one class: through the warp tile, or in place (SWIR).
-template <int MODEL, int V, int TEAM, bool WARP_ROW, int BT, bool CG>
+template <int MODEL, int V, int TEAM, bool WARP_ROW, int BT, bool CG, int WB = kWideBits, int AG = 1>
 __device__ __forceinline__ void rows_class(const StepArgs &A, int which, uint8_t *smem, int32_t *s_lane,
                                            unsigned long long *s_pc, int bid, int nb) {
     if constexpr (ModelTraits<MODEL>::tiled) rows_tile<MODEL, V, TEAM, WARP_ROW, BT, CG>(A, which, smem, s_lane, s_pc, bid, nb);
-    else rows_body<MODEL, V, TEAM, WARP_ROW, BT, CG>(A, which, s_lane, s_pc, bid, nb);
+    else rows_body<MODEL, V, TEAM, WARP_ROW, BT, CG, WARP_ROW ? WB : BT, AG>(A, which, s_lane, s_pc, bid, nb);
 }
 
 // Dynamic shared memory of a class's tiles, and of either class's (fused kernels).
@@ -1129,7 +1130,7 @@ __global__ void __launch_bounds__(kBlock, V == 4 ? 2 : 3) k_rows_fused(StepArgs 
 // (CG loads): a CTA reads at step k the words other CTAs wrote at step k-1.
 // (bounded for 2 resident CTAs per SM: the loop is meant for graphs that fill a few CTAs
 // per SM at most, and the body then keeps its state in registers)
-template <int MODEL, int TEAM>
+template <int MODEL, int TEAM, int WB, int AG>
 __global__ void __launch_bounds__(kBlock, 2)
     k_rows_persist(const __grid_constant__ StepArgs A0, const __grid_constant__ PersistArgs Q) {
     extern __shared__ __align__(16) uint8_t s_dyn[];
@@ -1168,11 +1169,14 @@ __global__ void __launch_bounds__(kBlock, 2)
             if (blockIdx.x == 0 && threadIdx.x == 0) C->stop = 1;
             break;
         }
-        if ((int)blockIdx.x < Q.warp_ctas)
-            rows_class<MODEL, 1, TEAM, true, kSmallBits, true>(sA, 1, s_dyn, s_lane, s_pc, blockIdx.x, Q.warp_ctas);
-        else
+        if constexpr (AG > 1) {
+            rows_class<MODEL, 1, TEAM, false, kSmallBits, true, WB, AG>(sA, 0, s_dyn, s_lane, s_pc, blockIdx.x, gridDim.x);
+        } else if ((int)blockIdx.x < Q.warp_ctas) {
+            rows_class<MODEL, 1, TEAM, true, kSmallBits, true, WB>(sA, 1, s_dyn, s_lane, s_pc, blockIdx.x, Q.warp_ctas);
+        } else {
             rows_class<MODEL, 1, TEAM, false, kSmallBits, true>(sA, 0, s_dyn, s_lane, s_pc, blockIdx.x - Q.warp_ctas,
                                                                 gridDim.x - Q.warp_ctas);
+        }
         if (!grid_barrier(&C->bar_count, &C->bar_gen, gridDim.x, &C->err, Q.spin_limit)) break;
         if (blockIdx.x == 0 && threadIdx.x == 0) C->steps_done = k;
         if (cascade)
@@ -2063,11 +2067,33 @@ int occupancy_rows(int V, int TEAM, size_t smem, RowOccupancy *o) {
 // can be resident at once, at most the launched step's (grid_mid + grid_small CTAs), shared
 // out between the two row classes in the same proportion; *grid_out gets the grid used.
 // FSGP_EUNSUPPORTED: it does not fit (the caller runs the launched loop instead).
-template <int MODEL, int TEAM>
+template <int MODEL, int TEAM, int WB = kWideBits, int AG = 1>
 int launch_persist_t(const StepArgs &A, const PersistArgs &Q, int grid_mid, int grid_small, size_t smem, int sm_count,
                      cudaStream_t s, int *grid_out) {
-    auto kern = k_rows_persist<MODEL, TEAM>;
-    const int per_sm = occupancy_one<k_rows_persist<MODEL, TEAM>>(smem, FusedBytes<MODEL, 1, TEAM>).ctas;
+    // SWIR, decided in place, pays for 16-bit counters in its chain, and at one or two words a row
+    // gets two teams where all rows are short and fit at once, on as few CTAs as that takes
+    // (T = 40; most rows a warp with 16-bit counters, and now: ER n = 1200, R = 32: 423 and
+    // 376 us; n = 2000, R = 64: 454 and 405; n = 10k, R = 650: 979 and 824.  Two teams on every
+    // row of BA n = 2000, R = 32: 568, two classes 418; of ER n = 500k, R = 64: 2376 and 1780).
+    constexpr int per_cta = kBlock / (TEAM * (AG > 1 ? AG : 2));   // rows of a CTA
+    const int64_t team_ctas = ((int64_t)A.n * A.nslices + per_cta - 1) / per_cta;
+    if constexpr (!ModelTraits<MODEL>::tiled && WB != kSmallBits) {
+        if (Q.max_deg < 1 << kSmallBits) {
+            if constexpr (TEAM <= 2)
+                if (Q.max_deg < 64 && team_ctas <= 2 * sm_count)
+                    return launch_persist_t<MODEL, TEAM, kSmallBits, 2>(A, Q, 0, (int)team_ctas, smem, sm_count, s, grid_out);
+            return launch_persist_t<MODEL, TEAM, kSmallBits>(A, Q, grid_mid, grid_small, smem, sm_count, s, grid_out);
+        }
+    }
+    StepArgs a = A;
+    PersistArgs q = Q;
+    if constexpr (AG > 1) {   // every row a team row
+        a.r_small = 0;
+        a.n_small = A.n;
+        a.n_mid = 0;
+    }
+    auto kern = k_rows_persist<MODEL, TEAM, WB, AG>;
+    const int per_sm = occupancy_one<k_rows_persist<MODEL, TEAM, WB, AG>>(smem, FusedBytes<MODEL, 1, TEAM>).ctas;
     const int cap = per_sm * sm_count;
     if (cap < 2) return FSGP_EUNSUPPORTED;
     if (grid_mid + grid_small > cap) {
@@ -2075,8 +2101,6 @@ int launch_persist_t(const StepArgs &A, const PersistArgs &Q, int grid_mid, int 
         grid_mid = grid_small ? std::min(m, cap - 1) : cap;
         grid_small = cap - grid_mid;
     }
-    StepArgs a = A;
-    PersistArgs q = Q;
     q.warp_ctas = grid_mid;
     void *args[] = {&a, &q};
     const cudaError_t e = cudaLaunchCooperativeKernel((const void *)kern, dim3(grid_mid + grid_small), dim3(kBlock), args,

@@ -542,9 +542,11 @@ static int run_wave(fsgp_graph *g, int model, int ic_mode, int weighted, const S
     // threads, so that a hub's warp has several teams to share its arcs (R-MAT n = 1899, SEIS,
     // R = 750: 7.0 ms with 1, 2.8 with 2, 2.3 with 4; BA n = 18k, SIS, R = 1010: 2.96, 1.38,
     // 1.48; BA n = 20k, SIR, R = 1000: 6.4, 4.7, 4.4; BA n = 250k, SEIR, R = 100: 8.7, 9.0,
-    // 13.5); rows of 16 words 2, for IC 4 (R-MAT n = 20k, R = 300: 15.7, 8.3, 6.3).
+    // 13.5); rows of 16 words 2, for IC 4 (R-MAT n = 20k, R = 300: 15.7, 8.3, 6.3).  SWIR keeps 1
+    // for twice the rows (ER n = 10k, R = 650: 979 us with 4, 824 with 1; n = 30k, R = 1000: 1415
+    // and 2290).
     const int w = std::min(32, pd);
-    const bool few = (int64_t)n * (Wn / w) <= (int64_t)g->sm_count * 48 && g->max_deg < 256;
+    const bool few = (int64_t)n * (Wn / w) <= (int64_t)g->sm_count * (model == FSGP_SWIR ? 96 : 48) && g->max_deg < 256;
     int V = opt.vector_words ? opt.vector_words
             : !fuse          ? (w >= 16 && model != FSGP_SWIR ? 4 : 2)
             : few            ? 1
@@ -964,6 +966,7 @@ static int run_wave(fsgp_graph *g, int model, int ic_mode, int weighted, const S
         Q.T = (int32_t)T;
         Q.t0 = (uint32_t)opt.t0;
         Q.spin_limit = kPersistSpinCycles;
+        Q.max_deg = g->max_deg;
         int grid_used = 0;
         rc = launch_persist_model(kmodel, A, Q, TEAM, L.grid_mid, L.grid_small, L.smem_lanes, g->sm_count, s, &grid_used);
         if (rc == FSGP_OK) {

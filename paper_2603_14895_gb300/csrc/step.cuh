@@ -56,6 +56,7 @@ struct PersistArgs {
     int32_t T;
     uint32_t t0;
     long long spin_limit;          // SM clock cycles one barrier wait may last
+    int32_t max_deg;               // longest row (sizes the counters of SWIR's warp rows)
     int32_t warp_ctas;             // CTAs on the warp-per-row rows (the first ones)
 };
 
