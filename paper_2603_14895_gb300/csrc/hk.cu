@@ -119,7 +119,7 @@ struct HkAcc {
 // degree-bucket order, so that the teams of a warp have rows of similar length.
 // order may be null (node order) when there are no long rows.
 // The first n_long * segments CTAs take one long row each: its sum has to run through all
-// arcs in order, so one team adds while the whole CTA copies the next kHkStages blocks of
+// arcs in order, so one team adds while the whole CTA (256 threads) copies the next kHkStages blocks of
 // rows to shared memory (a team on its own waits a memory latency for every eight arcs, and
 // the hub of a BA graph then outlasts the step: BA n = 1M, R = 64, a step 1.55 ms so, 0.66 with
 // the copies ahead and the padding arcs' infinities in place of their tests).
@@ -282,29 +282,38 @@ extern "C" int fsgp_hk(const fsgp_graph *gc, const float *h0, int32_t R, int32_t
     const float eps_f = (float)eps;
     // lanes per node: as wide a segment as divides the row (the column indices are loaded
     // once per segment)
-    const int TL = Rp % 128 == 0 ? 32 : (Rp % 64 == 0 ? 16 : 8);
-    const int segs = Rp / (4 * TL);
+    int TL = Rp % 128 == 0 ? 32 : (Rp % 64 == 0 ? 16 : 8);
     // long rows: at least 256 in-arcs and sixteen times the mean, a power of two, so that they
     // are the first of the degree-bucket order; from 32 arcs and four times the mean where four
     // CTAs per SM hold them all, since a small graph's step lasts as long as its longest row
     int lb = 8;
     while (lb < 31 && ((int64_t)n << lb) < 16 * g->nnz) ++lb;
     for (int b = 5; b < lb; ++b)
-        if (((int64_t)n << b) >= 4 * g->nnz && (int64_t)g->cls.bucket_start[b] * segs <= (int64_t)g->sm_count * 4) lb = b;
+        if (((int64_t)n << b) >= 4 * g->nnz && (int64_t)g->cls.bucket_start[b] * (Rp / (4 * TL)) <= (int64_t)g->sm_count * 4)
+            lb = b;
     const int32_t n_long = g->cls.bucket_start[lb];
+    // Where no row is long and every node has its teams at once, a step is the chain of one
+    // row: the narrowest teams (four nodes' chains to a warp) on CTAs of 128 threads, which
+    // spread over more SMs, and in node order, since the degree order would gain nothing and is
+    // one more load in the chain.  (ER, mean degree 4 to 6, R = 33..64, 20 steps: n = 1000 225 us
+    // with teams of 16 on CTAs of 256 threads, 184 so; n = 3000 224 and 184; n = 1500, mean degree
+    // 16, R = 50 267 and 186; a warp per node with 4 bytes per lane 186, 186 and 228.)
+    const bool one_round = n_long == 0 && (int64_t)n * (Rp / 32) * 8 <= (int64_t)g->sm_count * 8 * 256;
+    if (one_round) TL = 8;
+    const int threads = one_round ? 128 : 256;   // (long rows want 256)
+    const int segs = Rp / (4 * TL);
     const int64_t teams = (int64_t)(n - n_long) * segs;
-    const int grid = (int)(std::min<int64_t>((teams * TL + 255) / 256, (int64_t)g->sm_count * 8) + (int64_t)n_long * segs);
-    // (where every team has one row at most and none is long, the order gains nothing and is
-    // one more load in the step's chain)
+    const int grid = (int)(std::min<int64_t>((teams * TL + threads - 1) / threads, (int64_t)g->sm_count * (2048 / threads)) +
+                           (int64_t)n_long * segs);
     const int32_t *order = n_long == 0 && teams * TL <= (int64_t)g->sm_count * 8 * 256 ? nullptr : g->rows_sorted;
     float *cur = buf0, *nxt = buf1;
     for (int32_t k = 1; k <= T && n > 0; ++k) {
         if (TL == 32)
-            k_hk_step<32><<<grid, 256, 0, s>>>(g->row_ptr, g->col, order, n, n_long, R, Rp, eps_f, cur, nxt, d_ch + k);
+            k_hk_step<32><<<grid, threads, 0, s>>>(g->row_ptr, g->col, order, n, n_long, R, Rp, eps_f, cur, nxt, d_ch + k);
         else if (TL == 16)
-            k_hk_step<16><<<grid, 256, 0, s>>>(g->row_ptr, g->col, order, n, n_long, R, Rp, eps_f, cur, nxt, d_ch + k);
+            k_hk_step<16><<<grid, threads, 0, s>>>(g->row_ptr, g->col, order, n, n_long, R, Rp, eps_f, cur, nxt, d_ch + k);
         else
-            k_hk_step<8><<<grid, 256, 0, s>>>(g->row_ptr, g->col, order, n, n_long, R, Rp, eps_f, cur, nxt, d_ch + k);
+            k_hk_step<8><<<grid, threads, 0, s>>>(g->row_ptr, g->col, order, n, n_long, R, Rp, eps_f, cur, nxt, d_ch + k);
         std::swap(cur, nxt);
     }
     FSGP_CUDA(cudaGetLastError());
