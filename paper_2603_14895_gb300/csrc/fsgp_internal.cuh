@@ -137,7 +137,7 @@ constexpr int kExecCacheSize = 4;
 constexpr int32_t kSgLongMin = 32, kSgLongMax = 256;
 constexpr int32_t kSgChunk = 32;
 struct SgCache {
-    int built = 0;
+    void *mem = nullptr;          // one allocation holds all of them; null: not built yet
     int32_t long_min = kSgLongMin;
     float *inv_din = nullptr;     // [n] 1 / d_in (0 when d_in = 0)
     int4 *in_items = nullptr;     // chunks of long in-CSR rows: {row, begin, end, slot}
@@ -145,10 +145,13 @@ struct SgCache {
     int32_t n_in_long = 0;        // long in-CSR rows: the first of rows_sorted, slot = position
     int4 *out_items = nullptr;    // chunks of long out-CSR rows
     int32_t n_out_items = 0;
-    int32_t *out_long = nullptr;
+    int32_t *out_long = nullptr;  // [n_out_long] the long out-CSR rows, ascending
     int32_t n_out_long = 0;
     float *acc = nullptr;         // [max(n_in_long, n_out_long)][64]
 };
+
+// Exclusive scan of n counts (total < 2^31); tile_tmp: one entry per 2048 counts.
+int exclusive_scan_i32(const int32_t *in, int64_t n, int32_t *out, int64_t *tile_tmp, cudaStream_t s);
 
 }  // namespace fsgp
 

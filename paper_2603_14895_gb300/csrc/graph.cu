@@ -305,11 +305,7 @@ static void release(fsgp_graph *g) {
     cudaFree(g->arc_w);
     for (HubTable &T : g->hubs) cudaFree(T.d_chunk_base);
     cudaFree(g->ws.ptr);
-    cudaFree(g->sgc.inv_din);
-    cudaFree(g->sgc.in_items);
-    cudaFree(g->sgc.out_items);
-    cudaFree(g->sgc.out_long);
-    cudaFree(g->sgc.acc);
+    cudaFree(g->sgc.mem);
     delete g;
 }
 

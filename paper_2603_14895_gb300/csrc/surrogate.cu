@@ -841,22 +841,56 @@ __global__ void k_agg_bwd_fin(const int32_t *__restrict__ long_rows, int32_t n_l
     }
 }
 
-// Per-graph tables: 1 / d_in and the long rows of a CSR.
-__global__ void k_inv_deg(const int32_t *__restrict__ row_ptr, int32_t n, float *inv) {
+// Per-graph tables, built on the device: what each row has of long-row chunks.  Position i
+// of the degree order (in-rows, its first n_in_long) and node v (out-rows); the entries past
+// the last are zero, so that the scans end in the totals.
+__device__ __forceinline__ int32_t chunks_of(int32_t d, int32_t long_min) {
+    return d >= long_min ? (int32_t)(((int64_t)d + kSgChunk - 1) / kSgChunk) : 0;
+}
+__global__ void k_table_counts(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ out_ptr,
+                               const int32_t *__restrict__ order, int32_t n, int32_t n_in_long, int32_t long_min,
+                               int32_t *in_chunks, int32_t *out_long, int32_t *out_chunks) {
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v <= n; v += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t d = v < n ? out_ptr[v + 1] - out_ptr[v] : 0;
+        out_long[v] = d >= long_min;
+        out_chunks[v] = chunks_of(d, long_min);
+        if (v <= n_in_long) {
+            const int32_t u = v < n_in_long ? order[v] : 0;
+            in_chunks[v] = v < n_in_long ? chunks_of(row_ptr[u + 1] - row_ptr[u], long_min) : 0;
+        }
+    }
+}
+__global__ void k_table_totals(const int32_t *in_total, const int32_t *long_total, const int32_t *out_total, int32_t *totals) {
+    totals[0] = *in_total;
+    totals[1] = *long_total;
+    totals[2] = *out_total;
+}
+
+// 1 / d_in, and the long out-rows by slot.
+__global__ void k_table_rows(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ out_ptr, int32_t n,
+                             int32_t long_min, const int32_t *__restrict__ out_slot, float *inv, int32_t *out_rows) {
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
         const int32_t d = row_ptr[v + 1] - row_ptr[v];
         inv[v] = d > 0 ? 1.f / (float)d : 0.f;
+        if (out_ptr[v + 1] - out_ptr[v] >= long_min) out_rows[out_slot[v]] = (int32_t)v;
     }
 }
 
-__global__ void k_long_rows(const int32_t *__restrict__ ptr, int32_t n, int32_t long_min, int32_t cap, const int32_t *__restrict__ pos,
-                            int4 *out, int32_t *count) {
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t b = ptr[v], e = ptr[v + 1];
-        if (e - b >= long_min) {
-            const int32_t i = atomicAdd(count, 1);
-            if (i < cap) out[i] = make_int4((int32_t)v, b, e, pos ? pos[v] : (int32_t)v);
+// Chunk t of the m rows whose first chunks are first[0 .. m] (row j: ids[j], or j; its slot:
+// slots[j], or j): one thread per chunk, so that a hub's thousands spread out.
+__global__ void k_table_items(const int32_t *__restrict__ ptr, const int32_t *__restrict__ ids,
+                              const int32_t *__restrict__ slots, const int32_t *__restrict__ first, int32_t m,
+                              int32_t total, int4 *items) {
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
+        int32_t lo = 0, hi = m - 1;   // the last row whose first chunk is t or before
+        while (lo < hi) {
+            const int32_t mid = lo + (hi - lo + 1) / 2;
+            if (first[mid] <= t) lo = mid;
+            else hi = mid - 1;
         }
+        const int32_t row = ids ? ids[lo] : lo;
+        const int64_t b = ptr[row] + (t - first[lo]) * kSgChunk;
+        items[t] = make_int4(row, (int32_t)b, (int32_t)min(b + kSgChunk, (int64_t)ptr[row + 1]), slots ? slots[lo] : lo);
     }
 }
 
@@ -973,71 +1007,67 @@ int grid_of(const fsgp_surrogate *s, int64_t work, int threads, int per_sm = 8) 
     return (int)std::max<int64_t>(g, 1);
 }
 
-// Long rows of one CSR (ptr) as chunk items and, if wanted, a slot -> row list (host build,
-// once).  Slots
-// follow the rows' positions pos (null: the node order).
-int sg_long_table(const int32_t *ptr, int32_t n, int64_t nnz, int32_t long_min, const int32_t *pos, int sm_count, int4 **items, int32_t *n_items,
-                  int32_t **long_rows, int32_t *n_long) {
-    const int64_t cap = nnz / long_min + 1;
-    int4 *d_tmp = nullptr;
-    int32_t *d_cnt = nullptr;
-    FSGP_CUDA(cudaMalloc(&d_tmp, sizeof(int4) * (size_t)cap));
-    cudaError_t e = cudaMalloc(&d_cnt, sizeof(int32_t));
-    int32_t cnt = 0;
-    std::vector<int4> rows;
-    if (e == cudaSuccess) e = cudaMemset(d_cnt, 0, sizeof(int32_t));
-    if (e == cudaSuccess) {
-        const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)n + 255) / 256, (int64_t)sm_count * 8));
-        k_long_rows<<<grid, 256>>>(ptr, n, long_min, (int32_t)cap, pos, d_tmp, d_cnt);
-        e = cudaMemcpy(&cnt, d_cnt, sizeof(int32_t), cudaMemcpyDeviceToHost);
-    }
-    if (e == cudaSuccess && cnt > 0) {
-        rows.resize((size_t)cnt);
-        e = cudaMemcpy(rows.data(), d_tmp, sizeof(int4) * (size_t)cnt, cudaMemcpyDeviceToHost);
-    }
-    cudaFree(d_tmp);
-    cudaFree(d_cnt);
-    if (e != cudaSuccess) return cuda_fail(e, "surrogate long rows");
-    std::sort(rows.begin(), rows.end(), [](const int4 &x, const int4 &y) { return x.w < y.w; });
-    std::vector<int4> it;
-    std::vector<int32_t> lr;
-    for (size_t sl = 0; sl < rows.size(); ++sl) {
-        lr.push_back(rows[sl].x);
-        for (int32_t b = rows[sl].y; b < rows[sl].z; b += kSgChunk)
-            it.push_back(make_int4(rows[sl].x, b, std::min(b + kSgChunk, rows[sl].z), (int32_t)sl));
-    }
-    *n_items = (int32_t)it.size();
-    *n_long = (int32_t)lr.size();
-    if (!it.empty()) {
-        FSGP_CUDA(cudaMalloc(items, sizeof(int4) * it.size()));
-        FSGP_CUDA(cudaMemcpy(*items, it.data(), sizeof(int4) * it.size(), cudaMemcpyHostToDevice));
-        if (!long_rows) return FSGP_OK;
-        FSGP_CUDA(cudaMalloc(long_rows, sizeof(int32_t) * lr.size()));
-        FSGP_CUDA(cudaMemcpy(*long_rows, lr.data(), sizeof(int32_t) * lr.size(), cudaMemcpyHostToDevice));
-    }
-    return FSGP_OK;
-}
-
-// Build the graph's aggregation tables on first use (synchronous; call outside captures).
-int sg_cache(const fsgp_graph *gc, int sm_count) {
+// Build the graph's aggregation tables on first use (synchronises st; call outside
+// captures).  Scratch: activation and gradient buffers of s, which hold nothing yet and
+// have room for n + 1 counts each.
+// (Copying the long rows to the host, sorting and expanding them there took as much as the
+// call: the first gradient on BA n = 300k 1.82 ms, 1.10 so, later ones 0.88; on R-MAT n = 4M
+// 33.7, 14.0 and 13.7; screening 8 candidates on R-MAT n = 4M 62.0, 41.6 and 41.1.)
+int sg_cache(fsgp_surrogate *s, const fsgp_graph *gc, cudaStream_t st) {
     fsgp_graph *g = const_cast<fsgp_graph *>(gc);   // lazily built cache of the handle
-    SgCache &C = g->sgc;
-    if (C.built) return FSGP_OK;
-    while (C.long_min < kSgLongMax && (int64_t)C.long_min * g->n < 4 * g->nnz) C.long_min *= 2;
-    FSGP_CUDA(cudaMalloc(&C.inv_din, sizeof(float) * (size_t)g->n));
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)g->n + 255) / 256, (int64_t)sm_count * 8));
-    k_inv_deg<<<grid, 256>>>(g->row_ptr, g->n, C.inv_din);
-    int rc = sg_long_table(g->row_ptr, g->n, g->nnz, C.long_min, g->pos, sm_count, &C.in_items, &C.n_in_items, nullptr, &C.n_in_long);
-    if (rc) return rc;
-    rc = sg_long_table(g->out_ptr, g->n, g->nnz, C.long_min, nullptr, sm_count, &C.out_items, &C.n_out_items, &C.out_long, &C.n_out_long);
-    if (rc) return rc;
-    const size_t nl = (size_t)std::max(C.n_in_long, C.n_out_long);
-    if (nl) {
-        FSGP_CUDA(cudaMalloc(&C.acc, sizeof(float) * nl * H));
-        FSGP_CUDA(cudaMemset(C.acc, 0, sizeof(float) * nl * H));
+    if (g->sgc.mem) return FSGP_OK;
+    SgCache C;
+    const int32_t n = g->n;
+    int bucket = 0;   // long_min is 2^bucket
+    while (C.long_min < kSgLongMax && (int64_t)C.long_min * n < 4 * g->nnz) C.long_min *= 2;
+    while ((1 << bucket) < C.long_min) ++bucket;
+    C.n_in_long = g->cls.bucket_start[bucket];
+    int32_t *in_chunks = (int32_t *)s->h1, *in_first = (int32_t *)s->h2;
+    int32_t *is_long = (int32_t *)s->dh, *out_slot = (int32_t *)s->dah;
+    int32_t *out_chunks = (int32_t *)s->dam, *out_first = (int32_t *)s->dh2;
+    int64_t *tiles = (int64_t *)s->m2;
+    int32_t *d_totals = (int32_t *)s->m3;
+    int32_t totals[3] = {0, 0, 0};
+    if (g->max_deg >= C.long_min || g->max_out_deg >= C.long_min) {
+        k_table_counts<<<grid_of(s, (int64_t)n + 1, 256), 256, 0, st>>>(g->row_ptr, g->out_ptr, g->rows_sorted, n, C.n_in_long,
+                                                                        C.long_min, in_chunks, is_long, out_chunks);
+        int rc = exclusive_scan_i32(in_chunks, (int64_t)C.n_in_long + 1, in_first, tiles, st);
+        if (rc == FSGP_OK) rc = exclusive_scan_i32(is_long, (int64_t)n + 1, out_slot, tiles, st);
+        if (rc == FSGP_OK) rc = exclusive_scan_i32(out_chunks, (int64_t)n + 1, out_first, tiles, st);
+        if (rc) return rc;
+        k_table_totals<<<1, 1, 0, st>>>(in_first + C.n_in_long, out_slot + n, out_first + n, d_totals);
+        FSGP_CUDA(cudaMemcpyAsync(totals, d_totals, sizeof totals, cudaMemcpyDeviceToHost, st));
+        FSGP_CUDA(cudaStreamSynchronize(st));
     }
-    FSGP_CUDA(cudaDeviceSynchronize());
-    C.built = 1;
+    C.n_in_items = totals[0];
+    C.n_out_long = totals[1];
+    C.n_out_items = totals[2];
+    auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
+    const size_t b_in = al(sizeof(int4) * (size_t)C.n_in_items), b_out = al(sizeof(int4) * (size_t)C.n_out_items);
+    const size_t b_inv = al(sizeof(float) * (size_t)n), b_long = al(sizeof(int32_t) * (size_t)C.n_out_long);
+    const size_t b_acc = al(sizeof(float) * H * (size_t)std::max(C.n_in_long, C.n_out_long));
+    FSGP_CUDA(cudaMalloc(&C.mem, b_in + b_out + b_inv + b_long + b_acc));
+    uint8_t *p = (uint8_t *)C.mem;
+    C.in_items = (int4 *)p;
+    C.out_items = (int4 *)(p += b_in);
+    C.inv_din = (float *)(p += b_out);
+    C.out_long = (int32_t *)(p += b_inv);
+    C.acc = (float *)(p += b_long);
+    k_table_rows<<<grid_of(s, n, 256), 256, 0, st>>>(g->row_ptr, g->out_ptr, n, C.long_min, out_slot, C.inv_din, C.out_long);
+    if (C.n_in_items)
+        k_table_items<<<grid_of(s, C.n_in_items, 256), 256, 0, st>>>(g->row_ptr, g->rows_sorted, nullptr, in_first,
+                                                                     C.n_in_long, C.n_in_items, C.in_items);
+    if (C.n_out_items)
+        k_table_items<<<grid_of(s, C.n_out_items, 256), 256, 0, st>>>(g->out_ptr, nullptr, out_slot, out_first, n,
+                                                                      C.n_out_items, C.out_items);
+    cudaError_t e = b_acc ? cudaMemsetAsync(C.acc, 0, b_acc, st) : cudaSuccess;
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) {
+        cudaFree(C.mem);
+        return cuda_fail(e, "surrogate tables");
+    }
+    g->sgc = C;
     return FSGP_OK;
 }
 
@@ -1068,7 +1098,7 @@ int sg_prepare_inputs(fsgp_surrogate *s, const fsgp_graph *g, const int32_t *see
         if (seeds_host[i] < 0 || seeds_host[i] >= g->n) return fail(FSGP_EINVAL, "seed node out of range");
     int rc = sg_ensure(s, g->n);
     if (rc) return rc;
-    rc = sg_cache(g, s->sm_count);
+    rc = sg_cache(s, g, st);
     if (rc) return rc;
     k_features<<<grid_of(s, g->n, 256), 256, 0, st>>>(g->row_ptr, g->out_ptr, g->n, (float)beta, (float)gamma, s->x);
     if (ns > 0) {
@@ -1280,7 +1310,7 @@ extern "C" int fsgp_surrogate_screen(fsgp_surrogate *s, const fsgp_graph *g, con
     cudaStream_t caller = (cudaStream_t)stream;
     int rc = sg_ensure(s, g->n);
     if (rc) return rc;
-    rc = sg_cache(g, s->sm_count);
+    rc = sg_cache(s, g, caller);
     if (rc) return rc;
     // captures are not allowed on the legacy default stream: work on a private stream
     // ordered after the caller's work
