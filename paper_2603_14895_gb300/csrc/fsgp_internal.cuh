@@ -133,7 +133,11 @@ constexpr int kExecCacheSize = 4;
 // float32 accumulator (zero between uses).  long_min is a power of two, so that the long
 // in-rows are the first of the degree-bucket order, and at least four times the mean degree,
 // so that they stay few: BA n = 300k, one layer: 143 us with 256 (a tile of 255-arc rows
-// outlasts the rest), 71 with 32.
+// outlasts the rest), 71 with 32.  On larger graphs a tile's rows may be longer before they
+// outlast the rest, and split rows cost their partial sums: at least n / 2^14 (screening 8
+// candidates, ms with 32, 64, 128, 256: R-MAT, 6 arcs per node, n = 500k 2.90, 2.82, 3.12, 3.54;
+// n = 2M 10.6, 9.9, 9.4, 9.6; n = 4M 20.5, 19.4, 19.3, 18.1; 16 arcs per node, n = 4M 43.7, 41.1,
+// 40.4, 39.0, with the layer as two kernels 38.7).
 constexpr int32_t kSgLongMin = 32, kSgLongMax = 256;
 constexpr int32_t kSgChunk = 32;
 struct SgCache {

@@ -1019,7 +1019,7 @@ int sg_cache(fsgp_surrogate *s, const fsgp_graph *gc, cudaStream_t st) {
     SgCache C;
     const int32_t n = g->n;
     int bucket = 0;   // long_min is 2^bucket
-    while (C.long_min < kSgLongMax && (int64_t)C.long_min * n < 4 * g->nnz) C.long_min *= 2;
+    while (C.long_min < kSgLongMax && ((int64_t)C.long_min * n < 4 * g->nnz || (C.long_min << 14) < n)) C.long_min *= 2;
     while ((1 << bucket) < C.long_min) ++bucket;
     C.n_in_long = g->cls.bucket_start[bucket];
     int32_t *in_chunks = (int32_t *)s->h1, *in_first = (int32_t *)s->h2;
