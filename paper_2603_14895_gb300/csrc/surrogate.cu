@@ -104,41 +104,81 @@ __global__ void k_seed_bits(const int32_t *__restrict__ cand, int32_t k, int32_t
 // Screening: take back candidate *cur's seed features and set candidate *cur + 1's (at most
 // kClusterSeeds seeds), then advance *cur; past the last candidate only the taking back is
 // done.  One cluster of CTAs with cluster barriers between its phases (clear, count, write
-// the counts' logarithms) in place of seven launches of a microsecond or two each.
-constexpr int kSeedCtas = 8, kClusterSeeds = 64;
+// the counts' logarithms) in place of seven launches of a microsecond or two each.  The
+// seeds' out-arcs are taken as one list, the cluster's threads side by side: with a CTA per
+// seed the largest hub held up the candidate, and eight CTAs are fewer than the seeds
+// (screening 16 candidates of the 64 largest hubs: R-MAT n = 600k 10.9 ms with a CTA per seed,
+// 9.1 so; n = 4M 116 and 104; 8 mixed candidates, R-MAT n = 2M, 16 arcs per node: 21.0 and 20.2).
+constexpr int kSeedCtas = 8, kSeedThreads = 256, kClusterSeeds = 64;
 __device__ __forceinline__ void cluster_barrier() {
     __threadfence();
     asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-__global__ void __cluster_dims__(kSeedCtas, 1, 1) __launch_bounds__(256)
+__global__ void __cluster_dims__(kSeedCtas, 1, 1) __launch_bounds__(kSeedThreads)
     k_seed_next(const int32_t *__restrict__ cand, int32_t k, int32_t n_cand, int32_t *cur,
                 const int32_t *__restrict__ out_ptr, const int32_t *__restrict__ out_dst, int32_t *cnt, bf16 *x) {
+    // [0] candidate c - 1, [1] candidate c: each seed's first out-arc, and the out-arcs before it
+    __shared__ int32_t s_beg[2][kClusterSeeds];
+    __shared__ int64_t s_off[2][kClusterSeeds + 1];
     const int c = *(volatile int32_t *)cur + 1;
-    auto each_out = [&](int cc, auto f) {
-        for (int i = blockIdx.x; i < k; i += gridDim.x) {
-            const int32_t sd = cand[(size_t)cc * k + i];
-            for (int32_t a = out_ptr[sd] + threadIdx.x; a < out_ptr[sd + 1]; a += blockDim.x) f(out_dst[a]);
+    const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (q < 2) {   // two seeds per lane
+        const int cc = c - 1 + q;
+        int32_t b[2] = {0, 0}, d[2] = {0, 0};
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int i = 2 * lane + j;
+            if (cc >= 0 && cc < n_cand && i < k) {
+                const int32_t sd = __ldg(cand + (size_t)cc * k + i);
+                b[j] = __ldg(out_ptr + sd);
+                d[j] = __ldg(out_ptr + sd + 1) - b[j];
+                if (blockIdx.x == 0 && q == 0) x[(size_t)sd * F0] = __float2bfloat16(0.f);
+            }
+        }
+        int64_t sum = (int64_t)d[0] + d[1];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int64_t up = __shfl_up_sync(0xffffffffu, sum, o);
+            if (lane >= o) sum += up;
+        }
+        s_beg[q][2 * lane] = b[0];
+        s_beg[q][2 * lane + 1] = b[1];
+        s_off[q][2 * lane + 1] = sum - d[1];
+        s_off[q][2 * lane + 2] = sum;
+        if (lane == 0) s_off[q][0] = 0;
+    }
+    __syncthreads();
+    // f(target) for the out-arcs of candidate c - 1 + w, four of a thread's targets in flight
+    auto each_out = [&](int w, auto f) {
+        const int64_t total = s_off[w][kClusterSeeds], step = (int64_t)kSeedCtas * kSeedThreads;
+        int i = 0;   // seed of the arc at hand
+        for (int64_t t = (int64_t)blockIdx.x * kSeedThreads + threadIdx.x; t < total; t += 4 * step) {
+            int32_t v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int64_t a = t + u * step;
+                v[u] = -1;
+                if (a < total) {
+                    while (s_off[w][i + 1] <= a) ++i;
+                    v[u] = __ldg(out_dst + (s_beg[w][i] + (a - s_off[w][i])));
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (v[u] >= 0) f(v[u]);
         }
     };
-    if (c > 0) {
-        if (blockIdx.x == 0)
-            for (int i = threadIdx.x; i < k; i += blockDim.x)
-                x[(size_t)cand[(size_t)(c - 1) * k + i] * F0] = __float2bfloat16(0.f);
-        each_out(c - 1, [&](int32_t v) {
-            cnt[v] = 0;
-            x[(size_t)v * F0 + 5] = __float2bfloat16(0.f);
-        });
-    }
+    each_out(0, [&](int32_t v) {
+        cnt[v] = 0;
+        x[(size_t)v * F0 + 5] = __float2bfloat16(0.f);
+    });
     cluster_barrier();
-    if (c < n_cand) {
-        if (blockIdx.x == 0)
-            for (int i = threadIdx.x; i < k; i += blockDim.x)
-                x[(size_t)cand[(size_t)c * k + i] * F0] = __float2bfloat16(1.f);
-        each_out(c, [&](int32_t v) { atomicAdd(&cnt[v], 1); });
-    }
+    if (c < n_cand && blockIdx.x == 0)
+        for (int i = threadIdx.x; i < k; i += blockDim.x)
+            x[(size_t)cand[(size_t)c * k + i] * F0] = __float2bfloat16(1.f);
+    each_out(1, [&](int32_t v) { atomicAdd(&cnt[v], 1); });
     cluster_barrier();
-    if (c < n_cand)
-        each_out(c, [&](int32_t v) { x[(size_t)v * F0 + 5] = __float2bfloat16(log1pf((float)__ldcg(cnt + v))); });
+    each_out(1, [&](int32_t v) { x[(size_t)v * F0 + 5] = __float2bfloat16(log1pf((float)__ldcg(cnt + v))); });
     if (blockIdx.x == 0 && threadIdx.x == 0) *cur = c;
 }
 
@@ -1348,7 +1388,7 @@ extern "C" int fsgp_surrogate_screen(fsgp_surrogate *s, const fsgp_graph *g, con
         const int gk = std::min<int32_t>(k, 1024);
         const bool clustered = k <= kClusterSeeds;
         if (clustered) {
-            k_seed_next<<<kSeedCtas, 256, 0, st>>>(d_cand, k, n_cand, s->cur, g->out_ptr, g->out_dst, s->cnt, s->x);
+            k_seed_next<<<kSeedCtas, kSeedThreads, 0, st>>>(d_cand, k, n_cand, s->cur, g->out_ptr, g->out_dst, s->cnt, s->x);
         } else {
             k_seed_bits<<<1, 256, 0, st>>>(d_cand, k, s->cur, 1.f, 0, s->x);
             k_seed_count<<<gk, 256, 0, st>>>(d_cand, k, s->cur, g->out_ptr, g->out_dst, 1, s->cnt);
@@ -1369,7 +1409,7 @@ extern "C" int fsgp_surrogate_screen(fsgp_surrogate *s, const fsgp_graph *g, con
         }
         for (int32_t c = 0; c < n_cand && e == cudaSuccess; ++c) e = cudaGraphLaunch(exec, st);
         if (clustered)   // take the last candidate's seed features back
-            k_seed_next<<<kSeedCtas, 256, 0, st>>>(d_cand, k, n_cand, s->cur, g->out_ptr, g->out_dst, s->cnt, s->x);
+            k_seed_next<<<kSeedCtas, kSeedThreads, 0, st>>>(d_cand, k, n_cand, s->cur, g->out_ptr, g->out_dst, s->cnt, s->x);
         if (e == cudaSuccess) e = cudaMemcpyAsync(scores_out, d_scores, sizeof(float) * (size_t)n_cand, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         cudaGraphExecDestroy(exec);
