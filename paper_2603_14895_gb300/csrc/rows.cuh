@@ -288,11 +288,15 @@ __device__ __forceinline__ uint32_t pick(const uint32_t (&c)[V][B], int i, int b
 }
 
 // Resident CTAs per SM the register allocation is bounded for: wider thread words hold
-// more counters.  Three with two words per thread: a fourth leaves 64 registers, which spill
-// in the gather (R-MAT n = 8M, R = 256, a SIS step: team rows 602 us with four, 541 with
-// three, 669 with five; warp rows 333 with three, 377 with two, 586 with four).
-template <int V, bool WIDE>
-constexpr int min_ctas() { return V == 4 ? 2 : (V == 2 ? 3 : 4); }
+// more counters.  Three with one and two words per thread: their 80 registers hold the team
+// rows but for 4 to 36 bytes of spill stores, the warp rows with 16 counter planes per word
+// but for 28 to 104 (SIS and SIR); a fourth leaves 64 registers (R-MAT n = 8M, R = 256, a SIS
+// step with two words: team rows 602 us with four, 541 with three, 669 with five; warp rows 333
+// with three, 377 with two, 586 with four.  One word, R = 32, T = 40, ms with three, four,
+// five: SIS, R-MAT n = 4.2M 24.6, 26.2, 28.1; LT 28.3, 29.5, 34.2; SIR, BA n = 2M 10.7, 11.1,
+// 13.5).
+template <int V>
+constexpr int min_ctas() { return V == 4 ? 2 : 3; }
 
 // Row kernel that decides every word in the thread that gathered it (count models; SWIR,
 // whose second draw depends on its first): one work item is one slice (TEAM*V words) of one
@@ -1098,7 +1102,7 @@ constexpr size_t FusedBytes = std::max(TileBytes<MODEL, V, TEAM, true, kSmallBit
                                        TileBytes<MODEL, V, TEAM, false, kSmallBits>);
 
 template <int MODEL, int V, int TEAM, bool WARP_ROW, int BT = kSmallBits>
-__global__ void __launch_bounds__(kBlock, min_ctas<V, WARP_ROW>()) k_rows(StepArgs A, int which) {
+__global__ void __launch_bounds__(kBlock, min_ctas<V>()) k_rows(StepArgs A, int which) {
     extern __shared__ __align__(16) uint8_t s_dyn[];
     __shared__ unsigned long long s_pc[kPC * kMaxSets];
     constexpr size_t tile = TileBytes<MODEL, V, TEAM, WARP_ROW, BT>;
@@ -1194,7 +1198,7 @@ __global__ void __launch_bounds__(kBlock, 2)
 //     on decides the same way), so its other chunks need not be read;
 //   pass 2 (SIR/SIS): the other chunks of the slices not flagged.
 template <int MODEL, int V, int TEAM>
-__global__ void __launch_bounds__(kBlock, min_ctas<V, true>()) k_hub_chunks(StepArgs A, int pass) {
+__global__ void __launch_bounds__(kBlock, min_ctas<V>()) k_hub_chunks(StepArgs A, int pass) {
     __shared__ uint32_t s_cnt[kMaxR];
     constexpr int B = kWideBits;
     constexpr int TPB = kBlock / TEAM;
