@@ -224,17 +224,20 @@ __device__ __forceinline__ void mark_round(const StepArgs &A, int32_t x) {
             if (d < A.hub_min_deg) cls = d > A.small_max_deg ? 1 : 0;
         }
     }
+    // both classes' counts in one addition: with a bound within the degrees that are hit most
+    // often (cascades: 63) nearly every round has rows of either class (R-MAT n = 2M, R = 256,
+    // T = 50, marking in a run: IC 47.9 ms with an addition per class, 44.5 so; LT 62.3 and 58.6)
     const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
-        const unsigned m = __ballot_sync(0xffffffffu, cls == c);
-        if (!m) continue;
-        const int leader = __ffs(m) - 1;
-        uint32_t base = 0;
-        if (lane == leader) base = atomicAdd(&A.ctl->cand_n[c], (uint32_t)__popc(m));
-        base = __shfl_sync(0xffffffffu, base, leader);
-        if (cls == c) (c ? A.cand_mid : A.cand_small)[base + __popc(m & ((1u << lane) - 1u))] = x;
-    }
+    const unsigned m0 = __ballot_sync(0xffffffffu, cls == 0), m1 = __ballot_sync(0xffffffffu, cls == 1);
+    if (!(m0 | m1)) return;
+    unsigned long long base = 0;
+    if (lane == 0)
+        base = atomicAdd(reinterpret_cast<unsigned long long *>(A.ctl->cand_n),
+                         (unsigned long long)__popc(m0) | (unsigned long long)__popc(m1) << 32);
+    base = __shfl_sync(0xffffffffu, base, 0);
+    const unsigned below = (1u << lane) - 1u;
+    if (cls == 0) A.cand_small[(uint32_t)base + __popc(m0 & below)] = x;
+    if (cls == 1) A.cand_mid[(uint32_t)(base >> 32) + __popc(m1 & below)] = x;
 }
 
 __global__ void __launch_bounds__(kBlock) k_mark(StepArgs A) {
@@ -572,8 +575,8 @@ static int run_wave(fsgp_graph *g, int model, int ic_mode, int weighted, const S
     }
     // degree classes
     // (cascades run on frontier lists, whose few rows want a warp each: BA n = 1M, IC,
-    // R = 1024: 50.8 ms with 255, 44.7 with 63; LT, n = 700k: 18.0 and 15.9; where the steps
-    // are dense it costs a little: R-MAT n = 2M, IC, R = 256: 93.9 and 98.9)
+    // R = 1024: 50.8 ms with 255, 44.7 with 63; LT, n = 700k: 18.0 and 15.9; where the lists are
+    // long it costs a little: R-MAT n = 2M, IC, R = 256: 64.8 and 65.5)
     int small_max = opt.small_max_deg > 0 ? opt.small_max_deg : (cascade ? 63 : 255);
     int hub_min = fuse ? 65536 : (opt.hub_min_deg > 0 ? opt.hub_min_deg : kHubMinDeg);
     int bs = bitlen(small_max + 1) - 1;              // small: d <= 2^bs - 1

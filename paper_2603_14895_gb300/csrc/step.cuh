@@ -37,7 +37,8 @@ struct Ctl {
     int32_t err;           // a bounded wait of the persistent step loop ran out
     uint32_t list_n[2];    // rows listed for the next step (by step parity)
     uint64_t push_outdeg[2];
-    uint32_t cand_n[2];    // sparse candidates: 0 = small rows, 1 = mid rows
+    alignas(8) uint32_t cand_n[2];   // sparse candidates: 0 = small rows, 1 = mid rows (added to
+                           // as one 64-bit word, small rows in its low half)
     int32_t dense_steps;   // steps run on the full row lists
     int32_t sparse_steps;  // steps run on the frontier lists
     int32_t build_list;    // the current step lists its rows for the next step
