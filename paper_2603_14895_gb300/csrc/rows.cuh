@@ -298,9 +298,8 @@ __device__ __forceinline__ uint32_t pick(const uint32_t (&c)[V][B], int i, int b
 template <int V>
 constexpr int min_ctas() { return V == 4 ? 2 : 3; }
 
-// Row kernel that decides every word in the thread that gathered it (count models; SWIR,
-// whose second draw depends on its first): one work item is one slice (TEAM*V words) of one
-// row.
+// Row kernel that decides every word in the thread that gathered it (SWIR, whose second draw
+// depends on its first): one work item is one slice (TEAM*V words) of one row.
 // WARP_ROW = false: one team per item; true: one warp per item.
 // BT: counter bits of a team kernel, sized to its rows' in-degree bound (fewer planes =
 // fewer registers and cheaper counting and grouping).
@@ -313,11 +312,10 @@ constexpr int min_ctas() { return V == 4 ? 2 : 3; }
 template <int MODEL, int V, int TEAM, bool WARP_ROW, int BT, bool CG, int B, int AG>
 __device__ __forceinline__ void rows_body(const StepArgs &A, int which, int32_t *s_lane, unsigned long long *s_pc,
                                           int bid, int nb) {
-    static_assert(ModelTraits<MODEL>::counts, "arc models go through the warp tile");
+    static_assert(!ModelTraits<MODEL>::tiled && ModelTraits<MODEL>::planes == 3, "the other models go through the warp tile");
     static_assert(AG == 1 || (!WARP_ROW && V == 1 && TEAM * AG <= 32), "arc groups: team rows within a warp");
     constexpr int TPW = 32 / TEAM;
     constexpr int SW = TEAM * V;
-    constexpr int P = ModelTraits<MODEL>::planes;
     const Ctl *C = A.ctl;
     if (*(volatile const int32_t *)&C->stop) return;
     const bool sparse = *(volatile const int32_t *)&C->sparse != 0;
@@ -375,18 +373,13 @@ __device__ __forceinline__ void rows_body(const StepArgs &A, int which, int32_t 
             }
             ctx_slice = slice;
         }
-        // lanes that can change through their in-arcs: S (SIR/SIS) or inactive (IC/LT)
+        // lanes that can change through their in-arcs
         uint32_t need[V];
         {
-            Vec<V> a = has_row ? ld_vec<V, CG>(A.cur + off) : Vec<V>{};
-            Vec<V> b{}, e{};
-            if (P >= 2 && MODEL != FSGP_IC && MODEL != FSGP_LT && has_row) b = ld_vec<V, CG>(A.cur + A.plane_words + off);
-            if (MODEL == FSGP_SEIR && has_row) e = ld_vec<V, CG>(A.cur + 2 * A.plane_words + off);
+            const Vec<V> a = has_row ? ld_vec<V, CG>(A.cur + off) : Vec<V>{};
+            const Vec<V> b = has_row ? ld_vec<V, CG>(A.cur + A.plane_words + off) : Vec<V>{};
 #pragma unroll
-            for (int i = 0; i < V; ++i) {
-                const uint32_t vm = has_row ? x[i].vm : 0u;
-                need[i] = need_of<MODEL>(vm, a.w[i], b.w[i], e.w[i]);
-            }
+            for (int i = 0; i < V; ++i) need[i] = need_of<MODEL>(has_row ? x[i].vm : 0u, a.w[i], b.w[i], 0u);
         }
         uint32_t any_need = 0u;
 #pragma unroll
@@ -457,12 +450,12 @@ __device__ __forceinline__ void rows_body(const StepArgs &A, int which, int32_t 
                 for (int q = 1; q < V; ++q)
                     if (i == q) xw = x[q];
                 const uint32_t s0 = ld_word<CG>(A.cur + off + i);
-                const uint32_t s1 = P >= 2 ? ld_word<CG>(A.cur + A.plane_words + off + i) : 0u;
-                const uint32_t s2 = P >= 3 ? ld_word<CG>(A.cur + 2 * A.plane_words + off + i) : 0u;
+                const uint32_t s1 = ld_word<CG>(A.cur + A.plane_words + off + i);
+                const uint32_t s2 = ld_word<CG>(A.cur + 2 * A.plane_words + off + i);
                 const WordOut o = update_word<MODEL, B>(A, node, xw, s0, s1, s2, end - beg, cw, 0u);
                 A.nxt[off + i] = o.n0;
-                if (P >= 2) A.nxt[A.plane_words + off + i] = o.n1;
-                if (P >= 3) A.nxt[2 * A.plane_words + off + i] = o.n2;
+                A.nxt[A.plane_words + off + i] = o.n1;
+                A.nxt[2 * A.plane_words + off + i] = o.n2;
 #pragma unroll
                 for (int q = 0; q < V; ++q) {
                     if (i == q) {
@@ -473,8 +466,8 @@ __device__ __forceinline__ void rows_body(const StepArgs &A, int which, int32_t 
                 }
                 if (lanes_on) {
                     lane_deltas(s_lane, w0 + i, s0, o.n0);
-                    if (P >= 2) lane_deltas(s_lane + nl, w0 + i, s1, o.n1);
-                    if (P >= 3) lane_deltas(s_lane + 2 * nl, w0 + i, s2, o.n2);
+                    lane_deltas(s_lane + nl, w0 + i, s1, o.n1);
+                    lane_deltas(s_lane + 2 * nl, w0 + i, s2, o.n2);
                 }
                 fl |= word_flags<MODEL>(o, s0, s1, s2);
             }
@@ -487,15 +480,14 @@ __device__ __forceinline__ void rows_body(const StepArgs &A, int which, int32_t 
             // own state again (L1/L2-resident): not kept live across the gather
             uint32_t s0[V], s1[V], s2[V];
             {
-                Vec<V> a = ld_vec<V, CG>(A.cur + off);
-                Vec<V> b{}, e{};
-                if (P >= 2) b = ld_vec<V, CG>(A.cur + A.plane_words + off);
-                if (P >= 3) e = ld_vec<V, CG>(A.cur + 2 * A.plane_words + off);
+                const Vec<V> a = ld_vec<V, CG>(A.cur + off);
+                const Vec<V> b = ld_vec<V, CG>(A.cur + A.plane_words + off);
+                const Vec<V> e = ld_vec<V, CG>(A.cur + 2 * A.plane_words + off);
 #pragma unroll
                 for (int i = 0; i < V; ++i) {
                     s0[i] = a.w[i];
-                    s1[i] = P >= 2 ? b.w[i] : 0u;
-                    s2[i] = P >= 3 ? e.w[i] : 0u;
+                    s1[i] = b.w[i];
+                    s2[i] = e.w[i];
                 }
             }
             uint32_t n0[V], n1[V], n2[V];
@@ -510,14 +502,14 @@ __device__ __forceinline__ void rows_body(const StepArgs &A, int which, int32_t 
                 d2[i] += __popc(o.n2) - __popc(s2[i]);
                 if (lanes_on) {
                     lane_deltas(s_lane, w0 + i, s0[i], o.n0);
-                    if (P >= 2) lane_deltas(s_lane + nl, w0 + i, s1[i], o.n1);
-                    if (P >= 3) lane_deltas(s_lane + 2 * nl, w0 + i, s2[i], o.n2);
+                    lane_deltas(s_lane + nl, w0 + i, s1[i], o.n1);
+                    lane_deltas(s_lane + 2 * nl, w0 + i, s2[i], o.n2);
                 }
                 fl |= word_flags<MODEL>(o, s0[i], s1[i], s2[i]);
             }
             st_vec<V>(A.nxt + off, n0);
-            if (P >= 2) st_vec<V>(A.nxt + A.plane_words + off, n1);
-            if (P >= 3) st_vec<V>(A.nxt + 2 * A.plane_words + off, n2);
+            st_vec<V>(A.nxt + A.plane_words + off, n1);
+            st_vec<V>(A.nxt + 2 * A.plane_words + off, n2);
         }
 #pragma unroll
         for (int o = 1; o < TEAM; o <<= 1) fl |= __shfl_xor_sync(0xffffffffu, fl, o);
@@ -525,7 +517,7 @@ __device__ __forceinline__ void rows_body(const StepArgs &A, int which, int32_t 
         const bool leader = writer && tl == 0;
         const bool want = leader && fl != 0u;
         if (want && (fl & 1u)) acc.push_deg += out_degree(A, v);
-        if (A.prof_bytes && leader) acc.bytes += row_bytes(SW, P, any_need != 0u, end - beg);
+        if (A.prof_bytes && leader) acc.bytes += row_bytes(SW, 3, any_need != 0u, end - beg);
         list_append(A, build, want, (int32_t)((uint32_t)v | ((fl & 1u) ? kPushBit : 0u)), list_slot);
         if (sparse && leader) atomicAnd(&A.bitmap[v >> 5], ~(1u << (v & 31)));
     }
@@ -1457,29 +1449,21 @@ __global__ void __launch_bounds__(kBlock) k_hub_finalize(StepArgs A) {
 // k_rows).  Most rows of a power-law graph
 // are of this kind and carry little gather work, so the cost is the chain of dependent
 // loads per row: one THREAD per item (a slice of SWL <= 8 words of one row) keeps four
-// to eight times as many rows in flight per SM as a team per row.  The thread loads its
-// own words and the (at most three) sources' words at once, stages them in shared memory,
-// and then decides its words one at a time through a single, non-unrolled copy of the
-// per-word update (counts of at most 3 need 2-bit counters).
+// to eight times as many rows in flight per SM as a team per row.
+// lane_body (SWIR): the thread loads its own words and the (at most three) sources' words at
+// once, stages them in shared memory, and then decides its words one at a time through a
+// single, non-unrolled copy of the per-word update (counts of at most 3 need 2-bit counters).
+// lane_tile (the other models): the same rows through the warp tile.
 constexpr int kLaneMaxDeg = 3;
 template <int SWL, int NP>
 struct LaneStage {
     uint32_t v[NP + 3][SWL][kBlock];   // own planes, then the sources' words (x0, x1, x2)
 };
 
-// Lanes that change on their own (without in-arcs): infectious lanes that may recover,
-// newly active lanes that stop being new (IC / LT), exposed lanes (SEIR / SEIS).
-template <int MODEL>
-__device__ __forceinline__ uint32_t self_lanes(uint32_t s0, uint32_t s1, uint32_t s2) {
-    if constexpr (MODEL == FSGP_IC || MODEL == FSGP_LT) return s1;
-    else if constexpr (MODEL == FSGP_SEIR) return s0 | s2;
-    else if constexpr (MODEL == FSGP_SEIS) return s0 | s1;
-    else return s0;
-}
-
 template <int MODEL, int SWL>
 __device__ __forceinline__ void lane_body(const StepArgs &A, uint8_t *smem, int32_t *s_lane, unsigned long long *s_pc) {
-    constexpr int P = ModelTraits<MODEL>::planes;
+    static_assert(!ModelTraits<MODEL>::tiled && ModelTraits<MODEL>::planes == 3, "the other models go through the warp tile");
+    constexpr int P = 3;
     LaneStage<SWL, P> &st = *reinterpret_cast<LaneStage<SWL, P> *>(smem);
     const Ctl *C = A.ctl;
     if (*(volatile const int32_t *)&C->stop) return;
@@ -1503,7 +1487,7 @@ __device__ __forceinline__ void lane_body(const StepArgs &A, uint8_t *smem, int3
     for (int64_t item = (int64_t)blockIdx.x * blockDim.x + tid; item - tid < nitems;
          item += (int64_t)gridDim.x * blockDim.x) {
         const bool has = item < nitems;
-        int32_t v = 0, beg = 0, d = 0;   // v: new id
+        int32_t v = 0, d = 0;            // v: new id
         uint32_t node = 0u;              // Philox subject
         int w0 = 0;
         uint32_t busy = 0u;
@@ -1521,7 +1505,6 @@ __device__ __forceinline__ void lane_body(const StepArgs &A, uint8_t *smem, int3
             node = (uint32_t)e.x;
             const int32_t u[kLaneMaxDeg] = {e.y, e.z, e.w};
             d = (e.y >= 0) + (e.z >= 0) + (e.w >= 0);
-            if (!ModelTraits<MODEL>::counts && d > 0) beg = __ldg(A.arc0 + v);   // arc positions key the draws
             const size_t off = (size_t)v * A.Wn + w0;
             // own words and sources' words, 4 (or fewer) words per load; `busy` records
             // whether any lane can change at this step (an infected lane to recover, or a
@@ -1530,15 +1513,14 @@ __device__ __forceinline__ void lane_body(const StepArgs &A, uint8_t *smem, int3
             for (int q = 0; q < SWL; q += (SWL < 4 ? SWL : 4)) {
                 constexpr int VL = SWL < 4 ? SWL : 4;
                 const Vec<VL> a = ldg_vec<VL>(A.cur + off + q);
-                Vec<VL> bb{}, ee{};
-                if (P >= 2) bb = ldg_vec<VL>(A.cur + A.plane_words + off + q);
-                if (P >= 3) ee = ldg_vec<VL>(A.cur + 2 * A.plane_words + off + q);
+                const Vec<VL> bb = ldg_vec<VL>(A.cur + A.plane_words + off + q);
+                const Vec<VL> ee = ldg_vec<VL>(A.cur + 2 * A.plane_words + off + q);
                 uint32_t xs[VL];
 #pragma unroll
                 for (int i = 0; i < VL; ++i) {
                     st.v[0][q + i][tid] = a.w[i];
-                    if (P >= 2) st.v[1][q + i][tid] = bb.w[i];
-                    if (P >= 3) st.v[2][q + i][tid] = ee.w[i];
+                    st.v[1][q + i][tid] = bb.w[i];
+                    st.v[2][q + i][tid] = ee.w[i];
                     xs[i] = 0u;
                 }
 #pragma unroll
@@ -1553,9 +1535,8 @@ __device__ __forceinline__ void lane_body(const StepArgs &A, uint8_t *smem, int3
                 }
 #pragma unroll
                 for (int i = 0; i < VL; ++i) {
-                    const uint32_t s0 = a.w[i], s1 = P >= 2 ? bb.w[i] : 0u, s2 = P >= 3 ? ee.w[i] : 0u;
-                    // a lane changes on its own, or can change with a set source lane
-                    busy |= self_lanes<MODEL>(s0, s1, s2) | (need_of<MODEL>(~0u, s0, s1, s2) & xs[i]);
+                    // an infectious lane may recover, and a set source lane can change another
+                    busy |= a.w[i] | (need_of<MODEL>(~0u, a.w[i], bb.w[i], ee.w[i]) & xs[i]);
                 }
             }
         }
@@ -1579,31 +1560,16 @@ __device__ __forceinline__ void lane_body(const StepArgs &A, uint8_t *smem, int3
             for (int i = 0; i < SWL; ++i) {
                 const WordCtx x = word_ctx(A, w0 + i);
                 const uint32_t s0 = st.v[0][i][tid];
-                const uint32_t s1 = P >= 2 ? st.v[1][i][tid] : 0u;
-                const uint32_t s2 = P >= 3 ? st.v[2][i][tid] : 0u;
+                const uint32_t s1 = st.v[1][i][tid];
+                const uint32_t s2 = st.v[2][i][tid];
                 const uint32_t x0 = st.v[P][i][tid], x1 = st.v[P + 1][i][tid], x2 = st.v[P + 2][i][tid];
                 const uint32_t need = need_of<MODEL>(x.vm, s0, s1, s2);
-                uint32_t c[2] = {0u, 0u}, newly = 0u;
-                if constexpr (!ModelTraits<MODEL>::counts) {
-                    constexpr bool W = ModelTraits<MODEL>::weighted;
-                    const uint64_t thr = W ? 0ull : ic_threshold(A, x.s, d);
-                    const uint32_t xs[kLaneMaxDeg] = {x0, x1, x2};
-#pragma unroll
-                    for (int j = 0; j < kLaneMaxDeg; ++j) {
-                        const uint32_t m = xs[j] & need & ~newly;
-                        if (m)
-                            newly |= lanes_u_less(m, W ? arc_threshold(A, x.s, beg + j) : thr, (uint32_t)(beg + j),
-                                                  A.t, x.g, W ? TAG_ARC_INFECT : TAG_IC_EDGE, x.k0, x.k1);
-                    }
-                } else {
-                    // counts of set source lanes (at most 3): two bit-planes
-                    c[0] = (x0 ^ x1 ^ x2) & need;
-                    c[1] = ((x0 & x1) | (x2 & (x0 ^ x1))) & need;
-                }
-                const WordOut o = update_word<MODEL, 2>(A, node, x, s0, s1, s2, d, c, newly);
+                // counts of set source lanes (at most 3): two bit-planes
+                const uint32_t c[2] = {(x0 ^ x1 ^ x2) & need, ((x0 & x1) | (x2 & (x0 ^ x1))) & need};
+                const WordOut o = update_word<MODEL, 2>(A, node, x, s0, s1, s2, d, c, 0u);
                 st.v[0][i][tid] = o.n0;
-                if (P >= 2) st.v[1][i][tid] = o.n1;
-                if (P >= 3) st.v[2][i][tid] = o.n2;
+                st.v[1][i][tid] = o.n1;
+                st.v[2][i][tid] = o.n2;
                 if (x.s != cur_s) {
                     if (cur_s >= 0) set_acc_add(s_pc, cur_s, dd0, dd1, dd2);
                     cur_s = x.s;
@@ -1614,8 +1580,8 @@ __device__ __forceinline__ void lane_body(const StepArgs &A, uint8_t *smem, int3
                 dd2 += __popc(o.n2) - __popc(s2);
                 if (lanes_on) {
                     lane_deltas(s_lane, w0 + i, s0, o.n0);
-                    if (P >= 2) lane_deltas(s_lane + nl, w0 + i, s1, o.n1);
-                    if (P >= 3) lane_deltas(s_lane + 2 * nl, w0 + i, s2, o.n2);
+                    lane_deltas(s_lane + nl, w0 + i, s1, o.n1);
+                    lane_deltas(s_lane + 2 * nl, w0 + i, s2, o.n2);
                 }
                 fl |= word_flags<MODEL>(o, s0, s1, s2);
             }
