@@ -533,10 +533,10 @@ __device__ __forceinline__ void rows_body(const StepArgs &A, int which, int32_t 
 // Shape of one warp's tile: SPP word slots per pass (one row slice per team, or one row
 // slice per warp), NP passes.  128 slots keep the queues several batches of 32 long;
 // the wide rows' 16 counter planes take 64.
-template <int MODEL, int V, int TEAM, bool WARP_ROW, int BT>
+template <int MODEL, int V, int TEAM, bool WARP_ROW, int BT, int WB = kWideBits>
 struct TileShape {
     static constexpr bool counts = ModelTraits<MODEL>::counts;
-    static constexpr int B = counts ? (WARP_ROW ? kWideBits : BT) : 1;
+    static constexpr int B = counts ? (WARP_ROW ? WB : BT) : 1;
     static constexpr int SW = TEAM * V;
     static constexpr int SPP = WARP_ROW ? SW : 32 * V;
     static constexpr int RPP = WARP_ROW ? 1 : 32 / TEAM;
@@ -641,10 +641,10 @@ __device__ __forceinline__ void draw_counts(const StepArgs &A, TileT &T, int n, 
     __syncwarp();
 }
 
-template <int MODEL, class TileT, class CtxFn>
+template <int MODEL, bool PAIR, class TileT, class CtxFn>
 __device__ __forceinline__ void draw_arc_items(const StepArgs &A, TileT &T, int na, int lane, CtxFn ctx) {
     constexpr bool W = ModelTraits<MODEL>::weighted;
-    draw_arcs(A, T.c[0], T.arc_eq, T.arc_pos, T.arc_slot, na, W ? TAG_ARC_INFECT : TAG_IC_EDGE, lane, ctx,
+    draw_arcs<PAIR>(A, T.c[0], T.arc_eq, T.arc_pos, T.arc_slot, na, W ? TAG_ARC_INFECT : TAG_IC_EDGE, lane, ctx,
               [&A, &T](int row, uint32_t pos, const SetParams &sp) -> uint64_t {
                   if constexpr (W) return arc_thr(__ldg(&sp.beta_f), __ldg(A.arc_w + pos));
                   else if (A.ic_mode == FSGP_IC_WEIGHTED_CASCADE) return (uint64_t)T.thr[row] + 1ull;
@@ -653,12 +653,12 @@ __device__ __forceinline__ void draw_arc_items(const StepArgs &A, TileT &T, int 
 }
 
 // The tile's draws after its gather (queue lengths nq, nf, na).
-template <int MODEL, int B, class TileT, class CtxFn>
+template <int MODEL, int B, bool PAIR, class TileT, class CtxFn>
 __device__ __forceinline__ void draw_tile(const StepArgs &A, TileT &T, int nq, const int (&nf)[2], int na, int lane,
                                           CtxFn ctx) {
     __syncwarp();
     if constexpr (ModelTraits<MODEL>::counts) draw_counts<MODEL, B>(A, T, nq, lane, ctx);
-    else draw_arc_items<MODEL>(A, T, na, lane, ctx);
+    else draw_arc_items<MODEL, PAIR>(A, T, na, lane, ctx);
     if constexpr (ModelTraits<MODEL>::fixed_draws >= 1)
         draw_fixed<false>(A, T.f[0], T.eq(), T.qf[0], nf[0], lane, ctx);
     if constexpr (ModelTraits<MODEL>::fixed_draws >= 2)
@@ -735,7 +735,7 @@ __device__ __forceinline__ void gather_push(const StepArgs &A, TileT &T, int64_t
         for (int j = 0; j < 4; ++j) {
             if (na > NARC - 32 * V) {
                 __syncwarp();
-                draw_arc_items<MODEL>(A, T, na, lane, ctx);
+                draw_arc_items<MODEL, CG>(A, T, na, lane, ctx);
                 na = 0;
                 // lanes already reached need no more draws
                 bool left = false;
@@ -767,10 +767,10 @@ __device__ __forceinline__ void gather_push(const StepArgs &A, TileT &T, int64_t
 // WARP_ROW = false: one team per item; true: one warp per item.  which: as in rows_body.
 // CG: state planes through L2 only (persistent step loop).  bid of nb: the CTA's place among
 // those that work on these rows.
-template <int MODEL, int V, int TEAM, bool WARP_ROW, int BT, bool CG>
+template <int MODEL, int V, int TEAM, bool WARP_ROW, int BT, bool CG, int WB>
 __device__ __forceinline__ void rows_tile(const StepArgs &A, int which, uint8_t *smem, int32_t *s_lane,
                                           unsigned long long *s_pc, int bid, int nb) {
-    using S = TileShape<MODEL, V, TEAM, WARP_ROW, BT>;
+    using S = TileShape<MODEL, V, TEAM, WARP_ROW, BT, WB>;
     constexpr int B = S::B;
     constexpr int TPW = 32 / TEAM;
     constexpr int SW = TEAM * V;
@@ -966,7 +966,7 @@ __device__ __forceinline__ void rows_tile(const StepArgs &A, int which, uint8_t 
                 }
             }
         }
-        draw_tile<MODEL, B>(A, T, nq, nf, na, lane, ctx);
+        draw_tile<MODEL, B, CG>(A, T, nq, nf, na, lane, ctx);
         __syncwarp();
         // next states
         if constexpr (!WARP_ROW) {
@@ -1082,7 +1082,7 @@ __device__ __forceinline__ void rows_tile(const StepArgs &A, int which, uint8_t 
 template <int MODEL, int V, int TEAM, bool WARP_ROW, int BT, bool CG, int WB = kWideBits, int AG = 1>
 __device__ __forceinline__ void rows_class(const StepArgs &A, int which, uint8_t *smem, int32_t *s_lane,
                                            unsigned long long *s_pc, int bid, int nb) {
-    if constexpr (ModelTraits<MODEL>::tiled) rows_tile<MODEL, V, TEAM, WARP_ROW, BT, CG>(A, which, smem, s_lane, s_pc, bid, nb);
+    if constexpr (ModelTraits<MODEL>::tiled) rows_tile<MODEL, V, TEAM, WARP_ROW, BT, CG, WB>(A, which, smem, s_lane, s_pc, bid, nb);
     else rows_body<MODEL, V, TEAM, WARP_ROW, BT, CG, WARP_ROW ? WB : BT, AG>(A, which, s_lane, s_pc, bid, nb);
 }
 
@@ -1715,7 +1715,7 @@ __device__ __forceinline__ void lane_tile(const StepArgs &A, uint8_t *smem, int3
                         if (m == 0u) continue;
                         if (na > S::NARC - 32) {
                             __syncwarp();
-                            draw_arc_items<MODEL>(A, T, na, lane, ctx);
+                            draw_arc_items<MODEL, false>(A, T, na, lane, ctx);
                             na = 0;
                         }
                         if (xs[j]) {
@@ -1739,7 +1739,7 @@ __device__ __forceinline__ void lane_tile(const StepArgs &A, uint8_t *smem, int3
                 }
             }
         }
-        draw_tile<MODEL, S::B>(A, T, nq, nf, na, lane, ctx);
+        draw_tile<MODEL, S::B, false>(A, T, nq, nf, na, lane, ctx);
         __syncwarp();
         uint32_t fl = 0u;
         if (has) {
@@ -2045,11 +2045,14 @@ int launch_persist_t(const StepArgs &A, const PersistArgs &Q, int grid_mid, int 
     // (T = 40; most rows a warp with 16-bit counters, and now: ER n = 1200, R = 32: 423 and
     // 376 us; n = 2000, R = 64: 454 and 405; n = 10k, R = 650: 979 and 824.  Two teams on every
     // row of BA n = 2000, R = 32: 568, two classes 418; of ER n = 500k, R = 64: 2376 and 1780).
+    // The tiles gain from 8-bit counters where rows are short (ER n = 1289, R = 458, SEIR 721 and
+    // 697 us; n = 2000, R = 64, LT 522 and 490), and lose where they are not (BA n = 1752, R = 582, SIS
+    // 1543 and 1666).
     constexpr int per_cta = kBlock / (TEAM * (AG > 1 ? AG : 2));   // rows of a CTA
     const int64_t team_ctas = ((int64_t)A.n * A.nslices + per_cta - 1) / per_cta;
-    if constexpr (!ModelTraits<MODEL>::tiled && WB != kSmallBits) {
-        if (Q.max_deg < 1 << kSmallBits) {
-            if constexpr (TEAM <= 2)
+    if constexpr (ModelTraits<MODEL>::counts && WB != kSmallBits) {
+        if (Q.max_deg < (ModelTraits<MODEL>::tiled ? 64 : 1 << kSmallBits)) {
+            if constexpr (!ModelTraits<MODEL>::tiled && TEAM <= 2)
                 if (Q.max_deg < 64 && team_ctas <= 2 * sm_count)
                     return launch_persist_t<MODEL, TEAM, kSmallBits, 2>(A, Q, 0, (int)team_ctas, smem, sm_count, s, grid_out);
             return launch_persist_t<MODEL, TEAM, kSmallBits>(A, Q, grid_mid, grid_small, smem, sm_count, s, grid_out);
