@@ -1127,7 +1127,7 @@ __global__ void __launch_bounds__(kBlock, V == 4 ? 2 : 3) k_rows_fused(StepArgs 
 // (bounded for 2 resident CTAs per SM: the loop is meant for graphs that fill a few CTAs
 // per SM at most, and the body then keeps its state in registers)
 template <int MODEL, int TEAM, int WB, int AG>
-__global__ void __launch_bounds__(kBlock, 2)
+__global__ void __launch_bounds__(kBlock, kPersistCtas)
     k_rows_persist(const __grid_constant__ StepArgs A0, const __grid_constant__ PersistArgs Q) {
     extern __shared__ __align__(16) uint8_t s_dyn[];
     int32_t *s_lane = reinterpret_cast<int32_t *>(s_dyn + FusedBytes<MODEL, 1, TEAM>);
@@ -2051,7 +2051,7 @@ int launch_persist_t(const StepArgs &A, const PersistArgs &Q, int grid_mid, int 
     constexpr int per_cta = kBlock / (TEAM * (AG > 1 ? AG : 2));   // rows of a CTA
     const int64_t team_ctas = ((int64_t)A.n * A.nslices + per_cta - 1) / per_cta;
     if constexpr (ModelTraits<MODEL>::counts && WB != kSmallBits) {
-        if (Q.max_deg < (ModelTraits<MODEL>::tiled ? 64 : 1 << kSmallBits)) {
+        if (ModelTraits<MODEL>::tiled ? Q.max_deg < 64 && grid_mid > 0 : Q.max_deg < 1 << kSmallBits) {
             if constexpr (!ModelTraits<MODEL>::tiled && TEAM <= 2)
                 if (Q.max_deg < 64 && team_ctas <= 2 * sm_count)
                     return launch_persist_t<MODEL, TEAM, kSmallBits, 2>(A, Q, 0, (int)team_ctas, smem, sm_count, s, grid_out);

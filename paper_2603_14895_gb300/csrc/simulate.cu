@@ -783,16 +783,17 @@ static int run_wave(fsgp_graph *g, int model, int ic_mode, int weighted, const S
     L.carve_lane = occ.lane.carve;
     L.carve_fused = occ.fused.carve;
     const int per_block_small = (kBlock / 32) * (32 / TEAM);
-    FusedSplit split{};
-    if (fuse)
-        split = fused_split(g->cls.bucket_start, n, g->nnz, nslices, (int64_t)g->sm_count * std::max(occ.fused.ctas, 1),
-                            kBlock / 32, per_block_small, kSmallBits);
-    const int32_t fuse_split = split.warp_rows;
     // All T steps in one cooperative launch (no per-lane counts).  (27 graphs of 8k to 200k
     // words: 1.2 times faster than a launch per step on average; 16 of 200k to 1M words: 0.9
     // to 1.26.)
     const bool persist = fuse && opt.persistent >= 0 && !want_lanes && !profiling && V == 1 && T >= 1 &&
                          (words <= ((int64_t)1 << 20) || opt.persistent > 0);
+    FusedSplit split{};
+    if (fuse)
+        split = fused_split(g->cls.bucket_start, n, g->max_deg, nslices, (int64_t)g->sm_count * std::max(occ.fused.ctas, 1),
+                            (int64_t)g->sm_count * (persist ? kPersistCtas : std::max(occ.fused.ctas, 1)), kBlock / 32,
+                            per_block_small, kSmallBits);
+    const int32_t fuse_split = split.warp_rows;
     // the 16..small_max kernel also takes every small row of a frontier step
     L.fused = fuse;
     L.have_small = !fuse && n_small_all > 0;

@@ -50,6 +50,7 @@ struct Ctl {
 
 // The persistent step loop of a small graph (one launch for all T steps): the per-step
 // fields of StepArgs, and the bound on each grid-barrier wait.
+constexpr int kPersistCtas = 2;    // its resident CTAs per SM
 struct PersistArgs {
     uint32_t *buf0, *buf1;         // state buffers (step k reads buf[(k-1)&1], writes buf[k&1])
     unsigned long long *pc;        // [T+1][S][kPC]; rows 1..T are zero on entry and receive
