@@ -2046,12 +2046,13 @@ int launch_persist_t(const StepArgs &A, const PersistArgs &Q, int grid_mid, int 
     // 376 us; n = 2000, R = 64: 454 and 405; n = 10k, R = 650: 979 and 824.  Two teams on every
     // row of BA n = 2000, R = 32: 568, two classes 418; of ER n = 500k, R = 64: 2376 and 1780).
     // The tiles gain from 8-bit counters where rows are short (ER n = 1289, R = 458, SEIR 721 and
-    // 697 us; n = 2000, R = 64, LT 522 and 490), and lose where they are not (BA n = 1752, R = 582, SIS
-    // 1543 and 1666).
+    // 697 us; n = 2000, R = 64, LT 522 and 490) and few (n = 10k, R = 64, SIR 554 and 557), and lose
+    // where they are not short (BA n = 1752, R = 582, SIS 1543 and 1666).
     constexpr int per_cta = kBlock / (TEAM * (AG > 1 ? AG : 2));   // rows of a CTA
     const int64_t team_ctas = ((int64_t)A.n * A.nslices + per_cta - 1) / per_cta;
     if constexpr (ModelTraits<MODEL>::counts && WB != kSmallBits) {
-        if (ModelTraits<MODEL>::tiled ? Q.max_deg < 64 && grid_mid > 0 : Q.max_deg < 1 << kSmallBits) {
+        if (ModelTraits<MODEL>::tiled ? Q.max_deg < 64 && grid_mid > 0 && (int64_t)A.n * A.nslices <= 48 * sm_count
+                                      : Q.max_deg < 1 << kSmallBits) {
             if constexpr (!ModelTraits<MODEL>::tiled && TEAM <= 2)
                 if (Q.max_deg < 64 && team_ctas <= 2 * sm_count)
                     return launch_persist_t<MODEL, TEAM, kSmallBits, 2>(A, Q, 0, (int)team_ctas, smem, sm_count, s, grid_out);
