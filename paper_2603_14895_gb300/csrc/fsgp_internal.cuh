@@ -8,6 +8,7 @@
 #include <string>
 #include <vector>
 
+#include "arc_index.h"
 #include "fsgp.h"
 #include "hub_slots.h"
 

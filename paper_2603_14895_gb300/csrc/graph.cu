@@ -163,7 +163,7 @@ __global__ void k_out_scatter(const int32_t *__restrict__ row_ptr, const int32_t
     const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t v = warp; v < n; v += n_warps) {
         const int32_t b = row_ptr[v], e = row_ptr[v + 1];
-        for (int32_t k = b + lane; k < e; k += 32) {
+        for (int64_t k = (int64_t)b + lane; k < e; k += 32) {
             const int32_t u = col[k];
             const int32_t pos = atomicAdd(&cursor[u], 1);
             out_dst[out_ptr[u] + pos] = (int32_t)v;
@@ -274,7 +274,7 @@ __global__ void k_relabel_cols(const int32_t *__restrict__ arc0, const int32_t *
     const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t i = warp; i < n; i += n_warps) {
         const int32_t b = arc0[i], o = rp2[i], d = rp2[i + 1] - o;
-        for (int32_t k = lane; k < d; k += 32) col2[o + k] = pos[col[b + k]];
+        for (int64_t k = lane; k < d; k += 32) col2[o + k] = pos[col[b + k]];
     }
 }
 

@@ -142,25 +142,28 @@ __global__ void __launch_bounds__(256) k_hk_step(const int32_t *__restrict__ row
         const float *base = cur + (seg * TL + t) * 4;
         const int32_t r0 = (seg * TL + t) * 4;
         const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&s_row[0][tid]);
-        const int32_t blocks = (e - b + RPS - 1) / RPS;
-        auto col_of = [&](int32_t k) { return b + k * RPS + tid / TL < e ? __ldg(col + b + k * RPS + tid / TL) : -1; };
+        const uint32_t len = (uint32_t)(e - b), blocks = (len + RPS - 1) / RPS;
+        auto col_of = [&](uint32_t k) {
+            const uint32_t at = k * RPS + tid / TL;   // (past the row's end by up to kHkStages blocks)
+            return at < len ? __ldg(col + b + at) : -1;
+        };
         int32_t c = col_of(0);
-        auto copy = [&](int32_t k) {    // block k, whose column index is in c; c of the next
+        auto copy = [&](uint32_t k) {    // block k, whose column index is in c; c of the next
             if (c >= 0)
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + (uint32_t)(k % kHkStages) * 4096u),
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + k % kHkStages * 4096u),
                              "l"(base + (size_t)c * Rp));
             asm volatile("cp.async.commit_group;");
             c = col_of(k + 1);
         };
-        for (int32_t k = 0; k < kHkStages - 1; ++k) copy(k);
+        for (uint32_t k = 0; k < kHkStages - 1; ++k) copy(k);
         HkAcc acc(__ldg(reinterpret_cast<const float4 *>(base + (size_t)node * Rp)));
-        for (int32_t k = 0; k < blocks; ++k) {
+        for (uint32_t k = 0; k < blocks; ++k) {
             asm volatile("cp.async.wait_group %0;" ::"n"(kHkStages - 2));
             __syncthreads();            // block k has landed; block k - 1 has been added
             copy(k + kHkStages - 1);
             if (tid < TL) {
                 const float4 *x = s_row[k % kHkStages] + t;
-                const int m = min(RPS, e - b - k * RPS);
+                const int m = (int)min((uint32_t)RPS, len - k * RPS);
                 if (m == RPS) {
 #pragma unroll
                     for (int u = 0; u < RPS; ++u) acc.add(x[u * TL], eps);
@@ -191,11 +194,12 @@ __global__ void __launch_bounds__(256) k_hk_step(const int32_t *__restrict__ row
         fetch(team);
         // the whole warp iterates together (the column indices are handed out by shuffles)
         for (int64_t it = team; __any_sync(0xffffffffu, i >= 0); it += nteams) {
-            const int32_t node = i, e = end, r0 = (seg * TL + tl) * 4;
-            int32_t b = beg;
+            const int32_t node = i, r0 = (seg * TL + tl) * 4;
+            const uint32_t e = end;
+            uint32_t b = beg;
             const float *base = cur + r0;
             const size_t own = (size_t)max(node, 0) * Rp;
-            int32_t mine = tl < kHkUnroll && b + tl < e ? __ldg(col + b + tl) : -1;
+            int32_t mine = tl < kHkUnroll && arc_in(b, tl, e) ? __ldg(col + b + tl) : -1;
             HkAcc acc(hk_row16(base + own, node >= 0));
             fetch(it + nteams);
             while (__any_sync(0xffffffffu, b < e)) {
@@ -206,7 +210,7 @@ __global__ void __launch_bounds__(256) k_hk_step(const int32_t *__restrict__ row
                     x[u] = hk_row16(base + (size_t)max(j, 0) * Rp, j >= 0);
                 }
                 b += kHkUnroll;
-                mine = tl < kHkUnroll && b + tl < e ? __ldg(col + b + tl) : -1;
+                mine = tl < kHkUnroll && arc_in(b, tl, e) ? __ldg(col + b + tl) : -1;
 #pragma unroll
                 for (int u = 0; u < kHkUnroll; ++u) acc.add(x[u], eps);
             }

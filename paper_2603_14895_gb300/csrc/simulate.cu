@@ -254,8 +254,8 @@ __global__ void __launch_bounds__(kBlock) k_mark(StepArgs A) {
         if (entry & kPushBit) {
             const uint32_t node = node_of(A, v);   // out-arcs are listed by node
             const int32_t b = __ldg(A.out_ptr + node), e = __ldg(A.out_ptr + node + 1);
-            for (int32_t j = b; j < e; j += 32) {
-                const int32_t x = j + lane < e ? row_of(A, __ldg(A.out_dst + j + lane)) : -1;
+            for (uint32_t j = b; j < (uint32_t)e; j += 32) {
+                const int32_t x = arc_in(j, lane, e) ? row_of(A, __ldg(A.out_dst + j + lane)) : -1;
                 mark_round(A, x);
             }
         }
@@ -391,7 +391,7 @@ static int build_hub_table(const fsgp_graph *g, int chunk, cudaStream_t s, HubTa
     if (e != cudaSuccess) return cuda_fail(e, "hub degrees");
     std::vector<int64_t> base((size_t)n_hubs + 1);
     base[0] = 0;
-    for (int32_t i = 0; i < n_hubs; ++i) base[i + 1] = base[i] + (deg[i] + chunk - 1) / chunk;
+    for (int32_t i = 0; i < n_hubs; ++i) base[i + 1] = base[i] + arc_chunks(deg[i], chunk);
     FSGP_CUDA(cudaMalloc(&H.d_chunk_base, sizeof(int64_t) * base.size()));
     FSGP_CUDA(cudaMemcpyAsync(H.d_chunk_base, base.data(), sizeof(int64_t) * base.size(),
                               cudaMemcpyHostToDevice, s));

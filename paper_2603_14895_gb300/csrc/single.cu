@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(256) k_rows(const int32_t *__restrict__ row_pt
         int64_t k = 0;
         bool live = false;
         if (gather)
-            for (int32_t a = b + lane; a < e; a += kTeam) arc_fact<MODEL>(p, X[__ldg(col + a)], a, d, t, k, live);
+            for (int64_t a = (int64_t)b + lane; a < e; a += kTeam) arc_fact<MODEL>(p, X[__ldg(col + a)], a, d, t, k, live);
         // team reduction (k < 2^12 here)
         int kk = (int)k;
         int lv = live ? 1 : 0;
@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(256) k_big_rows(const int32_t *__restrict__ ro
         int64_t k = 0;
         bool live = false;
         if (s == 0)
-            for (int32_t a = b + threadIdx.x; a < e; a += blockDim.x) arc_fact<MODEL>(p, X[__ldg(col + a)], a, d, t, k, live);
+            for (int64_t a = (int64_t)b + threadIdx.x; a < e; a += blockDim.x) arc_fact<MODEL>(p, X[__ldg(col + a)], a, d, t, k, live);
         unsigned long long kk = (unsigned long long)k;
         int lv = live ? 1 : 0;
 #pragma unroll

@@ -72,7 +72,7 @@ __global__ void k_seed_count(const int32_t *__restrict__ cand, int32_t k, const 
     const int c = *cur;
     for (int i = blockIdx.x; i < k; i += gridDim.x) {
         const int32_t sd = cand[(size_t)c * k + i];
-        for (int32_t a = out_ptr[sd] + threadIdx.x; a < out_ptr[sd + 1]; a += blockDim.x)
+        for (int64_t a = (int64_t)out_ptr[sd] + threadIdx.x; a < out_ptr[sd + 1]; a += blockDim.x)
             atomicAdd(&cnt[out_dst[a]], delta);
     }
 }
@@ -84,7 +84,7 @@ __global__ void k_seed_feat(const int32_t *__restrict__ cand, int32_t k, const i
     const int c = *cur;
     for (int i = blockIdx.x; i < k; i += gridDim.x) {
         const int32_t sd = cand[(size_t)c * k + i];
-        for (int32_t a = out_ptr[sd] + threadIdx.x; a < out_ptr[sd + 1]; a += blockDim.x) {
+        for (int64_t a = (int64_t)out_ptr[sd] + threadIdx.x; a < out_ptr[sd + 1]; a += blockDim.x) {
             const int32_t v = out_dst[a];
             x[(size_t)v * F0 + 5] = __float2bfloat16(log1pf((float)cnt[v]));
         }
@@ -217,9 +217,9 @@ __global__ void __launch_bounds__(256) k_agg_long(const int32_t *__restrict__ co
         int4 it = make_int4(0, 0, 0, -1);
         if (v < n_items) it = __ldg(items + v);
         float sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        int32_t b = it.y;
-        int32_t mine = b + j < it.z ? __ldg(col + b + j) : -1;
-        while (__any_sync(0xffffffffu, b < it.z)) {
+        uint32_t b = it.y;
+        int32_t mine = arc_in(b, j, it.z) ? __ldg(col + b + j) : -1;
+        while (__any_sync(0xffffffffu, b < (uint32_t)it.z)) {
             if constexpr (F == H) {
                 uint4 x[8];
 #pragma unroll
@@ -228,13 +228,13 @@ __global__ void __launch_bounds__(256) k_agg_long(const int32_t *__restrict__ co
                     x[q] = ld_row16(h + (size_t)max(u, 0) * F + 8 * j, u >= 0);
                 }
                 b += 8;
-                mine = b + j < it.z ? __ldg(col + b + j) : -1;
+                mine = arc_in(b, j, it.z) ? __ldg(col + b + j) : -1;
 #pragma unroll
                 for (int q = 0; q < 8; ++q) add_bf16x8(sum, x[q]);
             } else {
                 const int32_t u = mine;
                 b += 8;
-                mine = b + j < it.z ? __ldg(col + b + j) : -1;
+                mine = arc_in(b, j, it.z) ? __ldg(col + b + j) : -1;
                 if (u >= 0) add_bf16x8(sum, __ldg(reinterpret_cast<const uint4 *>(h + (size_t)u * F)));
             }
         }
@@ -401,8 +401,8 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtas)
 #pragma unroll
         for (int it = 0; it < ITS; ++it) {
             const bool mine = tile * kTcRows + r0 + it * RPW >= n_long;
-            c0[it] = mine && beg[it] + j < end[it] ? __ldg(col + beg[it] + j) : -1;
-            if constexpr (F != H) c1[it] = mine && beg[it] + j + 4 < end[it] ? __ldg(col + beg[it] + j + 4) : -1;
+            c0[it] = mine && arc_in(beg[it], j, end[it]) ? __ldg(col + beg[it] + j) : -1;
+            if constexpr (F != H) c1[it] = mine && arc_in(beg[it], j + 4, end[it]) ? __ldg(col + beg[it] + j + 4) : -1;
         }
     };
     nodes_of(blockIdx.x);
@@ -424,8 +424,9 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtas)
 #pragma unroll
         for (int it = 0; it < ITS; ++it) {
             const int r = r0 + it * RPW;
-            const int32_t v = node[it], e = end[it];
-            int32_t b = beg[it];
+            const int32_t v = node[it];
+            const uint32_t e = end[it];
+            uint32_t b = beg[it];
             const float inv = e > b ? 1.f / (float)(e - b) : 0.f;
             float sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
             if (i0 + r < n_long && v >= 0) {   // summed already; the accumulator goes back to zero
@@ -449,7 +450,7 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtas)
                         x[q] = ld_row16(h + (size_t)max(u, 0) * F + 8 * j, u >= 0);
                     }
                     b += 8;
-                    mine = b + j < e ? __ldg(col + b + j) : -1;
+                    mine = arc_in(b, j, e) ? __ldg(col + b + j) : -1;
 #pragma unroll
                     for (int q = 0; q < 8; ++q) add_bf16x8(sum, x[q]);
                 }
@@ -460,7 +461,7 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtas)
                 // a source row is 16 bytes: the four lanes take every fourth arc each, two at
                 // a time
                 int32_t mine2 = c1[it];
-                for (int32_t a = b + j; a < e; a += 8) {
+                for (uint32_t a = b + j; a < e; a += 8) {
                     const uint4 x = ld_row16(h + (size_t)mine * F, true);
                     const uint4 x2 = ld_row16(h + (size_t)max(mine2, 0) * F, mine2 >= 0);
                     mine = a + 8 < e ? __ldg(col + a + 8) : -1;
@@ -825,7 +826,8 @@ __global__ void __launch_bounds__(256) k_agg_bwd(const int32_t *__restrict__ out
     const int64_t groups = ((int64_t)gridDim.x * blockDim.x) >> 4;
     const int64_t total = (int64_t)n + n_items;
     for (int64_t v = t >> 4; __any_sync(0xffffffffu, v < total); v += groups) {
-        int32_t u = -1, b = 0, e = 0, slot = -1;
+        int32_t u = -1, slot = -1;
+        uint32_t b = 0, e = 0;
         if (v < n_items) {   // the long rows' chunks first
             const int4 it = __ldg(items + v);
             u = it.x, b = it.y, e = it.z, slot = it.w;
@@ -833,10 +835,10 @@ __global__ void __launch_bounds__(256) k_agg_bwd(const int32_t *__restrict__ out
             u = __ldg(order + (v - n_items));
             b = __ldg(out_ptr + u);
             e = __ldg(out_ptr + u + 1);
-            if (e - b >= long_min) u = -1, e = b;
+            if (e - b >= (uint32_t)long_min) u = -1, e = b;
         }
         float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-        int32_t mine = j < 8 && b + j < e ? __ldg(out_dst + b + j) : -1;
+        int32_t mine = j < 8 && arc_in(b, j, e) ? __ldg(out_dst + b + j) : -1;
         while (__any_sync(0xffffffffu, b < e)) {
             uint4 x[8];
 #pragma unroll
@@ -845,7 +847,7 @@ __global__ void __launch_bounds__(256) k_agg_bwd(const int32_t *__restrict__ out
                 x[q] = ld_row16(dam + (size_t)max(w, 0) * F + 4 * j, w >= 0);
             }
             b += 8;
-            mine = j < 8 && b + j < e ? __ldg(out_dst + b + j) : -1;
+            mine = j < 8 && arc_in(b, j, e) ? __ldg(out_dst + b + j) : -1;
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
                 s.x += __uint_as_float(x[q].x);
@@ -885,7 +887,7 @@ __global__ void k_agg_bwd_fin(const int32_t *__restrict__ long_rows, int32_t n_l
 // of the degree order (in-rows, its first n_in_long) and node v (out-rows); the entries past
 // the last are zero, so that the scans end in the totals.
 __device__ __forceinline__ int32_t chunks_of(int32_t d, int32_t long_min) {
-    return d >= long_min ? (int32_t)(((int64_t)d + kSgChunk - 1) / kSgChunk) : 0;
+    return d >= long_min ? (int32_t)arc_chunks(d, kSgChunk) : 0;
 }
 __global__ void k_table_counts(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ out_ptr,
                                const int32_t *__restrict__ order, int32_t n, int32_t n_in_long, int32_t long_min,
